@@ -3,21 +3,26 @@
 // block: the query projection of the selected tokens, the output projection and the MLP on selected
 // rows; with idx == NULL the key / value projections of all tokens).
 //
-// A dense contraction, so it runs on the tcgen05 tensor cores.  Persistent CTAs, one per SM, walk over
-// 256-row x 256-column output tiles (column tiles of one row tile are neighbours in the walk, so the
-// gathered rows stay in L2 while W, which is small, lives there anyway).  A tile is two 128-row sub-tiles
-// that share every W tile in shared memory.  Warp roles:
-//   warps 0-15  epilogue: two threads per output row (128 columns each); TMEM -> registers -> (+ bias, GELU, gate,
+// A dense contraction, so it runs on the tcgen05 tensor cores.  Persistent CTA pairs (clusters of two, one CTA per SM)
+// walk over 256-row x bn-column output tiles (column tiles of one row tile are neighbours in the walk, so the
+// gathered rows stay in L2 while W, which is small, lives there anyway).  Both SMs of a pair work on one
+// tcgen05.mma.cta_group::2 of 256 x bn x 16: each CTA holds 128 rows of A, half of the W tile and its 128 rows of the
+// accumulator, so a W tile is read from shared memory once per pair instead of once per 128 rows, and the accumulator takes
+// only half of a CTA's TMEM: there are two of them, and the epilogue of a tile runs under the main loop of the next.
+// Warp roles of each CTA:
+//   warps 0-15  epilogue: four threads per output row (every fourth group of 32 columns); TMEM -> registers -> (+ bias, GELU, gate,
 //               residual) -> bf16 -> the row of y that idx names (fused scatter);
-//   warps 16-23 gather of the A operand: the listed rows of x, 64 columns (128 bytes) per pipeline stage,
-//               by 16-byte cp.async into the 128-byte-swizzled layout the MMA reads (rows past the end
-//               are zero-filled); the copies arrive on the stage's barrier by themselves, so a thread never
-//               waits for its own copies, only for a free stage;
-//   warp 24     TMA producer of the B operand: a 256 x 64 tile of W per stage (rows past N_out read as zero);
-//   warp 25     tcgen05.mma issuer: per stage four 128 x 256 x 16 SS MMAs into each sub-tile's accumulator.
-// Stages: 3 x (2 x 16 KB of A + 32 KB of W); TMEM: two accumulators of 256 columns.  Every mbarrier wait
-// is bounded; on a timeout the CTA raises the error word, the remaining waits return at once, and the
-// CTA runs out.
+//   warp 16     TMA producer: this CTA's half of a W tile per stage (rows past N_out read as zero) and, when the rows
+//               of x are a contiguous matrix (no list, or compact rows), the CTA's 128 rows of x as well;
+//   warp 17     even CTA: tcgen05.mma issuer for the pair, four MMAs per stage; odd CTA: tells the even one which of its
+//               stages have landed;
+//   warps 18-19 (listed rows only) gather of the A operand: the listed rows of x, 64 columns (128 bytes) per
+//               pipeline stage, by 16-byte cp.async into the 128-byte-swizzled layout the MMA reads (rows past the end
+//               and entries out of range are zero-filled); the copies arrive on the stage's barrier by themselves, so a
+//               thread never waits for its own copies, only for a free stage.  (TMA gather4, one per lane and stage, was
+//               measured at 331 us where this takes 119, 9001 x 3072 x 3072.)
+// Every mbarrier wait is bounded; on a timeout the CTA raises the error word, its remaining waits return at once, the
+// other CTA of the pair runs into its own limit, and both run out.
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 #include "bounded_wait.cuh"
@@ -27,25 +32,24 @@ namespace {
 
 using namespace ptx;
 
-// 128-row sub-tiles of a CTA tile, each with its own 256-column accumulator.  Two: a 256 x 256 tile reads 128 flop
-// per byte of operands from L2 instead of 85, which is what bounds this kernel; it fills TMEM, so the epilogue is
-// not hidden under the next main loop any more, and is still 4-15 % faster than one sub-tile with two accumulator sets.
-constexpr int kMSub = 2;
-constexpr int kBM = 128 * kMSub, kBN = 256, kBK = 64;
-constexpr int kStages = (kMSub == 2) ? 3 : 4;
-constexpr int kAccSets = 2 / kMSub;                      // accumulator sets in TMEM: two sets let the epilogue run under the next main loop
-constexpr int kASubBytes = 128 * kBK * 2, kABytes = kMSub * kASubBytes, kBBytes = kBN * kBK * 2;
-// Epilogue warps: four per sub-tile cover its 128 rows (one TMEM lane quarter each); kEpiSplit such groups share the 256
-// columns of the accumulator.  Two: the epilogue is not hidden under the next tile's main loop (TMEM is full), so its
-// time counts in full, and bias, GELU (erf), gate and residual make it a third to a half of a tile's time with one group.
-constexpr int kEpiSplit = 2;
-constexpr int kEpiWarps = 4 * kMSub * kEpiSplit, kGatherWarps = 4 * kMSub;
-constexpr int kThreads = (kEpiWarps + kGatherWarps + 2) * 32;
-constexpr int kTmaWarp = kEpiWarps + kGatherWarps, kMmaWarp = kTmaWarp + 1;
+constexpr int kRowsCta = 128, kBM = 2 * kRowsCta, kBK = 64;
+constexpr int kAccSets = 2;                              // accumulators in TMEM: the epilogue runs under the next main loop
+// Epilogue warps: four cover the CTA's 128 rows (one TMEM lane quarter each); kEpiSplit such groups share the columns.
+// Four groups: a tile of a short contraction (K = 1152: 18 stages) is over in 5 us, and two groups take 6 us for its
+// bias, GELU (erf), gate, residual and stores.
+constexpr int kEpiSplit = 4;
+constexpr int kEpiWarps = 4 * kEpiSplit, kGatherWarps = 2;
+constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kTmaWarp + 1, kFirstGatherWarp = kMmaWarp + 1;
 constexpr int kEpiStageBytes = 32 * 64;                  // per epilogue warp: 32 rows x 32 bf16 columns on their way to / from global memory
-constexpr int kSmemBytes = kStages * (kABytes + kBBytes) + 256 + kEpiWarps * kEpiStageBytes + 1024;
-static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
-constexpr uint32_t kAccCols = kBN, kTmemCols = 2 * kBN;
+
+constexpr int kMaxBN = 256, kBNStep = 32;                // columns of an output tile: what cta_group::2 takes at M = 256
+constexpr int kStages = 6;
+constexpr int kABytes = kRowsCta * kBK * 2, kBBytes = kMaxBN / 2 * kBK * 2;
+constexpr int kBarBytes = 256;
+static_assert(8 * (3 * kStages + 2 * kAccSets) <= kBarBytes, "barrier area too small");
+constexpr int kSmemBytes = kStages * (kABytes + kBBytes) + kBarBytes + kEpiWarps * kEpiStageBytes + 1024;
+static_assert(kSmemBytes + 1536 <= 227 * 1024, "shared memory of one CTA");
+constexpr uint32_t kAccCols = kMaxBN, kTmemCols = kAccSets * kAccCols;
 
 struct LinParams {
     const __nv_bfloat16 *x;
@@ -54,6 +58,7 @@ struct LinParams {
     const __nv_bfloat16 *bias;
     __nv_bfloat16 *y;
     int B, N, K, N_out;
+    int bn;                      // columns of an output tile
     int compact;                 // y is [B, M, N_out]
     int compact_in;              // x is [B, M, K]
     int gelu;                    // y = GELU(x W^T + bias), exact (erf) form
@@ -94,81 +99,99 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *m, 
         ::"r"(dst), "l"(m), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
 
-// row of x that holds the g-th listed row (all batch elements in one list): -1 past the end, -2 for an index
-// outside [0, N) or one that does not exceed its predecessor; *out_row is the row of y it goes to, *res_row the row
-// of the residual, *batch the batch element
-__device__ __forceinline__ long long source_row(const LinParams &p, long long g, long long total, long long *out_row,
-                                                long long *res_row = nullptr, int *batch = nullptr) {
-    if (g >= total) return -1;
-    const int b = (int)(g / p.M), r = (int)(g - (long long)b * p.M);
+// The g-th listed row (all batch elements in one list): *out_row is the row of y it goes to, *res_row the row of the
+// residual, *batch the batch element.  False past the end of the list and for an index outside [0, N) or one that does
+// not exceed its predecessor (*bad).
+__device__ __forceinline__ bool target_row(const LinParams &p, long long g, long long total, long long *out_row,
+                                           long long *res_row, int *batch, bool *bad) {
+    *bad = false;
+    if (g >= total) return false;
+    const int b = (int)((unsigned)g / (unsigned)p.M), r = (int)((unsigned)g - (unsigned)b * (unsigned)p.M);   // fewer than 2^31 rows fit the device
     const int tok = p.idx ? __ldg(p.idx + g) : r;
-    if ((unsigned)tok >= (unsigned)p.N) return -2;
-    if (p.idx && r > 0 && __ldg(p.idx + g - 1) >= tok) return -2;      // not strictly ascending: a row would be written twice
-    if (out_row) *out_row = p.compact ? g : (long long)b * p.N + tok;
-    if (res_row) *res_row = p.res_compact ? g : (long long)b * p.N + tok;
-    if (batch) *batch = b;
-    return p.compact_in ? g : (long long)b * p.N + tok;
+    const int before = (p.idx && r > 0) ? __ldg(p.idx + g - 1) : -1;
+    // not strictly ascending: a row would be written twice
+    if ((unsigned)tok >= (unsigned)p.N || (r > 0 && before >= tok)) { *bad = true; return false; }
+    *out_row = p.compact ? g : (long long)b * p.N + tok;
+    *res_row = p.res_compact ? g : (long long)b * p.N + tok;
+    *batch = b;
+    return true;
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
-gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const LinParams p)
+// DENSE: the rows of x are one contiguous matrix
+template <bool DENSE> constexpr int kThreads = (kEpiWarps + 2 + (DENSE ? 0 : kGatherWarps)) * 32;
+
+template <bool DENSE>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads<DENSE>, 1)
+gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x, const LinParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ int row_list[2][kRowsCta];                          // listed rows only: the rows of x of a tile
 
+    // (both CTAs of a pair run the same kernel with the same static shared memory, so every offset below is the same in both)
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sA = smem_base, sB = sA + kStages * kABytes, bars = sB + kStages * kBBytes;
-    const uint32_t bar_full = bars, bar_empty = bars + 8 * kStages, bar_acc_full = bars + 16 * kStages,
-                   bar_acc_empty = bar_acc_full + 16;
+    const uint32_t bar_full = bars, bar_empty = bars + 8 * kStages, bar_peer = bars + 16 * kStages,
+                   bar_acc_full = bars + 24 * kStages, bar_acc_empty = bar_acc_full + 8 * kAccSets;
 
     const int tid = threadIdx.x;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);        // warp-uniform
     const int lane = tid & 31;
+    const uint32_t rank = cluster_ctarank();
+    const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const long long total_rows = (long long)p.B * p.M;
-    const int tiles_m = (int)((total_rows + kBM - 1) / kBM), tiles_n = (p.N_out + kBN - 1) / kBN;
+    const int tiles_m = (int)((total_rows + kBM - 1) / kBM), tiles_n = (p.N_out + p.bn - 1) / p.bn;
     const int total_tiles = tiles_m * tiles_n, k_steps = p.K / kBK;
 
     if (tid == 0) {
         abort_flag = 0;
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(bar_full + 8 * s, kGatherWarps * 32 + 1);     // every gather thread + the TMA producer
-            mbar_init(bar_empty + 8 * s, 1);
+            mbar_init(bar_full + 8 * s, (DENSE ? 0 : kGatherWarps * 32) + 1);     // every gather thread + the TMA producer
+            mbar_init(bar_empty + 8 * s, 1);                    // the issuer's commit
+            mbar_init(bar_peer + 8 * s, 1);                     // even CTA: the odd CTA's part of the stage has landed
         }
-        for (int a = 0; a < kAccSets; ++a) { mbar_init(bar_acc_full + 8 * a, 1); mbar_init(bar_acc_empty + 8 * a, kEpiWarps * 32); }
+        for (int a = 0; a < kAccSets; ++a) { mbar_init(bar_acc_full + 8 * a, 1); mbar_init(bar_acc_empty + 8 * a, 2 * kEpiWarps); }
         fence_barrier_init();
     }
     if (warp == kMmaWarp) {
-        tmem_alloc(smem_u32(&tmem_slot), kTmemCols);
-        tmem_relinquish();
+        tmem_alloc_pair(smem_u32(&tmem_slot), kTmemCols);
+        tmem_relinquish_pair();
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync_all();                                            // the barriers of both CTAs are set up
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
     if (warp < kEpiWarps) {
         // ------------------------------------------------ epilogue
-        // row of the CTA tile: sub-tile (warp / 4) % kMSub, TMEM lanes by warp % 4; columns [c0, c0 + kBN / kEpiSplit) by warp / (4 kMSub)
-        const int sub = (warp >> 2) % kMSub, part = warp / (4 * kMSub);
-        const int row = sub * 128 + (warp & 3) * 32 + lane;
-        const int c0 = part * (kBN / kEpiSplit);
-        const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16) + sub * kAccCols;
-        uint8_t *stage = smem_raw + (bars + 256 - smem_u32(smem_raw)) + warp * kEpiStageBytes;
+        // TMEM lanes (rows of the CTA) by warp % 4; columns c0 + 32 (kEpiSplit j) .. + 31 of the tile by warp / 4
+        const int part = warp >> 2;
+        const int row = (int)rank * kRowsCta + (warp & 3) * 32 + lane;
+        const int c0 = part * 32;
+        const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        uint8_t *stage = smem_raw + (bars + kBarBytes - smem_u32(smem_raw)) + warp * kEpiStageBytes;
         int it = 0;
-        for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
+        for (int tile = pair; tile < total_tiles; tile += n_pairs, ++it) {
             const int tm = tile / tiles_n, tn = tile - tm * tiles_n;
-            const int acc = it % kAccSets, n0 = tn * kBN;
+            const int acc = it % kAccSets, n0 = tn * p.bn;
             long long out_row = -1, res_row = -1;
             int batch = 0;
-            const long long src = source_row(p, (long long)tm * kBM + row, total_rows, &out_row, &res_row, &batch);
-            if (src == -2 && tn == 0 && part == 0) atomicExch(p.err_word, kErrBadIndex);
-            if (src < 0) { out_row = -1; res_row = -1; }
+            bool bad;
+            target_row(p, (long long)tm * kBM + row, total_rows, &out_row, &res_row, &batch, &bad);
+            if (bad && tn == 0 && part == 0) atomicExch(p.err_word, kErrBadIndex);
             if (!p.residual) res_row = -1;
             const __nv_bfloat16 *gate = p.gate ? p.gate + (long long)batch * p.N_out : nullptr;
             wait_bar(bar_acc_full + 8 * acc, (it / kAccSets) & 1, &abort_flag, p.err_word);
             tc_fence_after();
             if (abort_flag) out_row = -1;
+            auto release = [&] {                                   // this warp's part of the accumulator has been read
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(map_to_rank(bar_acc_empty + 8 * acc, 0));
+            };
+            if (c0 >= p.bn) release();                             // narrow tiles: nothing for this group
             // Global memory is touched in a transposed layout: a thread owns a row of the accumulator, so a warp that
             // stored its rows directly would touch 32 lines per instruction, 16 bytes in each (measured: ~9 us of a
             // 36 us tile, 16 us with a residual).  Instead lane l moves the 16-byte piece l & 3 of rows (l >> 2) + 8 j:
@@ -176,7 +199,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const LinPara
             // swizzled by the row so that both directions are free of bank conflicts).
             const int q = lane & 3;
 #pragma unroll 1
-            for (int c = c0; c < c0 + kBN / kEpiSplit; c += 32) {
+            for (int c = c0; c < p.bn; c += 32 * kEpiSplit) {
                 const int colq = n0 + c + q * 8;                    // the 8 columns this lane moves
                 uint32_t rw[16];                                    // this thread's row of the residual: 32 bf16
                 if (p.residual) {
@@ -202,12 +225,9 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const LinPara
                     __syncwarp();
                 }
                 uint32_t o[32];
-                tmem_ld32(t_row + acc * kMSub * kAccCols + c, o);
+                tmem_ld32(t_row + acc * kAccCols + c, o);
                 tc_wait_ld();
-                if (c + 32 == c0 + kBN / kEpiSplit) {    // this thread's part of the accumulator has been read: the MMA warp may reuse it
-                    tc_fence_before();
-                    mbar_arrive(bar_acc_empty + 8 * acc);
-                }
+                if (c + 32 * kEpiSplit >= p.bn) release();
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     const int col = n0 + c + v * 8;
@@ -264,43 +284,19 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const LinPara
                 __syncwarp();
             }
         }
-    } else if (warp < kEpiWarps + kGatherWarps) {
-        // ------------------------------------------------ gather of the A rows (cp.async, 128-byte swizzle)
-        const int t = tid - kEpiWarps * 32;                   // 0 .. 128 kMSub - 1
-        const int chunk = t & 7, row0 = t >> 3;               // this thread: 16-byte chunk `chunk` of rows row0 + 16 kMSub i
-        int g = 0;                                            // running stage count over all tiles
-        for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-            const int tm = tile / tiles_n;
-            const __nv_bfloat16 *src[8];
-            uint32_t off[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int r = row0 + 16 * kMSub * i;
-                const long long s = source_row(p, (long long)tm * kBM + r, total_rows, nullptr);
-                src[i] = (s >= 0) ? p.x + s * p.K + chunk * 8 : nullptr;
-                off[i] = (r >> 7) * kASubBytes + (r & 127) * 128 + ((chunk ^ (r & 7)) << 4);
-            }
-            for (int ks = 0; ks < k_steps; ++ks, ++g) {
-                const int st = g % kStages;
-                wait_bar(bar_empty + 8 * st, ((g / kStages) & 1) ^ 1, &abort_flag, p.err_word);
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    cp_async_16(sA + st * kABytes + off[i], src[i] ? (const void *)(src[i] + ks * kBK) : (const void *)p.x, src[i] != nullptr);
-                cp_async_arrive(bar_full + 8 * st);           // asynchronous: the thread goes on to the next free stage
-            }
-        }
     } else if (warp == kTmaWarp) {
-        // ------------------------------------------------ TMA producer of the W tiles
-        if (elect_one()) prefetch_tensormap(&tmap_w);
+        // ------------------------------------------------ TMA producer of the W tiles (and of contiguous rows of x)
+        if (elect_one()) { prefetch_tensormap(&tmap_w); if (DENSE) prefetch_tensormap(&tmap_x); }
         int g = 0;
-        for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-            const int tn = tile % tiles_n;
+        for (int tile = pair; tile < total_tiles; tile += n_pairs) {
+            const int tm = tile / tiles_n, tn = tile - tm * tiles_n;
             for (int ks = 0; ks < k_steps; ++ks, ++g) {
                 const int st = g % kStages;
                 wait_bar(bar_empty + 8 * st, ((g / kStages) & 1) ^ 1, &abort_flag, p.err_word);
                 if (elect_one()) {
-                    mbar_arrive_expect_tx(bar_full + 8 * st, kBBytes);
-                    tma_load_2d(sB + st * kBBytes, &tmap_w, bar_full + 8 * st, ks * kBK, tn * kBN);
+                    mbar_arrive_expect_tx(bar_full + 8 * st, p.bn * kBK + (DENSE ? kABytes : 0));
+                    tma_load_2d(sB + st * kBBytes, &tmap_w, bar_full + 8 * st, ks * kBK, tn * p.bn + (int)rank * (p.bn / 2));
+                    if (DENSE) tma_load_2d(sA + st * kABytes, &tmap_x, bar_full + 8 * st, ks * kBK, tm * kBM + (int)rank * kRowsCta);
                 }
                 __syncwarp();
             }
@@ -308,44 +304,150 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const LinPara
         // every copy issued above must have landed before the CTA's shared memory is released
         for (int gs = (g > kStages ? g - kStages : 0); gs < g; ++gs)
             wait_bar(bar_full + 8 * (gs % kStages), (gs / kStages) & 1, &abort_flag, p.err_word);
-    } else {
-        // ------------------------------------------------ MMA issuer
-        constexpr uint32_t idesc = idesc_bf16(128, kBN, false);
+    } else if (warp == kMmaWarp && rank == 0) {
+        // ------------------------------------------------ MMA issuer of the pair
+        const uint32_t idesc = idesc_bf16(kBM, p.bn, false);
         int g = 0, it = 0;
-        for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
+        for (int tile = pair; tile < total_tiles; tile += n_pairs, ++it) {
             const int acc = it % kAccSets;
             wait_bar(bar_acc_empty + 8 * acc, ((it / kAccSets) & 1) ^ 1, &abort_flag, p.err_word);
             for (int ks = 0; ks < k_steps; ++ks, ++g) {
                 const int st = g % kStages;
                 wait_bar(bar_full + 8 * st, (g / kStages) & 1, &abort_flag, p.err_word);
-                fence_proxy_async_smem();             // the gathered rows were written through the generic proxy
+                wait_bar(bar_peer + 8 * st, (g / kStages) & 1, &abort_flag, p.err_word);
+                if (!DENSE) fence_proxy_async_smem();     // gathered rows were written through the generic proxy
                 tc_fence_after();
                 if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < kBK / 16; ++kk) {
-#pragma unroll
-                        for (int sub = 0; sub < kMSub; ++sub)       // the sub-tiles share the W tile in shared memory
-                            mma_ss(tmem + (acc * kMSub + sub) * kAccCols,
-                                   smem_desc(sA + st * kABytes + sub * kASubBytes + kk * 32, 16, 1024, kSwizzle128B),
-                                   smem_desc(sB + st * kBBytes + kk * 32, 16, 1024, kSwizzle128B),
-                                   idesc, (ks > 0 || kk > 0) ? 1u : 0u);
-                    }
-                    tc_commit(bar_empty + 8 * st);
-                    if (ks == k_steps - 1) tc_commit(bar_acc_full + 8 * acc);
+                    for (int kk = 0; kk < kBK / 16; ++kk)
+                        mma_ss_pair(tmem + acc * kAccCols, smem_desc(sA + st * kABytes + kk * 32, 16, 1024, kSwizzle128B),
+                                    smem_desc(sB + st * kBBytes + kk * 32, 16, 1024, kSwizzle128B), idesc, (ks > 0 || kk > 0) ? 1u : 0u);
+                    tc_commit_pair(bar_empty + 8 * st);
+                    if (ks == k_steps - 1) tc_commit_pair(bar_acc_full + 8 * acc);
                 }
                 __syncwarp();
             }
         }
+    } else if (warp == kMmaWarp) {
+        // ------------------------------------------------ odd CTA: its part of a stage has landed
+        int g = 0;
+        for (int tile = pair; tile < total_tiles; tile += n_pairs)
+            for (int ks = 0; ks < k_steps; ++ks, ++g) {
+                const int st = g % kStages;
+                wait_bar(bar_full + 8 * st, (g / kStages) & 1, &abort_flag, p.err_word);
+                if (!DENSE) fence_proxy_async_smem();     // gathered rows were written through the generic proxy
+                if (elect_one()) mbar_arrive_cluster(map_to_rank(bar_peer + 8 * st, 0));
+                __syncwarp();
+            }
+    } else if constexpr (!DENSE) {
+        // ------------------------------------------------ gather of the A rows (cp.async, 128-byte swizzle)
+        constexpr int kGatherThreads = kGatherWarps * 32, kRowStep = kGatherThreads / 8, kRowsThread = kRowsCta / kRowStep;
+        static_assert(kRowStep % 8 == 0, "a row step keeps the swizzle phase of the thread's rows");
+        const int t = tid - kFirstGatherWarp * 32;
+        const int chunk = t & 7, row0 = t >> 3;               // this thread: 16-byte chunk `chunk` of rows row0 + kRowStep i
+        const uint32_t off = row0 * 128 + ((chunk ^ (row0 & 7)) << 4);
+        // The list entries of the next tile are fetched while this one is streamed (fetched where they are needed, two
+        // dependent loads for each of a thread's rows, they cost 4-11 us a tile), each by one thread, and go round
+        // through shared memory.
+        constexpr int kEnt = kRowsCta / kGatherThreads;
+        int ent[kEnt];
+        auto fetch = [&](int tile) {
+#pragma unroll
+            for (int i = 0; i < kEnt; ++i) {
+                const long long r = (long long)(tile / tiles_n) * kBM + (int)rank * kRowsCta + t + i * kGatherThreads;
+                ent[i] = (tile < total_tiles && r < total_rows) ? __ldg(p.idx + r) : -1;
+            }
+        };
+        fetch(pair);
+        int g = 0, it = 0;                                    // running stage and tile counts
+        for (int tile = pair; tile < total_tiles; tile += n_pairs, ++it) {
+            const int tm = tile / tiles_n;
+            int *list = row_list[it & 1];
+#pragma unroll
+            for (int i = 0; i < kEnt; ++i) {
+                // rows of 128 bytes or more: their number is below 2^31
+                const unsigned r = (unsigned)tm * kBM + rank * kRowsCta + t + i * kGatherThreads;
+                list[t + i * kGatherThreads] = (unsigned)ent[i] < (unsigned)p.N ? (int)(r / (unsigned)p.M * (unsigned)p.N) + ent[i] : -1;
+            }
+            fetch(tile + n_pairs);
+            asm volatile("bar.sync 1, %0;" ::"n"(kGatherThreads) : "memory");      // two lists: one barrier per tile is enough
+            int src[kRowsThread];
+#pragma unroll
+            for (int i = 0; i < kRowsThread; ++i) src[i] = list[row0 + kRowStep * i];
+            const __nv_bfloat16 *xc = p.x + chunk * 8;
+            for (int ks = 0; ks < k_steps; ++ks, ++g, xc += kBK) {
+                const int st = g % kStages;
+                wait_bar(bar_empty + 8 * st, ((g / kStages) & 1) ^ 1, &abort_flag, p.err_word);
+#pragma unroll
+                for (int i = 0; i < kRowsThread; ++i)
+                    cp_async_16(sA + st * kABytes + off + i * (kRowStep * 128), xc + (size_t)(unsigned)max(src[i], 0) * (unsigned)p.K, src[i] >= 0);
+                cp_async_arrive(bar_full + 8 * st);           // asynchronous: the thread goes on to the next free stage
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
     }
 
+    // neither CTA leaves (or gives up its TMEM) while the other may still arrive on its barriers or read its shared memory
     tc_fence_before();
     __syncthreads();
-    if (warp == kMmaWarp) tmem_dealloc(tmem, kTmemCols);
+    cluster_sync_all();
+    if (warp == kMmaWarp) tmem_dealloc_pair(tmem, kTmemCols);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// a row-major bf16 matrix [rows, K] with 128-byte-swizzled boxes of 64 columns x box_rows
+int32_t make_matrix_map(CUtensorMap *map, const void *base, long long rows, int K, int box_rows, const char *what)
+{
+    const EncodeTiledFn enc = reinterpret_cast<EncodeTiledFn>(tensor_map_encoder());
+    if (!enc) return fail(ASTRAEA_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
+    cuuint64_t strides[1] = {(cuuint64_t)K * 2};
+    cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
+    cuuint32_t estr[2] = {1, 1};
+    CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(ASTRAEA_ERR_INVALID_ARG, "astraea_gathered_linear: tensor map of %s rejected (CUresult %d)", what, (int)r);
+    return ASTRAEA_OK;
+}
+
+template <bool DENSE>
+int32_t launch_linear(const LinParams &p, const void *x, const void *w, int pairs, cudaStream_t stream)
+{
+    CUtensorMap mw, mx;
+    int32_t rc = make_matrix_map(&mw, w, p.N_out, p.K, p.bn / 2, "W");
+    if (rc != ASTRAEA_OK) return rc;
+    mx = mw;
+    if (DENSE) rc = make_matrix_map(&mx, x, (long long)p.B * p.M, p.K, kRowsCta, "x");
+    if (rc != ASTRAEA_OK) return rc;
+    static PerDeviceOnce attrs;                   // the attribute is per device
+    if (attrs.run([] { return cudaFuncSetAttribute(gathered_linear_kernel<DENSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes); }) != cudaSuccess)
+        return check_launch("astraea_gathered_linear (shared memory attribute)");
+    const long long tiles = (((long long)p.B * p.M + kBM - 1) / kBM) * ((p.N_out + p.bn - 1) / p.bn);
+    const int grid = 2 * (int)(tiles < pairs ? tiles : pairs);
+    gathered_linear_kernel<DENSE><<<grid, kThreads<DENSE>, kSmemBytes, stream>>>(mw, mx, p);
+    return check_launch("astraea_gathered_linear");
+}
+
+// Columns of an output tile.  The launch takes ceil(tiles / pairs) rounds, and a round of narrower tiles costs less, but
+// not in proportion (the rows of x are streamed for fewer columns): measured 0.60-0.67 of a 256-column round at 128
+// columns on seven shapes.  256 unless another width saves 3 % by that estimate, which happens where a launch has a
+// few rounds only or the last tile of a row is mostly padding.
+int choose_bn(long long rows, int N_out, int pairs)
+{
+    const long long tiles_m = (rows + kBM - 1) / kBM;
+    int best_bn = kMaxBN;
+    double best = 0.0;
+    for (int bn = kMaxBN; bn >= kBNStep; bn -= kBNStep) {
+        const long long tiles = tiles_m * ((N_out + bn - 1) / bn);
+        const double t = (double)((tiles + pairs - 1) / pairs) * (0.26 + 0.74 * bn / kMaxBN);
+        if (best == 0.0 || t < 0.97 * best) { best = t; best_bn = bn; }
+    }
+    return best_bn;
+}
 
 }  // namespace
 
@@ -355,21 +457,6 @@ int32_t launch_gathered_linear(const void *x, const int32_t *idx, int M, const v
                                int B, int N, int K, int N_out, uint32_t flags, int *err_word, cudaStream_t stream,
                                const void *residual, const void *gate)
 {
-    const EncodeTiledFn enc = reinterpret_cast<EncodeTiledFn>(tensor_map_encoder());
-    if (!enc) return fail(ASTRAEA_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    // W as a 2-D tensor (K, N_out) with 128-byte-swizzled boxes of 64 columns x 256 rows
-    CUtensorMap mw;
-    cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)N_out};
-    cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)kBN};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(&mw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(w), dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(ASTRAEA_ERR_INVALID_ARG, "astraea_gathered_linear: tensor map of W rejected (CUresult %d)", (int)r);
-    static PerDeviceOnce attrs;                   // the attribute is per device
-    if (attrs.run([] { return cudaFuncSetAttribute(gathered_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes); }) != cudaSuccess)
-        return check_launch("astraea_gathered_linear (shared memory attribute)");
     LinParams p;
     p.x = reinterpret_cast<const __nv_bfloat16 *>(x);
     p.idx = idx;
@@ -384,12 +471,10 @@ int32_t launch_gathered_linear(const void *x, const int32_t *idx, int M, const v
     p.res_compact = (flags & ASTRAEA_LINEAR_COMPACT_RES) ? 1 : 0;
     p.gate = reinterpret_cast<const __nv_bfloat16 *>(gate);
     p.err_word = err_word;
-    const long long rows = (long long)B * p.M;
-    const long long tiles = ((rows + kBM - 1) / kBM) * ((N_out + kBN - 1) / kBN);
-    const int n_sm = sm_count();
-    const int grid = (int)(tiles < n_sm ? tiles : n_sm);
-    gathered_linear_kernel<<<grid, kThreads, kSmemBytes, stream>>>(mw, p);
-    return check_launch("astraea_gathered_linear");
+    const int pairs = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
+    p.bn = choose_bn((long long)B * p.M, N_out, pairs);
+    if (!idx || p.compact_in) return launch_linear<true>(p, x, w, pairs, stream);
+    return launch_linear<false>(p, x, w, pairs, stream);
 }
 
 }  // namespace astraea

@@ -88,6 +88,32 @@ def test_layernorm_plain_and_bad_index(oracle):
     assert e.value.code == A.ERR_UNSUPPORTED
 
 
+# ------------------------------------------------------------------ tile edges of the gathered GEMM
+@pytest.mark.parametrize("listed", [False, True])
+@pytest.mark.parametrize("rows,K,N_out", [(1, 64, 8), (127, 64, 24), (129, 128, 40), (255, 448, 136), (257, 384, 264), (130, 1152, 1152),
+                                          (2300, 64, 2056)])
+def test_gathered_linear_tile_edges(oracle, rows, K, N_out, listed):
+    """Row counts around a CTA's 128 and a pair's 256 rows, column counts around a group of 32 and a tile, fewer and more
+    stages than the pipeline has, one tile and several per CTA pair; B = 2, so that a tile holds rows of both lists."""
+    rng = np.random.default_rng(rows + N_out)
+    B, N = 2, rows + 5 if listed else rows
+    x, w, bias, cache = _bits(rng, B, N, K), _bits(rng, N_out, K, scale=K ** -0.5), _bits(rng, N_out), _bits(rng, B, N, N_out)
+    idx = _sorted_idx(rng, B, N, rows) if listed else None
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    g = Guarded((B, N, N_out), torch.bfloat16, init=to_dev_bf16(cache))
+    A.astraea_gathered_linear(to_dev_bf16(x), None if idx is None else dev(idx), rows, to_dev_bf16(w), to_dev_bf16(bias), g.t, B, N, K, N_out, workspace=ws)
+    A.astraea_poll_error(ws)
+    g.check("tile edges")
+    got, want = bf16_dev_to_f64(g.t), oracle.gathered_linear(f64(x), f64(w), f64(bias), idx)
+    if listed:
+        mask = np.ones((B, N), bool)
+        for b in range(B):
+            mask[b, idx[b]] = False
+        assert np.array_equal(got[mask], f64(cache)[mask])
+        got, want = oracle.take_rows(got, idx), oracle.take_rows(want, idx)
+    _close(got, want, "tile edges")
+
+
 # ------------------------------------------------------------------ linear layer with a gated residual
 @pytest.mark.parametrize("res_compact,out_compact,in_compact,gelu", [(False, False, False, False), (False, True, False, False),
                                                                      (True, True, True, False), (True, False, True, True)])
