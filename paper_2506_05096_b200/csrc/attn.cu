@@ -23,8 +23,8 @@
 //
 // The softmax is bound by the exponentials (XU pipe, 16 per clock per SM), by the issue slots and by the
 // latencies of its own chain, so the common path of a key tile is kept to: load S, one FFMA + one
-// exponential per element, (sum,) pack, store.  At head_dim 64 / 72 six / four of every sixteen
-// exponentials are a cubic on the FMA pipe instead of ex2 on the XU, and at head_dim 64 the row sums are
+// exponential per element, (sum,) pack, store.  A part of the exponentials (three of eight pairs at head_dim 64 and
+// 128, one of four at 72) are a polynomial on the FMA pipe instead of ex2 on the XU, and at head_dim 64 the row sums are
 // left to the tensor core (P times a column of ones, 16 more accumulator columns).  The reference maximum
 // is the exact row maximum of key tile 0 (plus a shift) and is then only checked through the sums of
 // exponentials: while they stay below a limit the probabilities are accepted as they are (they are relative
@@ -89,9 +89,14 @@ template <int DH, int TM> struct Cfg {
     // head_dim 72 gains nothing from it and 128 has no TMEM columns left: they sum the fp32 exponentials themselves.
     static constexpr bool kOnes = DH == 64;
     static constexpr int kSBufs = 2;                              // S buffers per query tile: one per softmax warpgroup
-    // exponentials per 16 that are computed on the FMA pipe instead of the XU (measured best: 6 at head_dim 64, 4 at
-    // 72, none at 128, where the tensor pipe is as busy as the XU)
-    static constexpr int kPolyOf16 = (DH == 64) ? 6 : (DH == 72) ? 4 : 0;
+    // Pairs of exponentials that are computed on the FMA pipe instead of the XU: three of eight at head_dim 64 and 128,
+    // one of four at 72 (us a launch, under the power cap: head_dim 64, 9001 x 17776 x 48 heads, 4 / 5 / 6 / 7 / 8 of 16:
+    // 2143 / 2123 / 2083 / 2140 / 2203; 72, 2 x 6553 x 16384 x 16, 2 / 4 / 5 / 6 / 8: 1190 / 1150 / 1152 / 1165 / 1233; 128,
+    // 3276 x 65536 x 24, none / 5 / 6 / 7 / 8: 2250 / 2170 / 2130 / 2457 / 2400).  Degree 3 where the row sum or the sums of P
+    // had that error already, 5 at head_dim 128, whose LSE keeps the precision it has with the XU alone.
+    static constexpr int kPolyPeriod = (DH == 72) ? 4 : 8;
+    static constexpr int kPolyPairs = (DH == 72) ? 1 : 3;
+    static constexpr int kPolyDeg = (DH == 128) ? 5 : 3;
     static constexpr int kSoftmaxWarps = 4 * kTilesM * kSplit;
     static constexpr int kAhead = kSBufs;                         // Q K^T runs this many key tiles ahead of P V
     static constexpr int kThreads = (kSoftmaxWarps + 4) * 32;     // + producer, two issuers, one register donor
@@ -164,29 +169,55 @@ __device__ __forceinline__ unsigned long long fadd2(unsigned long long a, float 
     return r;
 }
 
-// 2^x for a pair, without the XU pipe: x = n + f with n = floor(x) taken by adding 1.5 * 2^23 rounded down, a
-// cubic for 2^f on [0, 1) (relative error 8.6e-5, well below the bf16 rounding of P), and n added to the
-// exponent field.  x is clamped to the normal range first: below it the result is 2^-126 instead of 0, which no sum
-// notices; above it the exponent field would wrap around to a small number and hide the overflow from the check
-// on the tile's sum, so x stops at 127, whose 2^127 trips that check as surely as the XU's +inf does.
-__device__ __forceinline__ void exp2_poly2(float &x0, float &x1) {
-    x0 = fminf(fmaxf(x0, -126.0f), 127.0f);
-    x1 = fminf(fmaxf(x1, -126.0f), 127.0f);
-    unsigned long long x, t, pl;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(x0), "f"(x1));
-    asm("{\n\t.reg .b64 mg, c1, c2, c3, one, fr;\n\t"
-        "mov.b64 mg, 0x4B4000004B400000;\n\t"        // 1.5 * 2^23, twice
-        "mov.b64 c3, 0x3D9DD4DF3D9DD4DF;\n\t"        // 2^f ~ 1 + f (c1 + f (c2 + f c3))
-        "mov.b64 c2, 0x3E691C043E691C04;\n\t"
-        "mov.b64 c1, 0x3F31F3293F31F329;\n\t"
-        "mov.b64 one, 0x3F8000003F800000;\n\t"
-        "add.rm.f32x2 %0, %2, mg;\n\t"               // low mantissa bits of t = floor(x)
-        "sub.rn.f32x2 fr, %0, mg;\n\t"
-        "sub.rn.f32x2 fr, %2, fr;\n\t"               // f = x - floor(x)
-        "fma.rn.f32x2 %1, fr, c3, c2;\n\t"
-        "fma.rn.f32x2 %1, %1, fr, c1;\n\t"
-        "fma.rn.f32x2 %1, %1, fr, one;\n\t}"
-        : "=&l"(t), "=&l"(pl) : "l"(x));
+// 2^x for a pair of logits s, x = s * sl2 + neg, without the XU pipe: x = n + f with n = floor(x) taken by adding
+// 1.5 * 2^23 rounded down, a polynomial for 2^f on [0, 1) (fitted here for the least relative error with p(0) = 1: 8.6e-5
+// in degree 3, 1.6e-7, as much as ex2.approx has, in degree 5), and n added to the exponent field.  x has to stay in the
+// range of normal numbers: below -126 the result is 2^-126 instead of 0, which no sum notices; above 127 the exponent
+// field would wrap around to a small number and hide the overflow from the check on the sums, so x stops at 127, whose
+// 2^127 trips that check as surely as the XU's +inf does.  Both limits come with the scaling, for one instruction per logit
+// instead of two and a half: the saturating FMA leaves u = (x + 126) / 253 clamped to [0, 1] (mul = sl2 / 253,
+// add = (neg + 126) / 253; 3e-8 of rounding in u is 8e-6 in x, either way), and x = 253 u - 126 is never formed, only its
+// floor and its fraction are.
+constexpr float kExpLo = -126.0f, kExpSpan = 253.0f;
+template <int DEG>
+__device__ __forceinline__ void exp2_poly2(float &x0, float &x1, float mul, float add) {
+    float u0, u1;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(u0) : "f"(x0), "f"(mul), "f"(add));
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(u1) : "f"(x1), "f"(mul), "f"(add));
+    unsigned long long u, t, f, pl;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(u) : "f"(u0), "f"(u1));
+    asm("{\n\t.reg .b64 mg, sp;\n\t"
+        "mov.b64 mg, 0x4B3FFF824B3FFF82;\n\t"        // 1.5 * 2^23 - 126, twice
+        "mov.b64 sp, 0x437D0000437D0000;\n\t"        // 253
+        "fma.rm.f32x2 %0, %2, sp, mg;\n\t"           // 1.5 * 2^23 + floor(x): the low mantissa bits are floor(x)
+        "sub.rn.f32x2 %1, mg, %0;\n\t"               // -126 - floor(x)
+        "fma.rn.f32x2 %1, %2, sp, %1;\n\t}"          // f = x - floor(x)
+        : "=&l"(t), "=&l"(f) : "l"(u));
+    static_assert(DEG == 3 || DEG == 5, "fitted degrees");
+    if constexpr (DEG == 3)
+        asm("{\n\t.reg .b64 c1, c2, c3, one;\n\t"
+            "mov.b64 c3, 0x3D9DD4DF3D9DD4DF;\n\t"        // 2^f ~ 1 + f (c1 + f (c2 + f c3))
+            "mov.b64 c2, 0x3E691C043E691C04;\n\t"
+            "mov.b64 c1, 0x3F31F3293F31F329;\n\t"
+            "mov.b64 one, 0x3F8000003F800000;\n\t"
+            "fma.rn.f32x2 %0, %1, c3, c2;\n\t"
+            "fma.rn.f32x2 %0, %0, %1, c1;\n\t"
+            "fma.rn.f32x2 %0, %0, %1, one;\n\t}"
+            : "=&l"(pl) : "l"(f));
+    else
+        asm("{\n\t.reg .b64 c1, c2, c3, c4, c5, one;\n\t"
+            "mov.b64 c5, 0x3AF4BA7D3AF4BA7D;\n\t"        // 1 + f (c1 + f (c2 + f (c3 + f (c4 + f c5))))
+            "mov.b64 c4, 0x3C13BC2B3C13BC2B;\n\t"
+            "mov.b64 c3, 0x3D648E733D648E73;\n\t"
+            "mov.b64 c2, 0x3E75EDAB3E75EDAB;\n\t"
+            "mov.b64 c1, 0x3F31725D3F31725D;\n\t"
+            "mov.b64 one, 0x3F8000003F800000;\n\t"
+            "fma.rn.f32x2 %0, %1, c5, c4;\n\t"
+            "fma.rn.f32x2 %0, %0, %1, c3;\n\t"
+            "fma.rn.f32x2 %0, %0, %1, c2;\n\t"
+            "fma.rn.f32x2 %0, %0, %1, c1;\n\t"
+            "fma.rn.f32x2 %0, %0, %1, one;\n\t}"
+            : "=&l"(pl) : "l"(f));
     uint32_t t0, t1, p0, p1;
     asm("mov.b64 {%0, %1}, %2;" : "=r"(t0), "=r"(t1) : "l"(t));
     asm("mov.b64 {%0, %1}, %2;" : "=r"(p0), "=r"(p1) : "l"(pl));
@@ -325,15 +356,14 @@ __device__ __forceinline__ void softmax_step(SoftmaxState &st, int j, int g)
         else asm volatile("bar.arrive 4, 256;" ::: "memory");
     }
     const float neg = -st.m_ref * sl2 - st.shift;
+    const float mul = sl2 * (1.0f / kExpSpan), add = (neg - kExpLo) * (1.0f / kExpSpan);
+    // the first kPolyPairs of every kPolyPeriod pairs go to the FMA pipe, the rest to the XU
 #pragma unroll
-    for (int i = 0; i < NS; i += 2) ffma2(cur[i], cur[i + 1], sl2, neg);
-    // kPolyOf16 of every 16 exponentials go to the FMA pipe, the rest to the XU
-#pragma unroll
-    for (int i = 0; i < NS; i += 16) {
-#pragma unroll
-        for (int u = 0; u < 16; u += 2) {
-            if (u >= 16 - C::kPolyOf16) exp2_poly2(cur[i + u], cur[i + u + 1]);
-            else { cur[i + u] = ex2(cur[i + u]); cur[i + u + 1] = ex2(cur[i + u + 1]); }
+    for (int i = 0; i < NS; i += 2) {
+        if ((i / 2) % C::kPolyPeriod < C::kPolyPairs) exp2_poly2<C::kPolyDeg>(cur[i], cur[i + 1], mul, add);
+        else {
+            ffma2(cur[i], cur[i + 1], sl2, neg);
+            cur[i] = ex2(cur[i]); cur[i + 1] = ex2(cur[i + 1]);
         }
     }
     float tile_sum = 0.f;
