@@ -101,8 +101,7 @@ template <int DH, int TM> struct Cfg {
     static constexpr int kAhead = kSBufs;                         // Q K^T runs this many key tiles ahead of P V
     static constexpr int kThreads = (kSoftmaxWarps + 4) * 32;     // + producer, two issuers, one register donor
     static constexpr uint32_t kColO = kTilesM * kSBufs * kBlockN; // first O column
-    static constexpr uint32_t kOnesCol = kMain + kTailPad;       // accumulator column that receives the row sums
-    static constexpr uint32_t kOStride = kMain + kTailPad + (kOnes ? 16 : 0);   // columns between O accumulators
+    static constexpr uint32_t kOStride = kMain + kTailPad + (kOnes ? 16 : 0);   // columns between O accumulators (the row sums come right behind O)
     static_assert(kColO + kTilesM * kOStride <= kTmemCols, "TMEM budget");
     // setmaxnreg only redistributes what the CTA got at launch: an increase that the decreases of
     // the last warpgroup cannot cover would block forever
@@ -122,7 +121,7 @@ template <int DH, int TM> struct Cfg {
     static constexpr int kStagesV = (kCtasPerSM == 2) ? 4 : (DH == 128) ? 4 : 6;
     static_assert(kStagesK > kAhead, "K runs kAhead tiles ahead");
     static constexpr int kBarBytes = 512;
-    static constexpr int kOnesBytes = kOnes ? kBlockN * 32 : 0;  // a key tile x 16 columns of bf16: ones in column 0
+    static constexpr int kOnesBytes = kOnes ? kBlockN * 128 : 0; // a key tile x one 64-column chunk of bf16: ones in column 0
     static constexpr int kSmemBytes = kQTileBytes * kTilesM + kTileBytes * (kStagesK + kStagesV) + kOnesBytes + kBarBytes + 1024;
 };
 
@@ -483,7 +482,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
         // the reference was too low somewhere along the row
         tc_fence_after();
         uint32_t o[8];
-        tmem_ld8(st.t_o + C::kOnesCol, o);
+        tmem_ld8(st.t_o + C::kMain, o);
         tc_wait_ld();
         st.l_sum = __uint_as_float(o[0]);
         if (__any_sync(0xffffffffu, !(st.l_sum <= kTileSumLimit))) *redo_flag = 1;
@@ -504,7 +503,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
         if constexpr (C::kOnes) {
             tc_fence_after();
             uint32_t o[8];
-            tmem_ld8(st.t_o + C::kOnesCol, o);
+            tmem_ld8(st.t_o + C::kMain, o);
             tc_wait_ld();
             st.l_sum = __uint_as_float(o[0]);
         }
@@ -645,7 +644,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     const uint32_t sQ = smem_base;
     const uint32_t sK = sQ + kTilesM * C::kQTileBytes;
     const uint32_t sV = sK + C::kStagesK * C::kTileBytes;
-    const uint32_t sOnes = sV + C::kStagesV * C::kTileBytes;       // [key tile x 16 columns] bf16, 32-byte swizzle, column 0 = 1
+    const uint32_t sOnes = sV + C::kStagesV * C::kTileBytes;       // [key tile x 64 columns] bf16, 128-byte swizzle, column 0 = 1
     const uint32_t bars = sOnes + C::kOnesBytes;
     Bars bar;
     bar.q = bars; bar.s = bars + 16; bar.p = bars + 80; bar.done = bars + 144;
@@ -674,12 +673,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     const int q_tiles = (m0 + kBlockM < p.M) ? kTilesM : 1;
 
     if constexpr (C::kOnes) {
-        // row r: 32 bytes; the 16-byte unit that holds column 0 is unit (r >> 2) & 1 under the 32-byte swizzle
+        // row r: 128 bytes; under the 128-byte swizzle the 16-byte unit that holds column 0 is unit r & 7
         uint8_t *ones = smem_gen + (sOnes - smem_base);
-        for (int i = tid; i < kBlockN * 2; i += C::kThreads) {
-            const int r = i >> 1, unit = i & 1;
-            const uint32_t first = (unit == ((r >> 2) & 1)) ? 0x3F80u : 0u;      // bf16 1.0 in column 0
-            *reinterpret_cast<uint4 *>(ones + r * 32 + unit * 16) = make_uint4(first, 0u, 0u, 0u);
+        for (int i = tid; i < kBlockN * 8; i += C::kThreads) {
+            const int r = i >> 3, unit = i & 7;
+            const uint32_t first = (unit == (r & 7)) ? 0x3F80u : 0u;      // bf16 1.0 in column 0
+            *reinterpret_cast<uint4 *>(ones + r * 128 + unit * 16) = make_uint4(first, 0u, 0u, 0u);
         }
         fence_proxy_async_smem();
     }
@@ -798,7 +797,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
         // ------------------------------------------------ MMA issuer (warp-uniform, one elected lane issues)
         constexpr uint32_t idesc_qk = idesc_bf16(kBlockM, kBlockN, false);
-        constexpr uint32_t idesc_pv = idesc_bf16(kBlockM, C::kMain, true);
+        // (the ones chunk lies behind V's columns: the leading offset of the descriptor leads from the stage to it, and one MMA of
+        // kMain + 16 columns does both)
+        constexpr uint32_t idesc_pv = idesc_bf16(kBlockM, C::kMain + (C::kOnes ? 16 : 0), true);
         constexpr uint32_t idesc_pv_tail = idesc_bf16(kBlockM, 16, true);
         // S[t][g % kSBufs] = Q_t K^T of the key tile in shared memory at kbase (one elected lane); g counts the
         // S-buffer uses of the query tile over all passes
@@ -851,15 +852,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
 #pragma unroll
                         for (int ks = 0; ks < kBlockN / 16; ++ks) {
                             mma_ts(tmem + o_col, tmem + (t * kSBufs + u) * kBlockN + ks * 8,
-                                   smem_desc(vbase + ks * 2048, C::kChunkBytes, 1024, kSwizzle128B),
+                                   smem_desc(vbase + ks * 2048, C::kOnes ? sOnes - vbase : C::kChunkBytes, 1024, kSwizzle128B),
                                    idesc_pv, (j > 0 || ks > 0) ? 1u : 0u);
                             if (C::kTail)  // O columns 64..79 from the 16-column chunk of V
                                 mma_ts(tmem + o_col + C::kMain, tmem + (t * kSBufs + u) * kBlockN + ks * 8,
                                        smem_desc(vbase + C::kChunks * C::kChunkBytes + ks * 512, 256, 256, kSwizzle32B),
-                                       idesc_pv_tail, (j > 0 || ks > 0) ? 1u : 0u);
-                            if (C::kOnes)  // the row sums: P times the column of ones
-                                mma_ts(tmem + o_col + C::kOnesCol, tmem + (t * kSBufs + u) * kBlockN + ks * 8,
-                                       smem_desc(sOnes + ks * 512, 256, 256, kSwizzle32B),
                                        idesc_pv_tail, (j > 0 || ks > 0) ? 1u : 0u);
                         }
                         tc_commit(bar.ve + 8 * sv);
