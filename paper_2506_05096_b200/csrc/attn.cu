@@ -420,7 +420,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
         const int m = m_base + r;
         gtok[it] = -1;
         if (m < p.M && c * 8 < C::kDH)                   // the upper half of the tail chunk stays zero
-            gtok[it] = p.q_idx ? __ldg(p.q_idx + (size_t)b * p.M + m) : m;
+            gtok[it] = p.q_idx ? __ldcg(p.q_idx + (size_t)b * p.M + m) : m;
     }
     uint4 gval[kGatherIters];
 #pragma unroll
@@ -430,7 +430,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
         gval[it] = make_uint4(0, 0, 0, 0);
         if ((unsigned)gtok[it] < (unsigned)p.N_tok) {
             const __nv_bfloat16 *src = p.q + (size_t)b * p.q_sb + (size_t)gtok[it] * p.q_sn + (size_t)h * p.q_sh + c * 8;
-            gval[it] = __ldg(reinterpret_cast<const uint4 *>(src));
+            gval[it] = __ldcg(reinterpret_cast<const uint4 *>(src));
         }
     }
 #pragma unroll
@@ -459,11 +459,11 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
     const int m = m_base + wtid;
     int tok = -1;
     if (m < p.M) {
-        tok = p.q_idx ? __ldg(p.q_idx + (size_t)b * p.M + m) : m;
+        tok = p.q_idx ? __ldcg(p.q_idx + (size_t)b * p.M + m) : m;
         // an entry out of range, or one that does not exceed its predecessor (two rows would race on one output
         // row), is reported and its row is not written
         const bool bad = (unsigned)tok >= (unsigned)p.N_tok ||
-                         (p.q_idx && m > 0 && __ldg(p.q_idx + (size_t)b * p.M + m - 1) >= tok);
+                         (p.q_idx && m > 0 && __ldcg(p.q_idx + (size_t)b * p.M + m - 1) >= tok);
         if (bad) { if (par == 0 && p.err_word) atomicExch(p.err_word, kErrBadIndex); tok = -1; }
     }
 
@@ -510,6 +510,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
     }
 
     // ------------------------------------------------ epilogue: normalise and scatter
+    grid_launch_dependents();
     tc_fence_after();
     // both warpgroups accumulated into one O against one reference: add the row sums, split the columns
     float l_sum = st.l_sum;                                      // with the ones column: the row's whole sum already
@@ -698,10 +699,13 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     // (nobody else touches these barriers or the stages before that barrier).
     if (warp == kProducerWarp) {
         if (elect_one()) {
+            prefetch_tensormap(&tmap_k); prefetch_tensormap(&tmap_v);
+            if (C::kTail) { prefetch_tensormap(&tmap_k_tail); prefetch_tensormap(&tmap_v_tail); }
             // a K/V stage is free once the issuer of every active query tile has committed its MMAs on it
             for (int s = 0; s < C::kStagesK; ++s) { mbar_init(bar.kf + 8 * s, 1); mbar_init(bar.ke + 8 * s, q_tiles); }
             for (int s = 0; s < C::kStagesV; ++s) { mbar_init(bar.vf + 8 * s, 1); mbar_init(bar.ve + 8 * s, q_tiles); }
             fence_barrier_init();
+            grid_dependency_wait();
             for (int j = 0; j < kAhead && j < n_tiles; ++j) {
                 mbar_arrive_expect_tx(bar.kf + 8 * j, C::kLoadBytes);
 #pragma unroll
@@ -727,6 +731,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    grid_dependency_wait();
 
     if (warp < C::kSoftmaxWarps) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsSoftmax));
@@ -739,10 +744,6 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     } else if (warp == kProducerWarp) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
         // ------------------------------------------------ TMA producer (warp-uniform, one elected lane issues)
-        if (elect_one()) {
-            prefetch_tensormap(&tmap_k); prefetch_tensormap(&tmap_v);
-            if (C::kTail) { prefetch_tensormap(&tmap_k_tail); prefetch_tensormap(&tmap_v_tail); }
-        }
         // g: running count of K (or V) tiles over all passes: stage g % kStages, phase (g / kStages) & 1
         auto load_k = [&](int g, int j) {
             const int st = g % C::kStagesK;
@@ -896,14 +897,16 @@ template <int DH, int ROWS>
 __global__ void __launch_bounds__(ROWS) merge_parts_kernel(const Params p)
 {
     constexpr int kChunksRow = DH / 8;
+    grid_launch_dependents();
+    grid_dependency_wait();
     const int unit = p.n_full + blockIdx.y;
     const int m0 = (unit % p.tiles_x) * ROWS, h = p.h0 + (unit / p.tiles_x) % p.heads, b = unit / (p.tiles_x * p.heads);
     const int idx = blockIdx.x * ROWS + threadIdx.x;
     const int r = idx / kChunksRow, c = idx - r * kChunksRow;
     const int m = m0 + r;
     if (m >= p.M) return;
-    const int tok = p.q_idx ? __ldg(p.q_idx + (size_t)b * p.M + m) : m;
-    if ((unsigned)tok >= (unsigned)p.N_tok || (p.q_idx && m > 0 && __ldg(p.q_idx + (size_t)b * p.M + m - 1) >= tok)) return;   // reported by the attention kernel
+    const int tok = p.q_idx ? __ldcg(p.q_idx + (size_t)b * p.M + m) : m;
+    if ((unsigned)tok >= (unsigned)p.N_tok || (p.q_idx && m > 0 && __ldcg(p.q_idx + (size_t)b * p.M + m - 1) >= tok)) return;   // reported by the attention kernel
     const size_t part0 = (size_t)blockIdx.y * p.split;
     float lse[8], mx = -INFINITY;
     bool gave_up = false;
@@ -911,7 +914,7 @@ __global__ void __launch_bounds__(ROWS) merge_parts_kernel(const Params p)
     for (int i = 0; i < 8; ++i) {
         lse[i] = -INFINITY;
         if (i < p.split) {
-            lse[i] = __ldg(p.part_lse + (part0 + i) * ROWS + r);
+            lse[i] = __ldcg(p.part_lse + (part0 + i) * ROWS + r);
             gave_up |= lse[i] != lse[i];
             mx = fmaxf(mx, lse[i]);
         }
@@ -924,7 +927,7 @@ __global__ void __launch_bounds__(ROWS) merge_parts_kernel(const Params p)
             const float w = __expf(lse[i] - mx);
             wsum += w;
             const float4 *src = reinterpret_cast<const float4 *>(p.part_o + ((part0 + i) * ROWS + r) * DH + c * 8);
-            const float4 a = __ldg(src), d = __ldg(src + 1);
+            const float4 a = __ldcg(src), d = __ldcg(src + 1);
             acc[0] += w * a.x; acc[1] += w * a.y; acc[2] += w * a.z; acc[3] += w * a.w;
             acc[4] += w * d.x; acc[5] += w * d.y; acc[6] += w * d.z; acc[7] += w * d.w;
         }
@@ -1028,10 +1031,10 @@ int32_t launch_dh(const AttnArgs &a, cudaStream_t stream, SplitPlan plan = Split
         p.part_o = p.part_lse + (rows + 63) / 64 * 64;
     }
     const unsigned grid = (unsigned)(p.n_full + (split ? plan.units * plan.split : 0));
-    sparse_attn_kernel<C><<<grid, C::kThreads, C::kSmemBytes, stream>>>(mk, mv, mkt, mvt, p);
+    launch_overlapped(sparse_attn_kernel<C>, grid, C::kThreads, C::kSmemBytes, stream, mk, mv, mkt, mvt, p);
     if (split) {
         static_assert((TM * kBlockM * (DH / 8)) % (TM * kBlockM) == 0, "whole blocks per unit");
-        merge_parts_kernel<DH, TM * kBlockM><<<dim3(DH / 8, plan.units), TM * kBlockM, 0, stream>>>(p);
+        launch_overlapped(merge_parts_kernel<DH, TM * kBlockM>, dim3(DH / 8, plan.units), TM * kBlockM, 0, stream, p);
     }
     return check_launch("astraea_sparse_attn");
 }
@@ -1060,6 +1063,8 @@ __global__ void __launch_bounds__(256)
 gather_kv_kernel(uint4 *__restrict__ dst, const __nv_bfloat16 *__restrict__ src, int64_t sb, int64_t sh, int64_t sn,
                  const int32_t *__restrict__ idx, int B, int H, int N, int M_kv, int vec_per_row, int *err_word)
 {
+    grid_launch_dependents();
+    grid_dependency_wait();
     const long long total = (long long)B * M_kv * H * vec_per_row;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
         const int v = (int)(t % vec_per_row);
@@ -1067,9 +1072,9 @@ gather_kv_kernel(uint4 *__restrict__ dst, const __nv_bfloat16 *__restrict__ src,
         const int h = (int)(r % H); r /= H;
         const int m = (int)(r % M_kv);
         const int b = (int)(r / M_kv);
-        const int tok = __ldg(idx + (size_t)b * M_kv + m);
+        const int tok = __ldcg(idx + (size_t)b * M_kv + m);
         uint4 val = make_uint4(0, 0, 0, 0);
-        if ((unsigned)tok < (unsigned)N) val = __ldg(reinterpret_cast<const uint4 *>(src + b * sb + tok * sn + h * sh) + v);
+        if ((unsigned)tok < (unsigned)N) val = __ldcg(reinterpret_cast<const uint4 *>(src + b * sb + tok * sn + h * sh) + v);
         else if (v == 0 && h == 0) atomicExch(err_word, kErrBadIndex);
         dst[t] = val;
     }
@@ -1090,9 +1095,9 @@ int32_t launch_sparse_attn_kv(AttnArgs a, const int32_t *kv_idx, int M_kv, void 
     const long long total = (long long)a.B * M_kv * a.H * vec;
     const long long cap = (long long)sm_count() * 16;
     const int grid = (int)((total + 255) / 256 < cap ? (total + 255) / 256 : cap);
-    gather_kv_kernel<<<grid, 256, 0, stream>>>(kc, reinterpret_cast<const __nv_bfloat16 *>(a.k), a.k_sb, a.k_sh, a.k_sn,
+    launch_overlapped(gather_kv_kernel, grid, 256, 0, stream, kc, reinterpret_cast<const __nv_bfloat16 *>(a.k), a.k_sb, a.k_sh, a.k_sn,
                                                kv_idx, a.B, a.H, a.N, M_kv, vec, a.err_word);
-    gather_kv_kernel<<<grid, 256, 0, stream>>>(vc, reinterpret_cast<const __nv_bfloat16 *>(a.v), a.v_sb, a.v_sh, a.v_sn,
+    launch_overlapped(gather_kv_kernel, grid, 256, 0, stream, vc, reinterpret_cast<const __nv_bfloat16 *>(a.v), a.v_sb, a.v_sh, a.v_sn,
                                                kv_idx, a.B, a.H, a.N, M_kv, vec, a.err_word);
     int32_t rc = check_launch("astraea_sparse_attn (gather of K/V)");
     if (rc != ASTRAEA_OK) return rc;

@@ -45,6 +45,41 @@ void set_error(const char *fmt, ...);
 int32_t fail(int32_t code, const char *fmt, ...);
 int32_t check_launch(const char *what);
 
+// Programmatic dependent launch.  Every kernel but the scatter is launched with it (launch_overlapped) and starts with
+// its own set-up (barriers, TMEM, descriptors, cleared histograms) while the kernel before it in the stream drains, then
+// waits: grid_dependency_wait() comes before a kernel's first access to global memory, in every thread, so that a kernel
+// has completed only when all kernels before it have.  grid_launch_dependents() lets the next kernel's CTAs in once all
+// CTAs of this one have called it.  Kernels that share an SM with others call it at their start; the tensor-core kernels,
+// whose CTA takes the whole SM, call it at their last epilogue: by then a CTA has long got its TMEM (a CTA of the next
+// kernel must not take columns that one of this kernel still has to get), and the next kernel's CTAs find all SMs free or
+// about to be (called at the start, a kernel behind an attention launch of 120 CTAs went to the 28 idle SMs as a whole).  What an earlier kernel of the library may have written is read through L2 (ld.cg, TMA) or
+// without .nc, never through the read-only path: a line of it may sit in the SM's L1 from before.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// 16-byte load of data that is used once (no L1 allocation)
+__device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
+    uint4 r;
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    return r;
+}
+
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // kernel launchers (one per .cu file)

@@ -15,12 +15,6 @@ constexpr int kWarpsPerBlock = 8;
 constexpr int kBlocksPerSM = 8;
 constexpr int kMaxVecPerLane = 16;     // rows of up to 32 * 16 * 8 = 4096 channels
 
-__device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
-    uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
-    return r;
-}
 __device__ __forceinline__ void unpack8(const uint4 &v, float (&f)[8]) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -36,13 +30,15 @@ layernorm_modulate_kernel(const uint4 *__restrict__ x, const int32_t *__restrict
                           const uint4 *__restrict__ shift, uint4 *__restrict__ y, int B, int N, int vec_per_row, float eps,
                           int compact_in, int compact_out, int *__restrict__ err_word)
 {
+    grid_launch_dependents();
+    grid_dependency_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long total = (long long)B * M;
     const float inv_D = 1.0f / (float)(vec_per_row * 8);
     for (long long t = (long long)blockIdx.x * kWarpsPerBlock + warp; t < total; t += (long long)gridDim.x * kWarpsPerBlock) {
         const int b = (int)(t / M), r = (int)(t - (long long)b * M);
-        const int tok = idx ? __ldg(idx + t) : r;
-        if ((unsigned)tok >= (unsigned)N || (idx && r > 0 && __ldg(idx + t - 1) >= tok)) {      // see astraea_scatter_reuse
+        const int tok = idx ? __ldcg(idx + t) : r;
+        if ((unsigned)tok >= (unsigned)N || (idx && r > 0 && __ldcg(idx + t - 1) >= tok)) {      // see astraea_scatter_reuse
             if (lane == 0 && err_word) atomicExch(err_word, kErrBadIndex);
             continue;
         }
@@ -114,13 +110,13 @@ int32_t launch_layernorm_modulate(const void *x, const int32_t *idx, int M, cons
     const int ci = (flags & ASTRAEA_LN_COMPACT_IN) ? 1 : 0, co = (flags & ASTRAEA_LN_COMPACT_OUT) ? 1 : 0;
     dim3 block(kWarpsPerBlock * 32);
     if (vec_per_row <= 32 * 4)
-        layernorm_modulate_kernel<4><<<grid, block, 0, stream>>>(xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
+        launch_overlapped(layernorm_modulate_kernel<4>, grid, block, 0, stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
     else if (vec_per_row <= 32 * 8)
-        layernorm_modulate_kernel<8><<<grid, block, 0, stream>>>(xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
+        launch_overlapped(layernorm_modulate_kernel<8>, grid, block, 0, stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
     else if (vec_per_row <= 32 * 12)
-        layernorm_modulate_kernel<12><<<grid, block, 0, stream>>>(xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
+        launch_overlapped(layernorm_modulate_kernel<12>, grid, block, 0, stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
     else
-        layernorm_modulate_kernel<16><<<grid, block, 0, stream>>>(xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
+        launch_overlapped(layernorm_modulate_kernel<16>, grid, block, 0, stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
     return check_launch("astraea_layernorm_modulate");
 }
 

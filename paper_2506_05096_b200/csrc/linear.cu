@@ -107,8 +107,8 @@ __device__ __forceinline__ bool target_row(const LinParams &p, long long g, long
     *bad = false;
     if (g >= total) return false;
     const int b = (int)((unsigned)g / (unsigned)p.M), r = (int)((unsigned)g - (unsigned)b * (unsigned)p.M);   // fewer than 2^31 rows fit the device
-    const int tok = p.idx ? __ldg(p.idx + g) : r;
-    const int before = (p.idx && r > 0) ? __ldg(p.idx + g - 1) : -1;
+    const int tok = p.idx ? __ldcg(p.idx + g) : r;
+    const int before = (p.idx && r > 0) ? __ldcg(p.idx + g - 1) : -1;
     // not strictly ascending: a row would be written twice
     if ((unsigned)tok >= (unsigned)p.N || (r > 0 && before >= tok)) { *bad = true; return false; }
     *out_row = p.compact ? g : (long long)b * p.N + tok;
@@ -154,6 +154,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
         for (int a = 0; a < kAccSets; ++a) { mbar_init(bar_acc_full + 8 * a, 1); mbar_init(bar_acc_empty + 8 * a, 2 * kEpiWarps); }
         fence_barrier_init();
     }
+    if (warp == kTmaWarp && elect_one()) { prefetch_tensormap(&tmap_w); if (DENSE) prefetch_tensormap(&tmap_x); }
     if (warp == kMmaWarp) {
         tmem_alloc_pair(smem_u32(&tmem_slot), kTmemCols);
         tmem_relinquish_pair();
@@ -162,6 +163,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
     __syncthreads();
     cluster_sync_all();                                            // the barriers of both CTAs are set up
     tc_fence_after();
+    grid_dependency_wait();
     const uint32_t tmem = tmem_slot;
 
     if (warp < kEpiWarps) {
@@ -184,6 +186,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
             if (!p.residual) res_row = -1;
             const __nv_bfloat16 *gate = p.gate ? p.gate + (long long)batch * p.N_out : nullptr;
             wait_bar(bar_acc_full + 8 * acc, (it / kAccSets) & 1, &abort_flag, p.err_word);
+            if (tile + n_pairs >= total_tiles) grid_launch_dependents();       // the last epilogue of this CTA
             tc_fence_after();
             if (abort_flag) out_row = -1;
             auto release = [&] {                                   // this warp's part of the accumulator has been read
@@ -208,7 +211,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
                     for (int jj = 0; jj < 4; ++jj) {
                         const int r = (lane >> 2) + 8 * jj;
                         const long long rrow = __shfl_sync(0xffffffffu, res_row, r);
-                        rr[jj] = (rrow >= 0 && colq < p.N_out) ? __ldg(reinterpret_cast<const uint4 *>(p.residual + rrow * p.N_out + colq))
+                        rr[jj] = (rrow >= 0 && colq < p.N_out) ? __ldcg(reinterpret_cast<const uint4 *>(p.residual + rrow * p.N_out + colq))
                                                                 : make_uint4(0, 0, 0, 0);
                     }
 #pragma unroll
@@ -286,7 +289,6 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
         }
     } else if (warp == kTmaWarp) {
         // ------------------------------------------------ TMA producer of the W tiles (and of contiguous rows of x)
-        if (elect_one()) { prefetch_tensormap(&tmap_w); if (DENSE) prefetch_tensormap(&tmap_x); }
         int g = 0;
         for (int tile = pair; tile < total_tiles; tile += n_pairs) {
             const int tm = tile / tiles_n, tn = tile - tm * tiles_n;
@@ -355,7 +357,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
 #pragma unroll
             for (int i = 0; i < kEnt; ++i) {
                 const long long r = (long long)(tile / tiles_n) * kBM + (int)rank * kRowsCta + t + i * kGatherThreads;
-                ent[i] = (tile < total_tiles && r < total_rows) ? __ldg(p.idx + r) : -1;
+                ent[i] = (tile < total_tiles && r < total_rows) ? __ldcg(p.idx + r) : -1;
             }
         };
         fetch(pair);
@@ -428,7 +430,7 @@ int32_t launch_linear(const LinParams &p, const void *x, const void *w, int pair
         return check_launch("astraea_gathered_linear (shared memory attribute)");
     const long long tiles = (((long long)p.B * p.M + kBM - 1) / kBM) * ((p.N_out + p.bn - 1) / p.bn);
     const int grid = 2 * (int)(tiles < pairs ? tiles : pairs);
-    gathered_linear_kernel<DENSE><<<grid, kThreads<DENSE>, kSmemBytes, stream>>>(mw, mx, p);
+    launch_overlapped(gathered_linear_kernel<DENSE>, grid, kThreads<DENSE>, kSmemBytes, stream, mw, mx, p);
     return check_launch("astraea_gathered_linear");
 }
 

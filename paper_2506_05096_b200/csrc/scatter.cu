@@ -12,13 +12,6 @@ constexpr int kWarpsPerBlock = 8;
 constexpr int kBlocksPerSM = 16;
 constexpr int kUnroll = 6;
 
-__device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
-    uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
-    return r;
-}
-
 // LPR lanes copy one row: 32 for wide rows; 16 or 8 for narrow ones, so that a warp moves two or four rows at once and
 // every lane keeps several 16-byte loads in flight.
 template <int LPR>
@@ -39,10 +32,10 @@ scatter_kernel(uint4 *__restrict__ cache, const uint4 *__restrict__ rows, const 
         if (t >= total) continue;
         const int b = (int)(t / M);
         const int r = (int)(t - (long long)b * M);
-        const int i = __ldg(idx + t);
+        const int i = __ldcg(idx + t);
         // never write outside the cache, and never write a row twice: an entry that is out of range or does not
         // exceed its predecessor is skipped and reported
-        if ((unsigned)i >= (unsigned)N || (r > 0 && __ldg(idx + t - 1) >= i)) {
+        if ((unsigned)i >= (unsigned)N || (r > 0 && __ldcg(idx + t - 1) >= i)) {
             if (sl == 0 && err_word) atomicExch(err_word, kErrBadIndex);
             continue;
         }
@@ -72,6 +65,8 @@ int32_t launch_scatter(void *cache, const void *rows, const int32_t *idx, int B,
     long long want = (total + rows_per_block - 1) / rows_per_block;
     const long long cap = (long long)sm_count() * kBlocksPerSM;
     int grid = (int)(want < cap ? want : cap);
+    // An ordinary launch: with a programmatic one behind the attention the step of 1132 x 3594 tokens (24 heads of 128) took 74
+    // us instead of 69 (71 with no programmatic launches at all).
     uint4 *c = reinterpret_cast<uint4 *>(cache);
     const uint4 *rw = reinterpret_cast<const uint4 *>(rows);
     const int full = (flags & ASTRAEA_SCATTER_SRC_FULL) ? 1 : 0;

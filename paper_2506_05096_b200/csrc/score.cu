@@ -15,13 +15,6 @@ constexpr int kWarpsPerBlock = 8;
 constexpr int kBlocksPerSM = 16;     // twice what is resident: the second half evens out the tail
 constexpr int kUnroll = 6;           // 16-byte loads in flight per lane and tensor
 
-__device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
-    uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
-    return r;
-}
-
 template <int MODE>
 __device__ __forceinline__ float accum_pair(uint32_t a, uint32_t b, float acc) {
     // two bf16 per word: low half = even element
@@ -55,7 +48,8 @@ score_kernel(const uint4 *__restrict__ x_cur, const uint4 *__restrict__ x_ref,
 {
     // a kernel launched behind this one with programmatic stream serialization (the selection) may become resident
     // and set itself up as soon as SMs free up; it still waits for this whole grid before it reads the scores
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    grid_launch_dependents();
+    grid_dependency_wait();
     constexpr int kRowsPerWarp = 32 / LPR;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -83,9 +77,9 @@ score_kernel(const uint4 *__restrict__ x_cur, const uint4 *__restrict__ x_ref,
 #pragma unroll
         for (int u = 0; u < kLsePre; ++u) {
             const int h = sl + LPR * u;
-            lv[u] = (lse != nullptr && have && h < H) ? __ldg(lse + ((size_t)b * H + h) * N + i) : 0.f;
+            lv[u] = (lse != nullptr && have && h < H) ? __ldcg(lse + ((size_t)b * H + h) * N + i) : 0.f;
         }
-        int n = (n_skip != nullptr && have && sl == 0) ? n_skip[(size_t)b * N_sel + i] : 0;
+        int n = (n_skip != nullptr && have && sl == 0) ? __ldcg(n_skip + (size_t)b * N_sel + i) : 0;
 
         float acc0 = 0.f, acc1 = 0.f;
         for (int v = sl; have && v < vec_per_row; v += LPR * kUnroll) {
@@ -111,7 +105,7 @@ score_kernel(const uint4 *__restrict__ x_cur, const uint4 *__restrict__ x_ref,
             for (int u = 0; u < kLsePre; ++u)
                 if (sl + LPR * u < H) ls += (lse_mode == ASTRAEA_LSE_SUM_EXP) ? expf(fminf(lv[u], (float)ASTRAEA_LSE_CLAMP)) : lv[u];
             for (int h = sl + LPR * kLsePre; h < H; h += LPR) {          // more than 2 * LPR heads: the rest afterwards
-                float l = __ldg(lse + ((size_t)b * H + h) * N + i);
+                float l = __ldcg(lse + ((size_t)b * H + h) * N + i);
                 ls += (lse_mode == ASTRAEA_LSE_SUM_EXP) ? expf(fminf(l, (float)ASTRAEA_LSE_CLAMP)) : l;
             }
         }
@@ -138,9 +132,9 @@ void launch_mode(int lpr, int grid, cudaStream_t stream, const uint4 *xc, const 
                  float *score, int B, int N, int N_sel, int D, int H, float w_alpha, float w_beta, int lse_mode, float *part)
 {
     dim3 block(kWarpsPerBlock * 32);
-    if (lpr == 32) score_kernel<MODE, 32><<<grid, block, 0, stream>>>(xc, xr, lse, n_skip, score, B, N, N_sel, D, H, w_alpha, w_beta, lse_mode, part);
-    else if (lpr == 16) score_kernel<MODE, 16><<<grid, block, 0, stream>>>(xc, xr, lse, n_skip, score, B, N, N_sel, D, H, w_alpha, w_beta, lse_mode, part);
-    else score_kernel<MODE, 8><<<grid, block, 0, stream>>>(xc, xr, lse, n_skip, score, B, N, N_sel, D, H, w_alpha, w_beta, lse_mode, part);
+    if (lpr == 32) launch_overlapped(score_kernel<MODE, 32>, grid, block, 0, stream, xc, xr, lse, n_skip, score, B, N, N_sel, D, H, w_alpha, w_beta, lse_mode, part);
+    else if (lpr == 16) launch_overlapped(score_kernel<MODE, 16>, grid, block, 0, stream, xc, xr, lse, n_skip, score, B, N, N_sel, D, H, w_alpha, w_beta, lse_mode, part);
+    else launch_overlapped(score_kernel<MODE, 8>, grid, block, 0, stream, xc, xr, lse, n_skip, score, B, N, N_sel, D, H, w_alpha, w_beta, lse_mode, part);
 }
 
 // score[b, i] = w_alpha * (sum of exp(lse) / H) * (sum of differences / D) + w_beta * e^n from the summed partial sums
@@ -148,10 +142,12 @@ __global__ void __launch_bounds__(256)
 score_combine_kernel(const float *__restrict__ part, const int32_t *__restrict__ n_skip, float *__restrict__ score,
                      long long total, float inv_D, float inv_H, int has_lse, float w_alpha, float w_beta)
 {
+    grid_launch_dependents();
+    grid_dependency_wait();
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
-        const float delta = part[t] * inv_D;
-        const float s_lse = has_lse ? part[total + t] * inv_H : 1.0f;
-        int n = n_skip ? n_skip[t] : 0;
+        const float delta = __ldcg(part + t) * inv_D;
+        const float s_lse = has_lse ? __ldcg(part + total + t) * inv_H : 1.0f;
+        int n = n_skip ? __ldcg(n_skip + t) : 0;
         n = min(n, ASTRAEA_N_SKIP_CLAMP);
         score[t] = w_alpha * (s_lse * delta) + w_beta * expf((float)n);
     }
@@ -165,7 +161,7 @@ int32_t launch_score_combine(const float *part, const int32_t *n_skip, float *sc
     const long long total = (long long)B * N_sel;
     if (total == 0) return ASTRAEA_OK;
     const long long want = (total + 255) / 256, cap = (long long)sm_count() * 8;
-    score_combine_kernel<<<(int)(want < cap ? want : cap), 256, 0, stream>>>(part, n_skip, score, total, 1.0f / (float)D, 1.0f / (float)H,
+    launch_overlapped(score_combine_kernel, (int)(want < cap ? want : cap), 256, 0, stream, part, n_skip, score, total, 1.0f / (float)D, 1.0f / (float)H,
                                                                              has_lse, w_alpha, w_beta);
     return check_launch("astraea_score_combine");
 }

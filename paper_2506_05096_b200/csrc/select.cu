@@ -43,6 +43,8 @@ select_kernel(const float *__restrict__ score, int N_sel, int k, int n_always,
     __shared__ uint32_t hist[256];
     __shared__ uint32_t warp_tot[32];
     __shared__ uint32_t s_prefix, s_kk, s_chunk_tot;
+    grid_launch_dependents();
+    grid_dependency_wait();
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x;
@@ -64,7 +66,7 @@ select_kernel(const float *__restrict__ score, int N_sel, int k, int n_always,
                 bool live = false;
                 uint32_t bin = 0;
                 if (i < N_sel) {
-                    uint32_t key = score_key(s[i]);
+                    uint32_t key = score_key(__ldcg(s + i));
                     live = (key & mask) == prefix;
                     bin = (key >> shift) & 255u;
                 }
@@ -119,7 +121,7 @@ select_kernel(const float *__restrict__ score, int N_sel, int k, int n_always,
 #pragma unroll
         for (int u = 0; u < kItems; ++u) {
             int i = base + u;
-            uint32_t key = (i < N_sel) ? score_key(s[i]) : 0u;
+            uint32_t key = (i < N_sel) ? score_key(__ldcg(s + i)) : 0u;
             gt[u] = (i < N_sel) && (key > T);
             eq[u] = (i < N_sel) && (key == T);
             tg += gt[u];
@@ -168,11 +170,6 @@ select_kernel(const float *__restrict__ score, int N_sel, int k, int n_always,
     for (int t = tid; t < n_always; t += kThreads) sel[k + t] = N_sel + t;
 }
 
-
-// programmatic dependent launch: wait for the kernel before this one in the stream (all of its memory operations
-// are then visible); let the kernel after this one start its own prologue
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------------- cluster version (keys in registers)
 constexpr int kMaxCluster = 8;
@@ -243,10 +240,10 @@ select_cluster_kernel(const float *__restrict__ score, int N_sel, int k, int n_a
         for (int u = 0; u < ITEMS; u += kVec) {
             float f[kVec];
             if constexpr (kVec == 4) {
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(s + base + u));
+                const float4 v = __ldcg(reinterpret_cast<const float4 *>(s + base + u));
                 f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
             } else {
-                const float2 v = __ldg(reinterpret_cast<const float2 *>(s + base + u));
+                const float2 v = __ldcg(reinterpret_cast<const float2 *>(s + base + u));
                 f[0] = v.x; f[1] = v.y;
             }
 #pragma unroll
@@ -254,7 +251,7 @@ select_cluster_kernel(const float *__restrict__ score, int N_sel, int k, int n_a
         }
     } else {
 #pragma unroll
-        for (int u = 0; u < ITEMS; ++u) key[u] = (base + u < N_sel) ? score_key(__ldg(s + base + u)) : 0u;
+        for (int u = 0; u < ITEMS; ++u) key[u] = (base + u < N_sel) ? score_key(__ldcg(s + base + u)) : 0u;
     }
     if constexpr (kPrefetchCounters) {
         if (vec_n) {
@@ -498,7 +495,7 @@ int32_t launch_select(const float *score, int B, int N_sel, int k, int n_always,
         return launch_cluster<8>(score, B, N_sel, k, n_always, idx_sel, idx_rem, n_skip, stream);
     if (N_sel > 0 && N_sel <= 16 * kThreads * kMaxCluster)
         return launch_cluster<16>(score, B, N_sel, k, n_always, idx_sel, idx_rem, n_skip, stream);
-    select_kernel<<<B, kThreads, 0, stream>>>(score, N_sel, k, n_always, idx_sel, idx_rem, n_skip);
+    launch_overlapped(select_kernel, B, kThreads, 0, stream, score, N_sel, k, n_always, idx_sel, idx_rem, n_skip);
     return check_launch("astraea_select");
 }
 
