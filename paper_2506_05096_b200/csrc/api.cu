@@ -316,13 +316,13 @@ int32_t astraea_layernorm_modulate(const void *x, const int32_t *idx, int M, con
 }
 
 // ------------------------------------------------------------------ a whole compute block
-// workspace: [256 bytes: error word | gathered keys and values of the SelectQ&K variant, or the key shares of a split
-//             self-attention launch] [select scratch]
+// workspace: [256 bytes: error word | the key shares of a split self-attention launch (room for gathered keys and values
+//             too)] [select scratch]
 //            [5 token-sized buffers] [hidden-sized buffer]
 // (the first part is laid out as the workspace of astraea_sparse_attn with kv_idx, so that every call of the block
 // shares the one error word at the very start)
 static size_t block_buffer_bytes(int B, int N, int width) { return align_up((size_t)B * N * width * 2, 256); }
-// the head of the block's workspace serves the self-attention: gathered keys / values (SelectQ&K) or the key shares of a split launch
+// the head of the block's workspace serves the self-attention: the key shares of a split launch
 static size_t block_attn_region_bytes(int B, int H, int N, int d)
 {
     const size_t kv = attn_kv_workspace_bytes(B, H, N, d), plain = attn_workspace_bytes(B, H, N, N, d);
@@ -379,17 +379,20 @@ int32_t astraea_block_step(const void *x, const astraea_block_weights *w, const 
     const int64_t tsb = (int64_t)N_text * D;
     // self-attention group: keys / values from all tokens, everything else on the selected rows
     rc = astraea_layernorm_modulate(x, nullptr, 0, w->s1, w->t1, bufA, B, N, D, eps, 0u, err, stream);
-    // (SelectQ&K: keys and values of the selected tokens only, so only their rows are projected)
+    // (SelectQ&K: keys and values of the selected tokens only, so only their rows are projected, into compact buffers)
     const int32_t *kv_rows = select_qk ? idx_sel : nullptr;
-    if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, kv_rows, M, w->wk, w->bk, bufK, B, N, D, D, 0u, err, 256, stream);
-    if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, kv_rows, M, w->wv, w->bv, bufV, B, N, D, D, 0u, err, 256, stream);
+    const uint32_t kv_flags = select_qk ? ASTRAEA_LINEAR_COMPACT_OUT : 0u;
+    if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, kv_rows, M, w->wk, w->bk, bufK, B, N, D, D, kv_flags, err, 256, stream);
+    if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, kv_rows, M, w->wv, w->bv, bufV, B, N, D, D, kv_flags, err, 256, stream);
     if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, idx_sel, M, w->wq, w->bq, bufQ, B, N, D, D, 0u, err, 256, stream);
     if (rc == ASTRAEA_OK && !select_qk)
         rc = astraea_sparse_attn(bufQ, bufK, bufV, sb, sh, sn, sb, sh, sn, sb, sh, sn, idx_sel, M, nullptr, 0, bufO, st->lse_cache,
                                  B, H, N, d, 0.f, 0u, ws, block_attn_region_bytes(B, H, N, d), stream);
-    if (rc == ASTRAEA_OK && select_qk)       // the listed key / value rows are gathered into the head of the workspace
-        rc = astraea_sparse_attn(bufQ, bufK, bufV, sb, sh, sn, sb, sh, sn, sb, sh, sn, idx_sel, M, idx_sel, M, bufO, st->lse_cache,
-                                 B, H, N, d, 0.f, 0u, ws, attn_kv_workspace_bytes(B, H, N, d), stream);
+    if (rc == ASTRAEA_OK && select_qk) {     // the compact keys / values are a sequence of M tokens
+        const int64_t csb = (int64_t)M * D;
+        rc = sparse_attn_entry("astraea_block_step", M, bufQ, bufK, bufV, sb, sh, sn, csb, sh, sn, csb, sh, sn, idx_sel, M, nullptr, 0, bufO, st->lse_cache,
+                               B, H, N, d, 0.f, 0u, ws, block_attn_region_bytes(B, H, N, d), stream);
+    }
     // x1 (compact, over the dead keys) = x[I] + g1 * (attention rows Wo^T + bo)
     if (rc == ASTRAEA_OK)
         rc = astraea_gathered_linear_residual(bufO, idx_sel, M, w->wo, w->bo, x, w->g1, bufK, B, N, D, D, ASTRAEA_LINEAR_COMPACT_OUT, err, 256, stream);
