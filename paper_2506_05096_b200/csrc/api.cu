@@ -138,6 +138,14 @@ int32_t astraea_select(const float *score, int B, int N_sel, int k, int n_always
     return launch_select(score, B, N_sel, k, n_always, idx_sel, idx_rem, n_skip, workspace, (cudaStream_t)stream);
 }
 
+// whether the refresh of the reference inputs may run beside the attention: its rows must not be among what that reads or
+// writes (callers whose buffers overlap get the copy behind the attention, in the order of the calls)
+static bool disjoint(const void *a, size_t a_bytes, const void *b, size_t b_bytes)
+{
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x + a_bytes <= y || y + b_bytes <= x;
+}
+
 static int32_t sparse_attn_entry(const char *fn, int N_kv, const void *q, const void *k, const void *v,
                             int64_t q_sb, int64_t q_sh, int64_t q_sn,
                             int64_t k_sb, int64_t k_sh, int64_t k_sn,
@@ -145,7 +153,8 @@ static int32_t sparse_attn_entry(const char *fn, int N_kv, const void *q, const 
                             const int32_t *q_idx, int M, const int32_t *kv_idx, int M_kv,
                             void *out, float *lse_out,
                             int B, int H, int N, int d, float scale, uint32_t flags,
-                            void *workspace, size_t workspace_bytes, void *stream)
+                            void *workspace, size_t workspace_bytes, void *stream,
+                            const void *copy_src = nullptr, void *copy_dst = nullptr)      // rows q_idx of [B, N, H*d], see AttnArgs
 {
     REQUIRE(B > 0 && H > 0 && N > 0 && d > 0 && N_kv >= 0, "%s: B, H, N, d must be positive", fn);
     REQUIRE(!kv_idx || (M_kv > 0 && M_kv <= N), "%s: M_kv=%d outside [1, N=%d]", fn, M_kv, N);
@@ -180,6 +189,7 @@ static int32_t sparse_attn_entry(const char *fn, int N_kv, const void *q, const 
     a.err_word = reinterpret_cast<int *>(workspace);
     a.N_tok = N;
     if (N_kv > 0) a.N = N_kv;          // keys and values of another sequence: N stays the token count of q / out
+    a.copy_src = copy_src; a.copy_dst = copy_dst; a.copy_elems = H * d;
     if (kv_idx) return launch_sparse_attn_kv(a, kv_idx, M_kv, workspace, (cudaStream_t)stream);
     if (workspace_bytes > 256) { a.split_ws = static_cast<char *>(workspace) + 256; a.split_ws_bytes = workspace_bytes - 256; }
     return launch_sparse_attn(a, (cudaStream_t)stream);
@@ -385,14 +395,18 @@ int32_t astraea_block_step(const void *x, const astraea_block_weights *w, const 
     if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, kv_rows, M, w->wk, w->bk, bufK, B, N, D, D, kv_flags, err, 256, stream);
     if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, kv_rows, M, w->wv, w->bv, bufV, B, N, D, D, kv_flags, err, 256, stream);
     if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, idx_sel, M, w->wq, w->bq, bufQ, B, N, D, D, 0u, err, 256, stream);
-    if (rc == ASTRAEA_OK && !select_qk)
-        rc = astraea_sparse_attn(bufQ, bufK, bufV, sb, sh, sn, sb, sh, sn, sb, sh, sn, idx_sel, M, nullptr, 0, bufO, st->lse_cache,
-                                 B, H, N, d, 0.f, 0u, ws, block_attn_region_bytes(B, H, N, d), stream);
-    if (rc == ASTRAEA_OK && select_qk) {     // the compact keys / values are a sequence of M tokens
-        const int64_t csb = (int64_t)M * D;
-        rc = sparse_attn_entry("astraea_block_step", M, bufQ, bufK, bufV, sb, sh, sn, csb, sh, sn, csb, sh, sn, idx_sel, M, nullptr, 0, bufO, st->lse_cache,
-                               B, H, N, d, 0.f, 0u, ws, block_attn_region_bytes(B, H, N, d), stream);
-    }
+    // the reference inputs of the tokens that were computed become the current inputs, under the attention where they can
+    const size_t xb = (size_t)B * N * D * 2, lb = (size_t)B * H * N * 4, txb = (size_t)B * N_text * D * 2;
+    const bool refresh = !(flags & ASTRAEA_BLOCK_REUSE_SELECTION);
+    const bool beside = refresh && disjoint(st->x_ref, xb, x, xb) && disjoint(st->x_ref, xb, st->y_cache, xb) && disjoint(x, xb, st->y_cache, xb) &&
+                        disjoint(st->x_ref, xb, st->lse_cache, lb) && disjoint(x, xb, st->lse_cache, lb) &&
+                        disjoint(st->x_ref, xb, text_k, txb) && disjoint(st->x_ref, xb, text_v, txb) && disjoint(st->x_ref, xb, workspace, workspace_bytes);
+    // (SelectQ&K: the compact keys / values are a sequence of M tokens)
+    const int64_t kvb = select_qk ? (int64_t)M * D : sb;
+    if (rc == ASTRAEA_OK)
+        rc = sparse_attn_entry("astraea_block_step", select_qk ? M : 0, bufQ, bufK, bufV, sb, sh, sn, kvb, sh, sn, kvb, sh, sn, idx_sel, M, nullptr, 0,
+                               bufO, st->lse_cache, B, H, N, d, 0.f, 0u, ws, block_attn_region_bytes(B, H, N, d), stream,
+                               beside ? x : nullptr, beside ? st->x_ref : nullptr);
     // x1 (compact, over the dead keys) = x[I] + g1 * (attention rows Wo^T + bo)
     if (rc == ASTRAEA_OK)
         rc = astraea_gathered_linear_residual(bufO, idx_sel, M, w->wo, w->bo, x, w->g1, bufK, B, N, D, D, ASTRAEA_LINEAR_COMPACT_OUT, err, 256, stream);
@@ -415,8 +429,7 @@ int32_t astraea_block_step(const void *x, const astraea_block_weights *w, const 
     if (rc == ASTRAEA_OK)
         rc = astraea_gathered_linear_residual(bufU, idx_sel, M, w->w2, w->b2, bufO, w->g3, st->y_cache, B, N, hidden, D,
                                               ASTRAEA_LINEAR_COMPACT_IN | ASTRAEA_LINEAR_COMPACT_RES, err, 256, stream);
-    // the reference inputs of the tokens that were computed become the current inputs
-    if (rc == ASTRAEA_OK && !(flags & ASTRAEA_BLOCK_REUSE_SELECTION))
+    if (rc == ASTRAEA_OK && refresh && !beside)
         rc = astraea_scatter_reuse(st->x_ref, x, idx_sel, B, N, M, D, ASTRAEA_SCATTER_SRC_FULL, err, stream);
     return rc;
 }
@@ -446,10 +459,15 @@ int32_t astraea_step(const void *x_cur, void *x_ref, float *lse_cache, int32_t *
                         workspace_bytes - attn_ws, stream);
     if (rc != ASTRAEA_OK) return rc;
     const int64_t sb = (int64_t)N * D, sh = d, sn = D;
-    rc = astraea_sparse_attn(q, k, v, sb, sh, sn, sb, sh, sn, sb, sh, sn, idx_sel, M, nullptr, 0, out_cache,
-                             lse_cache, B, H, N, d, 0.f, 0u, ws, attn_ws, stream);
-    if (rc != ASTRAEA_OK) return rc;
-    // the reference inputs of the tokens that were computed become the current inputs
+    // the reference inputs of the tokens that were computed become the current inputs, under the attention where they can
+    const size_t tb = (size_t)B * N * D * 2, lb = (size_t)B * H * N * 4;
+    const bool beside = M > 0 && x_ref && x_cur && aligned16(x_ref) && aligned16(x_cur) && disjoint(x_ref, tb, x_cur, tb) &&
+                        disjoint(x_ref, tb, q, tb) && disjoint(x_ref, tb, k, tb) && disjoint(x_ref, tb, v, tb) &&
+                        disjoint(x_ref, tb, out_cache, tb) && disjoint(x_ref, tb, lse_cache, lb) &&
+                        disjoint(x_cur, tb, out_cache, tb) && disjoint(x_cur, tb, lse_cache, lb);
+    rc = sparse_attn_entry("astraea_step", 0, q, k, v, sb, sh, sn, sb, sh, sn, sb, sh, sn, idx_sel, M, nullptr, 0, out_cache,
+                           lse_cache, B, H, N, d, 0.f, 0u, ws, attn_ws, stream, beside ? x_cur : nullptr, beside ? x_ref : nullptr);
+    if (rc != ASTRAEA_OK || beside) return rc;
     return astraea_scatter_reuse(x_ref, x_cur, idx_sel, B, N, M, D, ASTRAEA_SCATTER_SRC_FULL, ws, stream);
 }
 

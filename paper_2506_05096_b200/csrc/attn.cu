@@ -12,7 +12,8 @@
 //   one warp   TMA producer: K and V tiles into multi-stage swizzled buffers;
 //   two warps  tcgen05.mma issuers, one per query tile: S = Q K^T (SS, K-major operands), O += P V (P from
 //              TMEM, V as an MN-major shared-memory operand); the first owns the TMEM allocation;
-//   one warp   only donates registers (setmaxnreg moves registers to the softmax warps).
+//   one warp   donates registers (setmaxnreg moves registers to the softmax warps) and, when the caller has rows to copy at
+//              the same indices (the reference inputs of a step), moves them by bulk copies through shared memory.
 //
 // Two softmax warpgroups per query tile put four softmax warps on every SM sub-partition, which hides the
 // serial chain of a key tile (wait, load, exponentials, sum, pack, publish).  Even key tiles go to one
@@ -121,8 +122,11 @@ template <int DH, int TM> struct Cfg {
     static constexpr int kStagesV = (kCtasPerSM == 2) ? 4 : (DH == 128) ? 4 : 6;
     static_assert(kStagesK > kAhead, "K runs kAhead tiles ahead");
     static constexpr int kBarBytes = 512;
+    static constexpr int kCopyStages = (kCtasPerSM == 2) ? 2 : 3, kCopyStageBytes = 4096;   // rows on their way through the copying warp
+    static constexpr int kCopyBytes = kCopyStages * kCopyStageBytes;
     static constexpr int kOnesBytes = kOnes ? kBlockN * 128 : 0; // a key tile x one 64-column chunk of bf16: ones in column 0
-    static constexpr int kSmemBytes = kQTileBytes * kTilesM + kTileBytes * (kStagesK + kStagesV) + kOnesBytes + kBarBytes + 1024;
+    static constexpr int kSmemBytes = kQTileBytes * kTilesM + kTileBytes * (kStagesK + kStagesV) + kOnesBytes + kCopyBytes + kBarBytes + 1024;
+    static_assert(kSmemBytes + TM * 2080 + 64 + 1024 <= 228 * 1024 / kCtasPerSM, "shared memory with the static part and the 1 KB a CTA reserves");
 };
 
 struct Params {
@@ -143,6 +147,10 @@ struct Params {
     // evenly: each writes normalised fp32 rows and their LSE to part_o / part_lse, which merge_parts_kernel combines.
     int tiles_x, heads;
     int n_full, split;
+    const uint4 *copy_src;       // rows q_idx of copy_src go to copy_dst (NULL: none), copy_bytes each
+    uint4 *copy_dst;
+    uint32_t copy_bytes;
+    int copy_rows;               // B * M
     float *part_o, *part_lse;    // [part][kTilesM * 128 rows][head_dim] and [part][kTilesM * 128 rows]
 };
 
@@ -626,6 +634,59 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
     }
 }
 
+// ---------------------------------------------------------------- copying warp
+// This CTA's even share of the listed rows goes from copy_src to copy_dst by bulk copies, through kCopyStages stages: the
+// load of a batch is sent kCopyStages - 1 batches before its store.  A batch is as many rows as fit a stage, a lane each, or a
+// piece of one row.  The standalone scatter is one more launch and a pass at memory speed in which the tensor cores idle;
+// here the bytes move under the key loop (a batch takes ~1.5 us, a CTA has 5-30 of them in 30-900 us).
+template <class C>
+__device__ __forceinline__ void copy_role(const Params &p, uint32_t s_copy, uint32_t bar, volatile int *abort_flag)
+{
+    constexpr int kS = C::kCopyStages;
+    const int lane = threadIdx.x & 31;
+    const int r0 = (int)((long long)p.copy_rows * blockIdx.x / gridDim.x), r1 = (int)((long long)p.copy_rows * (blockIdx.x + 1) / gridDim.x);
+    const int parts = (int)((p.copy_bytes + C::kCopyStageBytes - 1) / C::kCopyStageBytes);       // pieces of a row
+    const int rows = parts > 1 ? 1 : min(32, (int)(C::kCopyStageBytes / p.copy_bytes));            // rows of a batch
+    const int batches = parts > 1 ? (r1 - r0) * parts : (r1 - r0 + rows - 1) / rows;
+    // 16-byte units ahead of this lane's piece of batch i in both tensors; -1: none, or a bad entry (reported by the softmax warps)
+    auto piece = [&](int i) -> int {
+        const int r = parts > 1 ? r0 + i / parts : r0 + i * rows + lane;
+        if (i >= batches || lane >= rows || r >= r1) return -1;
+        const int b = r / p.M, m = r - b * p.M;
+        const int tok = __ldcg(p.q_idx + r), before = m > 0 ? __ldcg(p.q_idx + r - 1) : -1;
+        if ((unsigned)tok >= (unsigned)p.N_tok || before >= tok) return -1;
+        return (b * p.N_tok + tok) * (int)(p.copy_bytes >> 4) + (parts > 1 ? (i % parts) * (C::kCopyStageBytes / 16) : 0);
+    };
+    auto bytes = [&](int i) -> uint32_t {
+        return parts > 1 ? min((uint32_t)C::kCopyStageBytes, p.copy_bytes - (uint32_t)(i % parts) * C::kCopyStageBytes) : p.copy_bytes;
+    };
+    const uint32_t slot = lane * (rows > 1 ? p.copy_bytes : 0u);
+    int off[kS], next = piece(0);                 // off[u]: batch i - u
+#pragma unroll
+    for (int u = 0; u < kS; ++u) off[u] = -1;
+    for (int i = 0; i < batches + kS - 1; ++i) {
+#pragma unroll
+        for (int u = kS - 1; u > 0; --u) off[u] = off[u - 1];
+        off[0] = next;
+        next = piece(i + 1);
+        const int j = i - (kS - 1);
+        if (j >= 0) {
+            wait_bar(bar + 8 * (j % kS), (j / kS) & 1, abort_flag, p.err_word);
+            if (*abort_flag) break;
+            if (off[kS - 1] >= 0) bulk_store(p.copy_dst + off[kS - 1], s_copy + (j % kS) * C::kCopyStageBytes + slot, bytes(j));
+        }
+        bulk_commit();
+        if (i < batches) {
+            bulk_wait_read<1>();                        // the stage's last batch (stored one round ago) has left it
+            const uint32_t n = __popc(__ballot_sync(0xffffffffu, off[0] >= 0));
+            if (lane == 0) mbar_arrive_expect_tx(bar + 8 * (i % kS), n * bytes(i));
+            __syncwarp();
+            if (off[0] >= 0) bulk_load(s_copy + (i % kS) * C::kCopyStageBytes + slot, p.copy_src + off[0], bytes(i), bar + 8 * (i % kS));
+        }
+    }
+    bulk_wait<0>();
+}
+
 template <class C>
 __global__ void __launch_bounds__(C::kThreads, C::kCtasPerSM)
 sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v,
@@ -646,14 +707,16 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     const uint32_t sK = sQ + kTilesM * C::kQTileBytes;
     const uint32_t sV = sK + C::kStagesK * C::kTileBytes;
     const uint32_t sOnes = sV + C::kStagesV * C::kTileBytes;       // [key tile x 64 columns] bf16, 128-byte swizzle, column 0 = 1
-    const uint32_t bars = sOnes + C::kOnesBytes;
+    const uint32_t sCopy = sOnes + C::kOnesBytes;
+    const uint32_t bars = sCopy + C::kCopyBytes;
     Bars bar;
     bar.q = bars; bar.s = bars + 16; bar.p = bars + 80; bar.done = bars + 144;
     bar.kf = bars + 160;
     bar.ke = bar.kf + 8 * C::kStagesK;
     bar.vf = bar.ke + 8 * C::kStagesK;
     bar.ve = bar.vf + 8 * C::kStagesV;
-    static_assert(160 + 16 * (C::kStagesK + C::kStagesV) <= C::kBarBytes, "barrier area too small");
+    const uint32_t bar_copy = bar.ve + 8 * C::kStagesV;
+    static_assert(160 + 16 * (C::kStagesK + C::kStagesV) + 8 * C::kCopyStages <= C::kBarBytes, "barrier area too small");
 
     const int tid = threadIdx.x;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);        // warp-uniform
@@ -691,6 +754,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
             mbar_init(bar.done + 8 * t, 1);
             for (int u = 0; u < 4; ++u) { mbar_init(bar.s + 32 * t + 8 * u, 1); mbar_init(bar.p + 32 * t + 8 * u, 128); }
         }
+        for (int u = 0; u < C::kCopyStages; ++u) mbar_init(bar_copy + 8 * u, 1);
         fence_barrier_init();
     }
     constexpr int kProducerWarp = C::kSoftmaxWarps, kIssuerWarp = C::kSoftmaxWarps + 1;
@@ -883,6 +947,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
         }
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
+        if (p.copy_dst) copy_role<C>(p, sCopy, bar_copy, &abort_flag);
+        __syncwarp();
         pass_sync<C>();
     }
 
@@ -1031,12 +1097,25 @@ int32_t launch_dh(const AttnArgs &a, cudaStream_t stream, SplitPlan plan = Split
         p.part_o = p.part_lse + (rows + 63) / 64 * 64;
     }
     const unsigned grid = (unsigned)(p.n_full + (split ? plan.units * plan.split : 0));
+    // The rows to copy go with the attention when its CTAs live long enough for their shares: 4 KB a microsecond against
+    // 0.4 us a key tile and 4 us for a CTA's set-up and a launch less.  (Measured: a batch of 4 KB takes ~1.5 us with two or
+    // three of them in flight.)
+    const long long copy_rows = (long long)a.B * a.M;
+    const double copy_us = a.copy_dst ? (double)((copy_rows + grid - 1) / grid) * a.copy_elems * 2 / 4096 : 0.0;
+    const bool copy_here = a.copy_dst && (long long)a.B * a.N_tok * (a.copy_elems / 8) < 0x7fffffffll && copy_us <= 0.4 * ((a.N + C::kBlockN - 1) / C::kBlockN) / p.split + 4.0;
+    p.copy_src = copy_here ? reinterpret_cast<const uint4 *>(a.copy_src) : nullptr;
+    p.copy_dst = copy_here ? reinterpret_cast<uint4 *>(a.copy_dst) : nullptr;
+    p.copy_bytes = (uint32_t)a.copy_elems * 2;
+    p.copy_rows = copy_here ? (int)copy_rows : 0;
     launch_overlapped(sparse_attn_kernel<C>, grid, C::kThreads, C::kSmemBytes, stream, mk, mv, mkt, mvt, p);
     if (split) {
         static_assert((TM * kBlockM * (DH / 8)) % (TM * kBlockM) == 0, "whole blocks per unit");
         launch_overlapped(merge_parts_kernel<DH, TM * kBlockM>, dim3(DH / 8, plan.units), TM * kBlockM, 0, stream, p);
     }
-    return check_launch("astraea_sparse_attn");
+    rc = check_launch("astraea_sparse_attn");
+    if (rc == ASTRAEA_OK && a.copy_dst && !copy_here)
+        rc = launch_scatter(a.copy_dst, a.copy_src, a.q_idx, a.B, a.N_tok, a.M, a.copy_elems, ASTRAEA_SCATTER_SRC_FULL, a.err_word, stream);
+    return rc;
 }
 
 }  // namespace

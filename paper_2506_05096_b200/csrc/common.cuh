@@ -118,6 +118,12 @@ struct AttnArgs {
     // launches that may run at the same time must not share it.
     void *split_ws = nullptr;
     size_t split_ws_bytes = 0;
+    // rows q_idx of copy_src [B, N_tok, copy_elems] go to the same rows of copy_dst, in the attention kernel itself or by a
+    // scatter behind it (NULL: no copy).  Nothing that the attention reads or writes may overlap copy_dst, nor its outputs
+    // copy_src; copy_elems is a multiple of 8, both are 16-byte aligned, q_idx is given and all heads are in the launch.
+    const void *copy_src = nullptr;
+    void *copy_dst = nullptr;
+    int copy_elems = 0;
 };
 int32_t launch_sparse_attn(const AttnArgs &a, cudaStream_t stream);
 // the schedule launch_sparse_attn would pick (host logic only; uses B, H / head_count, N, M, d, flags, split_ws, split_ws_bytes)

@@ -827,3 +827,42 @@ def test_cross_attention_of_selected_rows(oracle, d, N_kv):
     for b in range(B):
         mask[b, idx[b]] = False
     assert np.array_equal(got[mask], f64(cache)[mask])
+
+
+# ------------------------------------------------------------------ refresh of the reference inputs beside the attention
+@pytest.mark.parametrize("B,H,d,N_v,n_always,k", [
+    (1, 2, 64, 256, 0, 1),            # one row of 256 bytes: one lane of one batch
+    (2, 3, 72, 700, 5, 333),          # 432-byte rows, nine to a batch, both batch elements in one CTA's share
+    (1, 32, 64, 600, 0, 599),         # 4096-byte rows: a row is a batch
+    (1, 33, 64, 400, 7, 100),         # 4224 bytes: a whole piece and one of 128 bytes
+    (1, 24, 128, 2500, 0, 1200),      # 6144-byte rows, many CTAs
+    (1, 8, 128, 300, 0, 300),         # every row
+    (2, 16, 72, 40, 3, 0),            # always-kept rows only
+    (1, 40, 72, 64, 0, 60),           # one key tile, 5760-byte rows
+])
+def test_step_refreshes_reference_rows(B, H, d, N_v, n_always, k):
+    """astraea_step leaves x_ref bit-equal to x_cur in the selected rows and untouched elsewhere, whichever kernel copies."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N_v + k)
+    N, D, M = N_v + n_always, H * d, k + n_always
+    mk = lambda: torch.randn(B, N, D, device="cuda", dtype=torch.bfloat16, generator=g)  # noqa: E731
+    x, old, q, kk, v, out = (mk() for _ in range(6))
+    ref = Guarded((B, N, D), torch.bfloat16, init=old)
+    lse, ns = torch.zeros(B, H, N, device="cuda"), torch.zeros(B, N_v, dtype=torch.int32, device="cuda")
+    score, sel = torch.empty(B, N_v, device="cuda"), torch.empty(B, M, dtype=torch.int32, device="cuda")
+    rem = torch.empty(B, max(1, N_v - k), dtype=torch.int32, device="cuda")
+    ws = A.new_workspace(A.OP_STEP, B, H, N, M, d)
+    A.astraea_step(x, ref.t, lse, ns, q, kk, v, out, score, sel, rem, B, H, N, N_v, d, k, workspace=ws)
+    A.astraea_poll_error(ws)
+    ref.check("x_ref")
+    want = old.clone()
+    for b in range(B):
+        want[b, sel[b].long()] = x[b, sel[b].long()]
+    assert torch.equal(ref.t.view(torch.int16), want.view(torch.int16))
+    # a reference that shares its memory with the values is refreshed behind the attention, which still reads the old ones
+    shared, out2, out3 = old.clone(), out.clone(), out.clone()
+    lse2, lse3, ns2, ns3 = (torch.zeros_like(t) for t in (lse, lse, ns, ns))
+    A.astraea_step(x, shared, lse2, ns2, q, kk, shared, out2, score, sel, rem, B, H, N, N_v, d, k, workspace=ws)
+    A.astraea_step(x, old.clone(), lse3, ns3, q, kk, old, out3, score, sel, rem, B, H, N, N_v, d, k, workspace=ws)
+    assert torch.equal(shared.view(torch.int16), want.view(torch.int16))
+    assert torch.equal(out2.view(torch.int16), out3.view(torch.int16))
