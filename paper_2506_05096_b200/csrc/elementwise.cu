@@ -6,26 +6,37 @@
 // HBM-bound: every row is read once and written once.  One warp owns one row and keeps it packed in registers (16-byte
 // loads, all in flight at once), takes mean and variance from the registers in one pass over shifted data, then
 // normalises, modulates and stores in a second pass over the registers.  fp32 arithmetic, one rounding to bf16 at the end.
+// Next to the bytes the issue slots bind it: element by element it is ~105 instructions per 16-byte vector, so the
+// arithmetic is on packed fp32 pairs, and the register array has five and six vectors too, the widths of 1152 and 1536
+// channels (before -> after: 32768 x 1152 36.4 -> 29.1 us, 17776 x 3072 44.7 -> 40.6 = 5.4 TB/s, 4276 x 1536 7.8 -> 5.5).
+// Four warps a block rather than eight even out short launches and are worth 2-5 % of the long ones; two rows a warp,
+// sharing the unpacked modulation vectors, gain nothing.
 #include "common.cuh"
 
 namespace astraea {
 namespace {
 
-constexpr int kWarpsPerBlock = 8;
-constexpr int kBlocksPerSM = 8;
+constexpr int kWarpsPerBlock = 4;
+constexpr int kBlocksPerSM = 16;
 constexpr int kMaxVecPerLane = 16;     // rows of up to 32 * 16 * 8 = 4096 channels
 
-__device__ __forceinline__ void unpack8(const uint4 &v, float (&f)[8]) {
+// fp32 pairs: two elements of a row in one 64-bit register
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) { f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; }
+__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) { f32x2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { f32x2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+// eight bf16 as four fp32 pairs
+__device__ __forceinline__ void unpack8(const uint4 &v, f32x2 (&f)[4]) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) { f[2 * i] = __uint_as_float(w[i] << 16); f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
+    for (int i = 0; i < 4; ++i) f[i] = pack2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
 }
 
-// VPL: 16-byte vectors per lane (compile-time bound of the register array; vec_per_row <= 32 * VPL)
-// (two or three blocks per SM: the row stays packed in registers and is unpacked again in every pass, instead of being
-// kept as 8 * VPL floats, which would leave room for one block per SM only and too few bytes in flight)
+// VPL: 16-byte vectors per lane (vec_per_row <= 32 * VPL)
 template <int VPL>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, VPL <= 8 ? 3 : 2)
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, VPL <= 6 ? 8 : VPL <= 8 ? 6 : 4)
 layernorm_modulate_kernel(const uint4 *__restrict__ x, const int32_t *__restrict__ idx, int M, const uint4 *__restrict__ scale,
                           const uint4 *__restrict__ shift, uint4 *__restrict__ y, int B, int N, int vec_per_row, float eps,
                           int compact_in, int compact_out, int *__restrict__ err_word)
@@ -38,7 +49,8 @@ layernorm_modulate_kernel(const uint4 *__restrict__ x, const int32_t *__restrict
     for (long long t = (long long)blockIdx.x * kWarpsPerBlock + warp; t < total; t += (long long)gridDim.x * kWarpsPerBlock) {
         const int b = (int)(t / M), r = (int)(t - (long long)b * M);
         const int tok = idx ? __ldcg(idx + t) : r;
-        if ((unsigned)tok >= (unsigned)N || (idx && r > 0 && __ldcg(idx + t - 1) >= tok)) {      // see astraea_scatter_reuse
+        const int before = (idx && r > 0) ? __ldcg(idx + t - 1) : -1;
+        if ((unsigned)tok >= (unsigned)N || before >= tok) {                               // see astraea_scatter_reuse
             if (lane == 0 && err_word) atomicExch(err_word, kErrBadIndex);
             continue;
         }
@@ -50,45 +62,59 @@ layernorm_modulate_kernel(const uint4 *__restrict__ x, const int32_t *__restrict
         // mean and variance in one pass over the packed registers, on data shifted by the row's first element: the
         // shift takes the cancellation out of E[(x - x0)^2] - (E[x - x0])^2 whenever the mean is large against the spread
         const float x0 = __shfl_sync(0xffffffffu, __uint_as_float(v[0].x << 16), 0);
-        float s1 = 0.f, s2 = 0.f;
+        const f32x2 minus_x0 = pack2(-x0, -x0);
+        f32x2 a1 = 0ull, a2 = 0ull;
 #pragma unroll
         for (int u = 0; u < VPL; ++u) {
             if (lane + 32 * u < vec_per_row) {
-                float f[8];
+                f32x2 f[4];
                 unpack8(v[u], f);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) { const float c = f[i] - x0; s1 += c; s2 = fmaf(c, c, s2); }
+                for (int i = 0; i < 4; ++i) { const f32x2 c = add2(f[i], minus_x0); a1 = add2(a1, c); a2 = fma2(c, c, a2); }
             }
         }
+        float lo, hi;
+        unpack2(a1, lo, hi);
+        float s1 = lo + hi;
+        unpack2(a2, lo, hi);
+        float s2 = lo + hi;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }
         const float ms = s1 * inv_D, mean = x0 + ms;
         const float sq = fmaxf(s2 - s1 * ms, 0.f);                 // sum of squares about the mean
-        const float rstd = rsqrtf(sq * inv_D + eps);
+        const float rs = rsqrtf(sq * inv_D + eps);
+        const f32x2 minus_mean = pack2(-mean, -mean), rstd = pack2(rs, rs);
 #pragma unroll
         for (int u = 0; u < VPL; ++u) {
             const int c = lane + 32 * u;
             if (c < vec_per_row) {
-                float f[8], sc[8], sh[8];
+                f32x2 f[4], sc[4], sh[4];
                 unpack8(v[u], f);
                 if (scale) unpack8(__ldg(scale + (long long)b * vec_per_row + c), sc);
                 if (shift) unpack8(__ldg(shift + (long long)b * vec_per_row + c), sh);
                 uint32_t w[4];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    f[i] = (f[i] - mean) * rstd;
-                    if (scale) f[i] = fmaf(f[i], sc[i], f[i]);
-                    if (shift) f[i] += sh[i];
-                }
-#pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    __nv_bfloat162 v2 = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
+                    f[i] = mul2(add2(f[i], minus_mean), rstd);
+                    if (scale) f[i] = fma2(f[i], sc[i], f[i]);
+                    if (shift) f[i] = add2(f[i], sh[i]);
+                    unpack2(f[i], lo, hi);
+                    __nv_bfloat162 v2 = __floats2bfloat162_rn(lo, hi);
                     w[i] = *reinterpret_cast<uint32_t *>(&v2);
                 }
                 dst[c] = make_uint4(w[0], w[1], w[2], w[3]);
             }
         }
     }
+}
+
+template <int VPL>
+void launch_ln(cudaStream_t stream, const uint4 *x, const int32_t *idx, int M, const uint4 *scale, const uint4 *shift, uint4 *y, int B, int N,
+               int vec_per_row, float eps, int ci, int co, int *err_word)
+{
+    const long long want = ((long long)B * M + kWarpsPerBlock - 1) / kWarpsPerBlock, cap = (long long)sm_count() * kBlocksPerSM;
+    launch_overlapped(layernorm_modulate_kernel<VPL>, (int)(want < cap ? want : cap), kWarpsPerBlock * 32, 0, stream, x, idx, M, scale, shift, y, B, N,
+                      vec_per_row, eps, ci, co, err_word);
 }
 
 }  // namespace
@@ -102,21 +128,19 @@ int32_t launch_layernorm_modulate(const void *x, const int32_t *idx, int M, cons
     const int vec_per_row = D >> 3;
     if (vec_per_row > 32 * kMaxVecPerLane)
         return fail(ASTRAEA_ERR_UNSUPPORTED, "astraea_layernorm_modulate: D=%d above %d", D, 32 * kMaxVecPerLane * 8);
-    long long want = (total + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    const long long cap = (long long)sm_count() * kBlocksPerSM;
-    const int grid = (int)(want < cap ? want : cap);
     const uint4 *xs = reinterpret_cast<const uint4 *>(x), *sc = reinterpret_cast<const uint4 *>(scale), *sh = reinterpret_cast<const uint4 *>(shift);
     uint4 *ys = reinterpret_cast<uint4 *>(y);
     const int ci = (flags & ASTRAEA_LN_COMPACT_IN) ? 1 : 0, co = (flags & ASTRAEA_LN_COMPACT_OUT) ? 1 : 0;
-    dim3 block(kWarpsPerBlock * 32);
-    if (vec_per_row <= 32 * 4)
-        launch_overlapped(layernorm_modulate_kernel<4>, grid, block, 0, stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
-    else if (vec_per_row <= 32 * 8)
-        launch_overlapped(layernorm_modulate_kernel<8>, grid, block, 0, stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
-    else if (vec_per_row <= 32 * 12)
-        launch_overlapped(layernorm_modulate_kernel<12>, grid, block, 0, stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
-    else
-        launch_overlapped(layernorm_modulate_kernel<16>, grid, block, 0, stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word);
+    const int vpl = (vec_per_row + 31) / 32;
+#define LN(V) launch_ln<V>(stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word)
+    if (vpl <= 2) LN(2);
+    else if (vpl <= 4) LN(4);
+    else if (vpl <= 5) LN(5);
+    else if (vpl <= 6) LN(6);
+    else if (vpl <= 8) LN(8);
+    else if (vpl <= 12) LN(12);
+    else LN(16);
+#undef LN
     return check_launch("astraea_layernorm_modulate");
 }
 
