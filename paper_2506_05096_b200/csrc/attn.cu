@@ -75,7 +75,12 @@ template <int DH, int TM> struct Cfg {
     static constexpr int kTilesM = TM;
     static constexpr int kCtasPerSM = (TM == 1) ? 2 : 1;
     static constexpr uint32_t kTmemCols = 512 / kCtasPerSM;
-    static_assert(TM == 2 || DH != 128, "head_dim 128 needs the whole SM");
+    // One query tile at head_dim 64: the CTAs stay and walk over the units with a stride of the grid, so that launch, TMEM
+    // allocation and set-up are paid once per SM slot and the next unit's first K / V tiles are under way while its query
+    // rows are fetched.  Mostly launches over a few key tiles take this shape (cross-attention over the text tokens), where a unit
+    // is 8 us of which 1-2 are its key loop: 9001 queries x 226 keys x 48 heads 92 -> 83 us.  (At head_dim 72 the same loop
+    // spills and is 3 % slower; query rows fetched a unit ahead, in registers across the epilogue, spill: 103 us.)
+    static constexpr bool kPersistent = TM == 1 && DH == 64;
     // head_dim = kMain (whole 64-column, 128-byte-swizzled chunks) + kTail (8 columns at head_dim 72,
     // carried as a 16-column, 32-byte-swizzled chunk whose upper half is zero)
     static constexpr int kMain = DH / 64 * 64;
@@ -91,11 +96,12 @@ template <int DH, int TM> struct Cfg {
     static constexpr bool kOnes = DH == 64;
     static constexpr int kSBufs = 2;                              // S buffers per query tile: one per softmax warpgroup
     // Pairs of exponentials that are computed on the FMA pipe instead of the XU: three of eight at head_dim 64 and 128,
-    // one of four at 72 (us a launch, under the power cap: head_dim 64, 9001 x 17776 x 48 heads, 4 / 5 / 6 / 7 / 8 of 16:
+    // one of four at 72, one of eight in its small CTAs, whose registers do not hold more (62 against 58.5 us for 13106 x 226
+    // x 16; us a launch, under the power cap: head_dim 64, 9001 x 17776 x 48 heads, 4 / 5 / 6 / 7 / 8 of 16:
     // 2143 / 2123 / 2083 / 2140 / 2203; 72, 2 x 6553 x 16384 x 16, 2 / 4 / 5 / 6 / 8: 1190 / 1150 / 1152 / 1165 / 1233; 128,
     // 3276 x 65536 x 24, none / 5 / 6 / 7 / 8: 2250 / 2170 / 2130 / 2457 / 2400).  Degree 3 where the row sum or the sums of P
     // had that error already, 5 at head_dim 128, whose LSE keeps the precision it has with the XU alone.
-    static constexpr int kPolyPeriod = (DH == 72) ? 4 : 8;
+    static constexpr int kPolyPeriod = (DH == 72 && TM == 2) ? 4 : 8;
     static constexpr int kPolyPairs = (DH == 72) ? 1 : 3;
     static constexpr int kPolyDeg = (DH == 128) ? 5 : 3;
     static constexpr int kSoftmaxWarps = 4 * kTilesM * kSplit;
@@ -409,7 +415,7 @@ __device__ __forceinline__ void pass_sync() {
 // tile: its query tile; par: which key tiles it takes (j = par, par + kSplit, ...)
 template <class C>
 __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, int tile, int par, uint8_t *sQ_gen, uint32_t tmem,
-                                             int m_base, int h, int b, int n_tiles, int key0, int part,
+                                             int m_base, int h, int b, int n_tiles, int key0, int part, bool last_unit,
                                              volatile int *abort_flag, volatile int *redo_flag, float2 *xchg)
 {
     const int wtid = threadIdx.x & 127;
@@ -518,7 +524,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
     }
 
     // ------------------------------------------------ epilogue: normalise and scatter
-    grid_launch_dependents();
+    if (last_unit) grid_launch_dependents();
     tc_fence_after();
     // both warpgroups accumulated into one O against one reference: add the row sums, split the columns
     float l_sum = st.l_sum;                                      // with the ones column: the row's whole sum already
@@ -722,19 +728,20 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);        // warp-uniform
     constexpr int kBlockN = C::kBlockN;
     int unit = blockIdx.x, kpart = 0, ksplit = 1;
+    const int n_units = p.n_full;                                  // (persistent CTAs: all units)
     int part = -1;                                                 // >= 0: this CTA takes a share of the keys only
-    if (unit >= p.n_full) {
+    if (!C::kPersistent && unit >= p.n_full) {
         part = unit - p.n_full;
         kpart = part % p.split; ksplit = p.split;
         unit = p.n_full + part / p.split;
     }
-    const int m0 = (unit % p.tiles_x) * (kTilesM * kBlockM), h = p.h0 + (unit / p.tiles_x) % p.heads, b = unit / (p.tiles_x * p.heads);
+    int m0 = (unit % p.tiles_x) * (kTilesM * kBlockM), h = p.h0 + (unit / p.tiles_x) % p.heads, b = unit / (p.tiles_x * p.heads);
     const int n_tiles_all = (p.N + kBlockN - 1) / kBlockN;
     const int tile0 = n_tiles_all * kpart / ksplit;                // first key tile of this CTA (split <= 8: no overflow)
     const int n_tiles = n_tiles_all * (kpart + 1) / ksplit - tile0;
     const int key0 = tile0 * kBlockN;
     // the last CTA of a head may have rows in its first query tile only: the second tile's warps and MMAs are skipped
-    const int q_tiles = (m0 + kBlockM < p.M) ? kTilesM : 1;
+    const int q_tiles = (kTilesM > 1 && m0 + kBlockM < p.M) ? kTilesM : 1;
 
     if constexpr (C::kOnes) {
         // row r: 128 bytes; under the 128-byte swizzle the 16-byte unit that holds column 0 is unit r & 7
@@ -746,14 +753,17 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
         }
         fence_proxy_async_smem();
     }
-    if (tid == 0) {
-        abort_flag = 0;
-        redo_flag = 0;
+    auto init_query_bars = [&] {
         for (int t = 0; t < kTilesM; ++t) {
             mbar_init(bar.q + 8 * t, 128 * kSplit);
             mbar_init(bar.done + 8 * t, 1);
             for (int u = 0; u < 4; ++u) { mbar_init(bar.s + 32 * t + 8 * u, 1); mbar_init(bar.p + 32 * t + 8 * u, 128); }
         }
+    };
+    if (tid == 0) {
+        abort_flag = 0;
+        redo_flag = 0;
+        init_query_bars();
         for (int u = 0; u < C::kCopyStages; ++u) mbar_init(bar_copy + 8 * u, 1);
         fence_barrier_init();
     }
@@ -761,29 +771,35 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     // The producer warp sets up the K/V stage barriers itself and sends for the first kAhead K tiles and the first V
     // tile at once: their flight then runs under the TMEM allocation, the CTA-wide barrier and the gather of the Q rows
     // (nobody else touches these barriers or the stages before that barrier).
+    auto init_kv_bars = [&] {
+        // a K/V stage is free once the issuer of every active query tile has committed its MMAs on it
+        for (int s = 0; s < C::kStagesK; ++s) { mbar_init(bar.kf + 8 * s, 1); mbar_init(bar.ke + 8 * s, q_tiles); }
+        for (int s = 0; s < C::kStagesV; ++s) { mbar_init(bar.vf + 8 * s, 1); mbar_init(bar.ve + 8 * s, q_tiles); }
+        fence_barrier_init();
+    };
+    auto send_first_tiles = [&] {
+        for (int j = 0; j < kAhead && j < n_tiles; ++j) {
+            mbar_arrive_expect_tx(bar.kf + 8 * j, C::kLoadBytes);
+#pragma unroll
+            for (int ch = 0; ch < C::kChunks; ++ch)
+                tma_load_4d(sK + j * C::kTileBytes + ch * C::kChunkBytes, &tmap_k, bar.kf + 8 * j, ch * 64, key0 + j * kBlockN, h, b);
+            if (C::kTail)
+                tma_load_4d(sK + j * C::kTileBytes + C::kChunks * C::kChunkBytes, &tmap_k_tail, bar.kf + 8 * j, C::kMain, key0 + j * kBlockN, h, b);
+        }
+        mbar_arrive_expect_tx(bar.vf, C::kLoadBytes);
+#pragma unroll
+        for (int ch = 0; ch < C::kChunks; ++ch)
+            tma_load_4d(sV + ch * C::kChunkBytes, &tmap_v, bar.vf, ch * 64, key0, h, b);
+        if (C::kTail)
+            tma_load_4d(sV + C::kChunks * C::kChunkBytes, &tmap_v_tail, bar.vf, C::kMain, key0, h, b);
+    };
     if (warp == kProducerWarp) {
         if (elect_one()) {
             prefetch_tensormap(&tmap_k); prefetch_tensormap(&tmap_v);
             if (C::kTail) { prefetch_tensormap(&tmap_k_tail); prefetch_tensormap(&tmap_v_tail); }
-            // a K/V stage is free once the issuer of every active query tile has committed its MMAs on it
-            for (int s = 0; s < C::kStagesK; ++s) { mbar_init(bar.kf + 8 * s, 1); mbar_init(bar.ke + 8 * s, q_tiles); }
-            for (int s = 0; s < C::kStagesV; ++s) { mbar_init(bar.vf + 8 * s, 1); mbar_init(bar.ve + 8 * s, q_tiles); }
-            fence_barrier_init();
+            init_kv_bars();
             grid_dependency_wait();
-            for (int j = 0; j < kAhead && j < n_tiles; ++j) {
-                mbar_arrive_expect_tx(bar.kf + 8 * j, C::kLoadBytes);
-#pragma unroll
-                for (int ch = 0; ch < C::kChunks; ++ch)
-                    tma_load_4d(sK + j * C::kTileBytes + ch * C::kChunkBytes, &tmap_k, bar.kf + 8 * j, ch * 64, key0 + j * kBlockN, h, b);
-                if (C::kTail)
-                    tma_load_4d(sK + j * C::kTileBytes + C::kChunks * C::kChunkBytes, &tmap_k_tail, bar.kf + 8 * j, C::kMain, key0 + j * kBlockN, h, b);
-            }
-            mbar_arrive_expect_tx(bar.vf, C::kLoadBytes);
-#pragma unroll
-            for (int ch = 0; ch < C::kChunks; ++ch)
-                tma_load_4d(sV + ch * C::kChunkBytes, &tmap_v, bar.vf, ch * 64, key0, h, b);
-            if (C::kTail)
-                tma_load_4d(sV + C::kChunks * C::kChunkBytes, &tmap_v_tail, bar.vf, C::kMain, key0, h, b);
+            send_first_tiles();
         }
         __syncwarp();
     }
@@ -797,14 +813,49 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     const uint32_t tmem = tmem_slot;
     grid_dependency_wait();
 
+    // Persistent CTAs: on to the next unit, if there is one (called by every warp, from its role).  Between the two CTA-wide
+    // barriers nothing of the last unit is in flight (the producer has waited for its copies and for the issuers' last commits, the
+    // softmax warps for the last MMAs), so the mbarriers are set up afresh and every role counts from zero again.
+    auto next_unit = [&]() -> bool {
+        if constexpr (!C::kPersistent) return false;
+        unit += gridDim.x;
+        if (unit >= n_units) return false;
+        m0 = (unit % p.tiles_x) * (kTilesM * kBlockM); h = p.h0 + (unit / p.tiles_x) % p.heads; b = unit / (p.tiles_x * p.heads);
+        tc_fence_before();
+        __syncwarp();
+        asm volatile("bar.sync 0;" ::: "memory");
+        if (tid == 0) {
+            redo_flag = 0;
+            for (uint32_t a = bars; a < bar.kf; a += 8)
+                if (a < bar.q + 8 * kTilesM || (a >= bar.s && a < bar.s + 32 * kTilesM) || (a >= bar.p && a < bar.p + 32 * kTilesM) ||
+                    (a >= bar.done && a < bar.done + 8 * kTilesM)) mbar_inval(a);
+            init_query_bars();
+            fence_barrier_init();
+        }
+        __syncwarp();
+        if (warp == kProducerWarp) {
+            if (elect_one()) {
+                for (uint32_t a = bar.kf; a < bar_copy; a += 8) mbar_inval(a);
+                init_kv_bars();
+                send_first_tiles();
+            }
+            __syncwarp();
+        }
+        asm volatile("bar.sync 0;" ::: "memory");
+        tc_fence_after();
+        return true;
+    };
+
     if (warp < C::kSoftmaxWarps) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsSoftmax));
         const int wg = warp >> 2;
         const int tile = wg / kSplit, par = wg % kSplit;
-        if (tile < q_tiles)
-            softmax_role<C>(p, bar, tile, par, smem_gen + tile * C::kQTileBytes, tmem, m0 + tile * kBlockM, h, b, n_tiles, key0, part,
-                             &abort_flag, &redo_flag, xchg[tile]);
-        else pass_sync<C>();
+        do {
+            if (tile < q_tiles)
+                softmax_role<C>(p, bar, tile, par, smem_gen + tile * C::kQTileBytes, tmem, m0 + tile * kBlockM, h, b, n_tiles, key0, part,
+                                 !C::kPersistent || unit + (int)gridDim.x >= n_units, &abort_flag, &redo_flag, xchg[tile]);
+            else pass_sync<C>();
+        } while (next_unit());
     } else if (warp == kProducerWarp) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
         // ------------------------------------------------ TMA producer (warp-uniform, one elected lane issues)
@@ -845,6 +896,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
                 if (pass != kMaxOnly && !(sent && j == 0)) load_v(gv0 + j, j);
             }
         };
+        do {
         produce_pass(kSpeculate);
         int k_loads = n_tiles, v_loads = n_tiles;
         pass_sync<C>();
@@ -858,6 +910,13 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
             wait_bar(bar.kf + 8 * (g % C::kStagesK), (g / C::kStagesK) & 1, &abort_flag, p.err_word);
         for (int g = (v_loads > C::kStagesV ? v_loads - C::kStagesV : 0); g < v_loads; ++g)
             wait_bar(bar.vf + 8 * (g % C::kStagesV), (g / C::kStagesV) & 1, &abort_flag, p.err_word);
+        if constexpr (C::kPersistent) {          // nor may a commit still be on its way to a barrier that is set up afresh
+            for (int g = (k_loads > C::kStagesK ? k_loads - C::kStagesK : 0); g < k_loads; ++g)
+                wait_bar(bar.ke + 8 * (g % C::kStagesK), (g / C::kStagesK) & 1, &abort_flag, p.err_word);
+            for (int g = (v_loads > C::kStagesV ? v_loads - C::kStagesV : 0); g < v_loads; ++g)
+                wait_bar(bar.ve + 8 * (g % C::kStagesV), (g / C::kStagesV) & 1, &abort_flag, p.err_word);
+        }
+        } while (next_unit());
     } else if (warp == kIssuerWarp || warp == kIssuerWarp + 1) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
         // ------------------------------------------------ MMA issuer (warp-uniform, one elected lane issues)
@@ -936,20 +995,22 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
                 __syncwarp();
             }
         };
-        if (t < q_tiles) {
-            wait_bar(bar.q + 8 * t, 0, &abort_flag, p.err_word);
-            issue_pass(kSpeculate);
-        }
-        pass_sync<C>();
-        if (redo_flag && t < q_tiles) {
-            issue_pass(kMaxOnly);
-            issue_pass(kExact);
-        }
+        do {
+            if (t < q_tiles) {
+                wait_bar(bar.q + 8 * t, 0, &abort_flag, p.err_word);
+                issue_pass(kSpeculate);
+            }
+            pass_sync<C>();
+            if (redo_flag && t < q_tiles) {
+                issue_pass(kMaxOnly);
+                issue_pass(kExact);
+            }
+        } while (next_unit());
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
         if (p.copy_dst) copy_role<C>(p, sCopy, bar_copy, &abort_flag);
         __syncwarp();
-        pass_sync<C>();
+        do pass_sync<C>(); while (next_unit());
     }
 
     tc_fence_before();
@@ -1096,13 +1157,15 @@ int32_t launch_dh(const AttnArgs &a, cudaStream_t stream, SplitPlan plan = Split
         p.part_lse = reinterpret_cast<float *>(static_cast<char *>(a.split_ws));
         p.part_o = p.part_lse + (rows + 63) / 64 * 64;
     }
-    const unsigned grid = (unsigned)(p.n_full + (split ? plan.units * plan.split : 0));
+    const int slots = sm_count() * C::kCtasPerSM;
+    const unsigned grid = C::kPersistent ? (unsigned)(p.n_full < slots ? p.n_full : slots) : (unsigned)(p.n_full + (split ? plan.units * plan.split : 0));
+    const int units_per_cta = C::kPersistent ? (int)((p.n_full + grid - 1) / grid) : 1;
     // The rows to copy go with the attention when its CTAs live long enough for their shares: 4 KB a microsecond against
     // 0.4 us a key tile and 4 us for a CTA's set-up and a launch less.  (Measured: a batch of 4 KB takes ~1.5 us with two or
     // three of them in flight.)
     const long long copy_rows = (long long)a.B * a.M;
     const double copy_us = a.copy_dst ? (double)((copy_rows + grid - 1) / grid) * a.copy_elems * 2 / 4096 : 0.0;
-    const bool copy_here = a.copy_dst && (long long)a.B * a.N_tok * (a.copy_elems / 8) < 0x7fffffffll && copy_us <= 0.4 * ((a.N + C::kBlockN - 1) / C::kBlockN) / p.split + 4.0;
+    const bool copy_here = a.copy_dst && (long long)a.B * a.N_tok * (a.copy_elems / 8) < 0x7fffffffll && copy_us <= 0.4 * ((a.N + C::kBlockN - 1) / C::kBlockN) * units_per_cta / p.split + 4.0;
     p.copy_src = copy_here ? reinterpret_cast<const uint4 *>(a.copy_src) : nullptr;
     p.copy_dst = copy_here ? reinterpret_cast<uint4 *>(a.copy_dst) : nullptr;
     p.copy_bytes = (uint32_t)a.copy_elems * 2;

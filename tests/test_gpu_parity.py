@@ -829,6 +829,20 @@ def test_cross_attention_of_selected_rows(oracle, d, N_kv):
     assert np.array_equal(got[mask], f64(cache)[mask])
 
 
+# ------------------------------------------------------------------ small CTAs that walk over several units
+@pytest.mark.parametrize("H,N,M,amp", [(60, 700, 700, 1.0),      # three units a CTA, eleven key tiles
+                                       (50, 400, 390, 12.0),     # sharp logits: some units are redone, their neighbours not
+                                       # one key tile (the odd warpgroups have none); two, the second with one key.  A row sum
+                                       # of bf16-rounded probabilities is within 2^-9 of the exact one, so a row's LSE within
+                                       # 2.0e-3: with 40 keys the roundings do not average out to the 1e-3 of long rows, and
+                                       # amp > 1 selects the 5e-3 bound that such rows have elsewhere
+                                       (150, 40, 33, 1.01),
+                                       (160, 65, 65, 1.01)])
+def test_small_ctas_walk_over_units(oracle, H, N, M, amp):
+    """More units than the 296 slots of a B200's SMs, so that barriers, stages and TMEM are reused from unit to unit."""
+    _attn_case(oracle, 2, H, N, 64, M, seed=H + N, amp=amp, small_ctas=True)
+
+
 # ------------------------------------------------------------------ refresh of the reference inputs beside the attention
 @pytest.mark.parametrize("B,H,d,N_v,n_always,k", [
     (1, 2, 64, 256, 0, 1),            # one row of 256 bytes: one lane of one batch
