@@ -24,9 +24,9 @@
 //
 // The softmax is bound by the exponentials (XU pipe, 16 per clock per SM), by the issue slots and by the
 // latencies of its own chain, so the common path of a key tile is kept to: load S, one FFMA + one
-// exponential per element, (sum,) pack, store.  A part of the exponentials (three of eight pairs at head_dim 64 and
-// 128, one of four at 72) are a polynomial on the FMA pipe instead of ex2 on the XU, and at head_dim 64 the row sums are
-// left to the tensor core (P times a column of ones, 16 more accumulator columns).  The reference maximum
+// exponential per element, (sum,) pack, store.  A part of the exponentials (three of eight pairs at head_dim 64, one
+// of four at 72, none at 128) are a polynomial on the FMA pipe instead of ex2 on the XU, and at head_dim 64 the row sums
+// are left to the tensor core (P times a column of ones, 16 more accumulator columns).  The reference maximum
 // is the exact row maximum of key tile 0 (plus a shift) and is then only checked through the sums of
 // exponentials: while they stay below a limit the probabilities are accepted as they are (they are relative
 // to a stale maximum, which the final normalisation cancels; fp32 and bf16 have the range).  Otherwise the
@@ -95,15 +95,15 @@ template <int DH, int TM> struct Cfg {
     // head_dim 72 gains nothing from it and 128 has no TMEM columns left: they sum the fp32 exponentials themselves.
     static constexpr bool kOnes = DH == 64;
     static constexpr int kSBufs = 2;                              // S buffers per query tile: one per softmax warpgroup
-    // Pairs of exponentials that are computed on the FMA pipe instead of the XU: three of eight at head_dim 64 and 128,
-    // one of four at 72, one of eight in its small CTAs, whose registers do not hold more (62 against 58.5 us for 13106 x 226
-    // x 16; us a launch, under the power cap: head_dim 64, 9001 x 17776 x 48 heads, 4 / 5 / 6 / 7 / 8 of 16:
-    // 2143 / 2123 / 2083 / 2140 / 2203; 72, 2 x 6553 x 16384 x 16, 2 / 4 / 5 / 6 / 8: 1190 / 1150 / 1152 / 1165 / 1233; 128,
-    // 3276 x 65536 x 24, none / 5 / 6 / 7 / 8: 2250 / 2170 / 2130 / 2457 / 2400).  Degree 3 where the row sum or the sums of P
-    // had that error already, 5 at head_dim 128, whose LSE keeps the precision it has with the XU alone.
+    // Pairs of exponentials that are computed on the FMA pipe instead of the XU: three of eight at head_dim 64, one of four
+    // at 72, one of eight in its small CTAs, whose registers do not hold more (62 against 58.5 us for 13106 x 226 x 16; us a
+    // launch, under the power cap: head_dim 64, 9001 x 17776 x 48 heads, 4 / 5 / 6 / 7 / 8 of 16: 2143 / 2123 / 2083 / 2140 /
+    // 2203; 72, 2 x 6553 x 16384 x 16, 2 / 4 / 5 / 6 / 8: 1190 / 1150 / 1152 / 1165 / 1233).  None at 128, whose row sums are
+    // fp32 sums of what the XU returns: a polynomial as exact as that (degree 5, the argument formed as for the XU) is
+    // slower than the XU in every share (0 / 1 / 2 / 3 of eight pairs: 3276 x 65536 x 24 heads 2128 / 2117 / 2149 / 2227,
+    // 35640 x 118800 x 24 40200 / 40300 / 40700 / 42300, 1132 x 3594 x 24 53.8 / 60 / 53.8 / 53.8).
     static constexpr int kPolyPeriod = (DH == 72 && TM == 2) ? 4 : 8;
-    static constexpr int kPolyPairs = (DH == 72) ? 1 : 3;
-    static constexpr int kPolyDeg = (DH == 128) ? 5 : 3;
+    static constexpr int kPolyPairs = (DH == 72) ? 1 : (DH == 64) ? 3 : 0;
     static constexpr int kSoftmaxWarps = 4 * kTilesM * kSplit;
     static constexpr int kAhead = kSBufs;                         // Q K^T runs this many key tiles ahead of P V
     static constexpr int kThreads = (kSoftmaxWarps + 4) * 32;     // + producer, two issuers, one register donor
@@ -183,16 +183,15 @@ __device__ __forceinline__ unsigned long long fadd2(unsigned long long a, float 
 }
 
 // 2^x for a pair of logits s, x = s * sl2 + neg, without the XU pipe: x = n + f with n = floor(x) taken by adding
-// 1.5 * 2^23 rounded down, a polynomial for 2^f on [0, 1) (fitted here for the least relative error with p(0) = 1: 8.6e-5
-// in degree 3, 1.6e-7, as much as ex2.approx has, in degree 5), and n added to the exponent field.  x has to stay in the
-// range of normal numbers: below -126 the result is 2^-126 instead of 0, which no sum notices; above 127 the exponent
-// field would wrap around to a small number and hide the overflow from the check on the sums, so x stops at 127, whose
-// 2^127 trips that check as surely as the XU's +inf does.  Both limits come with the scaling, for one instruction per logit
-// instead of two and a half: the saturating FMA leaves u = (x + 126) / 253 clamped to [0, 1] (mul = sl2 / 253,
-// add = (neg + 126) / 253; 3e-8 of rounding in u is 8e-6 in x, either way), and x = 253 u - 126 is never formed, only its
+// 1.5 * 2^23 rounded down, a cubic for 2^f on [0, 1) (fitted here for the least relative error with p(0) = 1: 8.6e-5),
+// and n added to the exponent field.  x has to stay in the range of normal numbers: below -126 the result is 2^-126
+// instead of 0, which no sum notices; above 127 the exponent field would wrap around to a small number and hide the
+// overflow from the check on the sums, so x stops at 127, whose 2^127 trips that check as surely as the XU's +inf does.
+// Both limits come with the scaling, for one instruction per logit instead of two and a half: the saturating FMA leaves
+// u = (x + 126) / 253 clamped to [0, 1] (mul = sl2 / 253, add = (neg + 126) / 253; the roundings of u, mul and add come to
+// 1.4e-5 in x, against 2e-6 on the XU, and are beside the cubic's error only), and x = 253 u - 126 is never formed, only its
 // floor and its fraction are.
 constexpr float kExpLo = -126.0f, kExpSpan = 253.0f;
-template <int DEG>
 __device__ __forceinline__ void exp2_poly2(float &x0, float &x1, float mul, float add) {
     float u0, u1;
     asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(u0) : "f"(x0), "f"(mul), "f"(add));
@@ -206,31 +205,15 @@ __device__ __forceinline__ void exp2_poly2(float &x0, float &x1, float mul, floa
         "sub.rn.f32x2 %1, mg, %0;\n\t"               // -126 - floor(x)
         "fma.rn.f32x2 %1, %2, sp, %1;\n\t}"          // f = x - floor(x)
         : "=&l"(t), "=&l"(f) : "l"(u));
-    static_assert(DEG == 3 || DEG == 5, "fitted degrees");
-    if constexpr (DEG == 3)
-        asm("{\n\t.reg .b64 c1, c2, c3, one;\n\t"
-            "mov.b64 c3, 0x3D9DD4DF3D9DD4DF;\n\t"        // 2^f ~ 1 + f (c1 + f (c2 + f c3))
-            "mov.b64 c2, 0x3E691C043E691C04;\n\t"
-            "mov.b64 c1, 0x3F31F3293F31F329;\n\t"
-            "mov.b64 one, 0x3F8000003F800000;\n\t"
-            "fma.rn.f32x2 %0, %1, c3, c2;\n\t"
-            "fma.rn.f32x2 %0, %0, %1, c1;\n\t"
-            "fma.rn.f32x2 %0, %0, %1, one;\n\t}"
-            : "=&l"(pl) : "l"(f));
-    else
-        asm("{\n\t.reg .b64 c1, c2, c3, c4, c5, one;\n\t"
-            "mov.b64 c5, 0x3AF4BA7D3AF4BA7D;\n\t"        // 1 + f (c1 + f (c2 + f (c3 + f (c4 + f c5))))
-            "mov.b64 c4, 0x3C13BC2B3C13BC2B;\n\t"
-            "mov.b64 c3, 0x3D648E733D648E73;\n\t"
-            "mov.b64 c2, 0x3E75EDAB3E75EDAB;\n\t"
-            "mov.b64 c1, 0x3F31725D3F31725D;\n\t"
-            "mov.b64 one, 0x3F8000003F800000;\n\t"
-            "fma.rn.f32x2 %0, %1, c5, c4;\n\t"
-            "fma.rn.f32x2 %0, %0, %1, c3;\n\t"
-            "fma.rn.f32x2 %0, %0, %1, c2;\n\t"
-            "fma.rn.f32x2 %0, %0, %1, c1;\n\t"
-            "fma.rn.f32x2 %0, %0, %1, one;\n\t}"
-            : "=&l"(pl) : "l"(f));
+    asm("{\n\t.reg .b64 c1, c2, c3, one;\n\t"
+        "mov.b64 c3, 0x3D9DD4DF3D9DD4DF;\n\t"        // 2^f ~ 1 + f (c1 + f (c2 + f c3))
+        "mov.b64 c2, 0x3E691C043E691C04;\n\t"
+        "mov.b64 c1, 0x3F31F3293F31F329;\n\t"
+        "mov.b64 one, 0x3F8000003F800000;\n\t"
+        "fma.rn.f32x2 %0, %1, c3, c2;\n\t"
+        "fma.rn.f32x2 %0, %0, %1, c1;\n\t"
+        "fma.rn.f32x2 %0, %0, %1, one;\n\t}"
+        : "=&l"(pl) : "l"(f));
     uint32_t t0, t1, p0, p1;
     asm("mov.b64 {%0, %1}, %2;" : "=r"(t0), "=r"(t1) : "l"(t));
     asm("mov.b64 {%0, %1}, %2;" : "=r"(p0), "=r"(p1) : "l"(pl));
@@ -373,7 +356,7 @@ __device__ __forceinline__ void softmax_step(SoftmaxState &st, int j, int g)
     // the first kPolyPairs of every kPolyPeriod pairs go to the FMA pipe, the rest to the XU
 #pragma unroll
     for (int i = 0; i < NS; i += 2) {
-        if ((i / 2) % C::kPolyPeriod < C::kPolyPairs) exp2_poly2<C::kPolyDeg>(cur[i], cur[i + 1], mul, add);
+        if ((i / 2) % C::kPolyPeriod < C::kPolyPairs) exp2_poly2(cur[i], cur[i + 1], mul, add);
         else {
             ffma2(cur[i], cur[i + 1], sl2, neg);
             cur[i] = ex2(cur[i]); cur[i + 1] = ex2(cur[i + 1]);

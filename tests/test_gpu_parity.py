@@ -382,6 +382,29 @@ def test_attn_single_overflowing_key_in_any_column_of_a_later_tile(oracle, d, co
     assert np.abs(want_o - f64(vb)[0, 64 + col][None, None]).max() < 1e-9            # the oracle agrees: one-hot rows
 
 
+@pytest.mark.parametrize("base", [0, 64])          # the key sits in the first tile, or it makes the CTA redo its pass
+def test_attn_head_dim_128_computes_every_key_column_alike(base):
+    """At head_dim 128 the row sums are fp32 sums of exponentials and the LSE is as exact as those.  One key holds a row's
+    whole weight (the others are 200 or more below it in the log2 domain and vanish in fp32): wherever it stands in its
+    tile, the same logit has to give the same LSE, bit for bit."""
+    N, d = 130, 128
+    q = torch.zeros(1, N, 1, d, dtype=torch.bfloat16, device="cuda")
+    q[0, :, 0, 0] = torch.linspace(16, 64, N, device="cuda").bfloat16()
+    v = torch.randn(1, N, 1, d, dtype=torch.bfloat16, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    ws, s = A.new_workspace(A.OP_SPARSE_ATTN, 1, 1, N, N, d), A.bhnd_strides(N, 1, d)
+    first = None
+    for col in list(range(16)) + [37, 62, 63]:
+        k = torch.zeros_like(q)
+        k[0, base + col, 0, 0] = 100.0
+        out, lse = torch.zeros_like(q), torch.zeros(1, 1, N, device="cuda")
+        A.astraea_sparse_attn(q, k, v, s, s, s, None, N, out, lse, 1, 1, N, d, workspace=ws)
+        A.astraea_poll_error(ws)
+        want = q[0, :, 0, 0].double() * 100.0 / math.sqrt(d)
+        assert (lse[0, 0].double() - want).abs().max().item() < 2e-6 * 64 * 100 / math.sqrt(d), col
+        first = lse if first is None else first
+        assert torch.equal(lse, first), col
+
+
 @pytest.mark.parametrize("d", [64, 72, 128])
 def test_attn_select_q_and_k_ablation(oracle, d):
     """kv_idx: the softmax runs over the listed keys/values only (the ablation that also masks K and V)."""
