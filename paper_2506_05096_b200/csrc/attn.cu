@@ -183,15 +183,16 @@ __device__ __forceinline__ unsigned long long fadd2(unsigned long long a, float 
 }
 
 // 2^x for a pair of logits s, x = s * sl2 + neg, without the XU pipe: x = n + f with n = floor(x) taken by adding
-// 1.5 * 2^23 rounded down, a cubic for 2^f on [0, 1) (fitted here for the least relative error with p(0) = 1: 8.6e-5),
-// and n added to the exponent field.  x has to stay in the range of normal numbers: below -126 the result is 2^-126
-// instead of 0, which no sum notices; above 127 the exponent field would wrap around to a small number and hide the
-// overflow from the check on the sums, so x stops at 127, whose 2^127 trips that check as surely as the XU's +inf does.
-// Both limits come with the scaling, for one instruction per logit instead of two and a half: the saturating FMA leaves
-// u = (x + 126) / 253 clamped to [0, 1] (mul = sl2 / 253, add = (neg + 126) / 253; the roundings of u, mul and add come to
-// 1.4e-5 in x, against 2e-6 on the XU, and are beside the cubic's error only), and x = 253 u - 126 is never formed, only its
-// floor and its fraction are.
-constexpr float kExpLo = -126.0f, kExpSpan = 253.0f;
+// 1.5 * 2^23 rounded down, a cubic for 2^f on [0, 1) (fitted here for the least relative error with p(0) = 1: 8.6e-5), and n
+// added to the exponent field.  x has to stay in the range of normal numbers: below -126 the result is 2^-126 instead of 0,
+// which no sum notices; above 127 the exponent field would wrap around to a small number and hide the overflow from the
+// check on the sums, so x stops at 105, whose 2^105 trips that check as surely as the XU's +inf does.  A NaN has to end
+// there as well: it trips the check, in the pass against exact maxima too, where nothing else can, and makes its row NaN.
+// Both limits come with the scaling, for one instruction per logit: the saturating FMA leaves u = (105 - x) / 231 clamped to
+// [0, 1], a NaN as 0 (mul = -sl2 / 231, add = (105 - neg) / 231), and x = 105 - 231 u is never formed, only its floor and
+// its fraction are.  u and add are rounded by up to 7e-6 of x each, well below the cubic's error.  (231 is a span whose
+// reciprocal fp32 holds to 1e-9: with 253, held to 4e-8, all these columns were 7e-6 too small, 3e-6 in the LSE.)
+constexpr float kExpHi = 105.0f, kExpSpan = 231.0f;
 __device__ __forceinline__ void exp2_poly2(float &x0, float &x1, float mul, float add) {
     float u0, u1;
     asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(u0) : "f"(x0), "f"(mul), "f"(add));
@@ -199,10 +200,10 @@ __device__ __forceinline__ void exp2_poly2(float &x0, float &x1, float mul, floa
     unsigned long long u, t, f, pl;
     asm("mov.b64 %0, {%1, %2};" : "=l"(u) : "f"(u0), "f"(u1));
     asm("{\n\t.reg .b64 mg, sp;\n\t"
-        "mov.b64 mg, 0x4B3FFF824B3FFF82;\n\t"        // 1.5 * 2^23 - 126, twice
-        "mov.b64 sp, 0x437D0000437D0000;\n\t"        // 253
+        "mov.b64 mg, 0x4B4000694B400069;\n\t"        // 1.5 * 2^23 + 105, twice
+        "mov.b64 sp, 0xC3670000C3670000;\n\t"        // -231
         "fma.rm.f32x2 %0, %2, sp, mg;\n\t"           // 1.5 * 2^23 + floor(x): the low mantissa bits are floor(x)
-        "sub.rn.f32x2 %1, mg, %0;\n\t"               // -126 - floor(x)
+        "sub.rn.f32x2 %1, mg, %0;\n\t"               // 105 - floor(x)
         "fma.rn.f32x2 %1, %2, sp, %1;\n\t}"          // f = x - floor(x)
         : "=&l"(t), "=&l"(f) : "l"(u));
     asm("{\n\t.reg .b64 c1, c2, c3, one;\n\t"
@@ -352,7 +353,7 @@ __device__ __forceinline__ void softmax_step(SoftmaxState &st, int j, int g)
         else asm volatile("bar.arrive 4, 256;" ::: "memory");
     }
     const float neg = -st.m_ref * sl2 - st.shift;
-    const float mul = sl2 * (1.0f / kExpSpan), add = (neg - kExpLo) * (1.0f / kExpSpan);
+    const float mul = sl2 * (-1.0f / kExpSpan), add = (kExpHi - neg) * (1.0f / kExpSpan);
     // the first kPolyPairs of every kPolyPeriod pairs go to the FMA pipe, the rest to the XU
 #pragma unroll
     for (int i = 0; i < NS; i += 2) {
@@ -504,6 +505,8 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
             tc_wait_ld();
             st.l_sum = __uint_as_float(o[0]);
         }
+        // against the exact maximum no term is above 1 but for a logit of NaN or +inf, which makes the row NaN
+        if (!(st.l_sum <= kTileSumLimit)) st.l_sum = __int_as_float(0x7fc00000);
     }
 
     // ------------------------------------------------ epilogue: normalise and scatter

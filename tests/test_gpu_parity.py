@@ -405,6 +405,41 @@ def test_attn_head_dim_128_computes_every_key_column_alike(base):
         assert torch.equal(lse, first), col
 
 
+@pytest.mark.parametrize("d,small", [(64, False), (64, True), (72, False), (72, True), (128, False)])
+@pytest.mark.parametrize("kind", ["nan_key", "inf_key", "nan_query"])
+def test_attn_non_finite_logits_reach_their_rows_from_every_column(d, small, kind):
+    """A logit of NaN or +inf makes its row NaN (output and LSE) whichever pipe computes its column; a logit of -inf has no
+    weight; rows without any are what they would be."""
+    B, H, N, M = 1, 2, 200, 150
+    g = torch.Generator("cuda").manual_seed(7)
+    q, k, v = (torch.randn(B, N, H, d, dtype=torch.bfloat16, device="cuda", generator=g) for _ in range(3))
+    q[..., 0] = q[..., 0].abs().clamp(min=0.25) * torch.where(torch.arange(N, device="cuda") % 2 == 0, 1.0, -1.0)[:, None].bfloat16()
+    ws, s = A.new_workspace(A.OP_SPARSE_ATTN, B, H, N, M, d), A.bhnd_strides(N, H, d)
+    idx = torch.arange(20, 20 + M, dtype=torch.int32, device="cuda")[None]
+    flags = A.ATTN_COMPACT_OUT | (A.ATTN_SMALL_CTAS if small else 0)
+    for pos in list(range(16)) + [47, 63, 64, 70, 78, 127, 128, 199]:
+        qq, kk = q.clone(), k.clone()
+        if kind == "nan_key":
+            kk[0, pos, 1, 3] = float("nan")
+        elif kind == "inf_key":
+            kk[0, pos, 1, 0] = float("inf")                # +inf against even tokens, -inf against odd ones
+        else:
+            qq[0, 20 + pos % M, 1, 5] = float("nan")
+        out, lse = torch.zeros(B, M, H, d, dtype=torch.bfloat16, device="cuda"), torch.zeros(B, H, M, device="cuda")
+        A.astraea_sparse_attn(qq, kk, v, s, s, s, idx, M, out, lse, B, H, N, d, flags=flags, workspace=ws)
+        A.astraea_poll_error(ws)
+        z = torch.einsum("mhd,nhd->hmn", qq[0, 20:20 + M].double(), kk[0].double()) / math.sqrt(d)
+        bad = (z.isnan() | (z == math.inf)).any(-1)                                      # [H, M]
+        assert bad.any() and not bad.all()
+        assert torch.equal(lse[0].isnan(), bad), (kind, pos)
+        assert torch.equal(out[0].isnan().all(-1).T, bad) and torch.equal(out[0].isnan().any(-1).T, bad), (kind, pos)
+        ok = ~bad
+        p = z.masked_fill(bad[..., None], 0.0).softmax(-1)
+        want = torch.einsum("hmn,nhd->hmd", p, v[0].double())
+        assert_attn_close(out[0].transpose(0, 1)[ok].double().cpu().numpy(), want[ok].cpu().numpy(), what=(kind, pos))
+        assert (lse[0].double() - z.logsumexp(-1))[ok].abs().max().item() < 2e-3, (kind, pos)
+
+
 @pytest.mark.parametrize("d", [64, 72, 128])
 def test_attn_select_q_and_k_ablation(oracle, d):
     """kv_idx: the softmax runs over the listed keys/values only (the ablation that also masks K and V)."""
