@@ -66,6 +66,8 @@ constexpr int kSplit = 2;                        // softmax warpgroups per query
 // row of most CTAs, but not 100.
 constexpr float kRefShift = 48.0f;
 constexpr float kTileSumLimit = 1267650600228229401496703205376.0f;   // 2^100
+// LSE of a key share whose CTA gave up: a NaN with a payload that no arithmetic produces (a row may be NaN on its own account)
+constexpr uint32_t kGaveUpLse = 0xffc0dead;
 
 // DH: head_dim.  TM: 128-row query tiles per CTA.  Two share every K/V tile in shared memory and run one CTA per SM;
 // one (head_dim 64 / 72 only) lets two CTAs share an SM, which costs ~5 % of throughput per SM but halves the
@@ -525,11 +527,11 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
     const float inv_l = 1.0f / l_sum;
     if (part >= 0) {
         // a share of the keys only: the normalised row and its LSE go to the workspace in fp32 (every row of the tile,
-        // listed or not; the merge knows which ones count).  A CTA that gave up marks its rows with NaN.
+        // listed or not; the merge knows which ones count).  A CTA that gave up marks its rows.
         const size_t prow = (size_t)part * (C::kTilesM * kBlockM) + tile * kBlockM + wtid;
         float *po = p.part_o + prow * C::kDH;
         if (par == 0)
-            p.part_lse[prow] = *abort_flag ? __int_as_float(0x7fc00000) : st.m_ref * p.scale + st.shift * 0.6931471805599453f + logf(l_sum);
+            p.part_lse[prow] = *abort_flag ? __uint_as_float(kGaveUpLse) : st.m_ref * p.scale + st.shift * 0.6931471805599453f + logf(l_sum);
 #pragma unroll
         for (int cc = 0; cc < ncol; cc += 32) {
             const int c = col0 + cc;
@@ -1028,7 +1030,7 @@ __global__ void __launch_bounds__(ROWS) merge_parts_kernel(const Params p)
         lse[i] = -INFINITY;
         if (i < p.split) {
             lse[i] = __ldcg(p.part_lse + (part0 + i) * ROWS + r);
-            gave_up |= lse[i] != lse[i];
+            gave_up |= __float_as_uint(lse[i]) == kGaveUpLse;
             mx = fmaxf(mx, lse[i]);
         }
     }

@@ -583,6 +583,26 @@ def test_attn_bad_indices_in_a_launch_that_is_split_by_keys():
     assert bool((out[0, untouched] == 3.0).all()) and bool((lse[0][:, untouched] == -7.0).all())
 
 
+@pytest.mark.parametrize("d", [64, 72, 128])
+def test_attn_non_finite_rows_in_a_launch_that_is_split_by_keys(d):
+    """A row that one share of the keys makes NaN is NaN after the merge (output and LSE), not the row that was cached."""
+    B, H, N, M = 1, 2, 2100, 260
+    g = torch.Generator("cuda").manual_seed(8)
+    q, k, v = (torch.randn(B, N, H, d, dtype=torch.bfloat16, device="cuda", generator=g) for _ in range(3))
+    ws, s = A.new_workspace(A.OP_SPARSE_ATTN, B, H, N, M, d), A.bhnd_strides(N, H, d)
+    assert A.astraea_sparse_attn_plan(B, H, N, M, d, workspace_bytes=ws.numel())["split"] == 2
+    idx = (torch.arange(M, dtype=torch.int32, device="cuda") * 8)[None]
+    q[0, 8 * 7, 0, 5] = float("nan")                 # one row of head 0, in both shares
+    k[0, 1700, 1, 9] = float("nan")                  # every row of head 1, in its second share
+    out, lse = torch.full((B, N, H, d), 3.0, dtype=torch.bfloat16, device="cuda"), torch.full((B, H, N), -7.0, device="cuda")
+    A.astraea_sparse_attn(q, k, v, s, s, s, idx, M, out, lse, B, H, N, d, workspace=ws)
+    A.astraea_poll_error(ws)
+    bad = torch.zeros(H, N, dtype=torch.bool, device="cuda")
+    bad[0, 8 * 7] = True
+    bad[1, idx[0].long()] = True
+    assert torch.equal(lse[0].isnan(), bad) and torch.equal(out[0].isnan().all(-1).T, bad) and torch.equal(out[0].isnan().any(-1).T, bad)
+
+
 # ------------------------------------------------------------- the whole step
 def _step_case(oracle, w, seed, theta, steps=1):
     inp = synth.make_step_inputs(w, seed)
