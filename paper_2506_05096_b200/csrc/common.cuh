@@ -72,6 +72,14 @@ cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// 16-byte load of data that is used again soon (vectors that every row of a launch shares): cached in L1, but not as
+// read-only data, since an earlier kernel of the library may have computed it (a modulation vector out of a linear layer)
+__device__ __forceinline__ uint4 ld_cached(const uint4 *p) {
+    uint4 r;
+    asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    return r;
+}
+
 // 16-byte load of data that is used once (no L1 allocation)
 __device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
     uint4 r;

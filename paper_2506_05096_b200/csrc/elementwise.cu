@@ -90,8 +90,8 @@ layernorm_modulate_kernel(const uint4 *__restrict__ x, const int32_t *__restrict
             if (c < vec_per_row) {
                 f32x2 f[4], sc[4], sh[4];
                 unpack8(v[u], f);
-                if (scale) unpack8(__ldg(scale + (long long)b * vec_per_row + c), sc);
-                if (shift) unpack8(__ldg(shift + (long long)b * vec_per_row + c), sh);
+                if (scale) unpack8(ld_cached(scale + (long long)b * vec_per_row + c), sc);
+                if (shift) unpack8(ld_cached(shift + (long long)b * vec_per_row + c), sh);
                 uint32_t w[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {

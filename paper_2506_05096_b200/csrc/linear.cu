@@ -239,7 +239,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
                     for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(o[v * 8 + i]);
                     if (col < p.N_out) {                 // N_out is a multiple of 8; columns past it are never stored
                         if (p.bias) {
-                            const uint4 bb = __ldg(reinterpret_cast<const uint4 *>(p.bias + col));
+                            const uint4 bb = ld_cached(reinterpret_cast<const uint4 *>(p.bias + col));
                             const uint32_t bw[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
@@ -252,7 +252,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
                             for (int i = 0; i < 8; ++i) f[i] = 0.5f * f[i] * (1.0f + erf_fast(f[i] * 0.70710678118654752f));
                         }
                         if (gate) {
-                            const uint4 gg = __ldg(reinterpret_cast<const uint4 *>(gate + col));
+                            const uint4 gg = ld_cached(reinterpret_cast<const uint4 *>(gate + col));
                             const uint32_t gw[4] = {gg.x, gg.y, gg.z, gg.w};
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {

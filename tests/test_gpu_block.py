@@ -114,6 +114,38 @@ def test_gathered_linear_tile_edges(oracle, rows, K, N_out, listed):
     _close(got, want, "tile edges")
 
 
+# ------------------------------------------------------------------ vectors that the library itself computed
+def test_modulation_vectors_out_of_the_kernel_just_before():
+    """Scale, shift, bias and gate may come out of a linear layer launched just before on the same stream, step after step in
+    the same buffers: every step sees that step's vectors, bit for bit as with fresh buffers and the device idle between."""
+    g = torch.Generator("cuda").manual_seed(3)
+    mk = lambda *sh: torch.randn(*sh, dtype=torch.bfloat16, device="cuda", generator=g)  # noqa: E731
+    N, D, T = 3000, 512, 12
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    x, wv, w = mk(1, N, D), mk(D, D) * D ** -0.5, mk(D, D) * D ** -0.5
+    cond = [mk(1, 1, D) for _ in range(T)]
+
+    def vec(t, out):
+        A.astraea_gathered_linear(cond[t], None, 1, wv, None, out, 1, 1, D, D, workspace=ws)
+
+    def use(v, h, y):
+        A.astraea_layernorm_modulate(x, None, N, v, v, h, 1, N, D, workspace=ws)
+        A.astraea_gathered_linear_residual(h, None, N, w, v, x, v, y, 1, N, D, D, workspace=ws)
+
+    v, hs, ys = mk(1, 1, D), [torch.empty_like(x) for _ in range(T)], [torch.empty_like(x) for _ in range(T)]
+    for t in range(T):
+        vec(t, v)
+        use(v, hs[t], ys[t])
+    A.astraea_poll_error(ws)
+    for t in range(T):
+        v2, h2, y2 = torch.empty_like(v), torch.empty_like(x), torch.empty_like(x)
+        vec(t, v2)
+        torch.cuda.synchronize()
+        use(v2.clone(), h2, y2)
+        torch.cuda.synchronize()
+        assert torch.equal(hs[t], h2) and torch.equal(ys[t], y2), t
+
+
 # ------------------------------------------------------------------ linear layer with a gated residual
 @pytest.mark.parametrize("res_compact,out_compact,in_compact,gelu", [(False, False, False, False), (False, True, False, False),
                                                                      (True, True, True, False), (True, False, True, True)])
