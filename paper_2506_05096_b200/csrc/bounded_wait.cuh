@@ -16,17 +16,19 @@ __device__ __forceinline__ bool elect_one() {
 
 // Bounded mbarrier wait.  Gives up after the limit, or at once when another wait of this CTA
 // already gave up; the caller carries on (its results are void, the error word says so).
+// CLUSTER: for arrivals from other CTAs, relaxed at cluster scope (see mbar_try_wait_cluster).
+template <bool CLUSTER = false>
 __device__ __forceinline__ void wait_bar(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err_word,
                                          uint64_t limit_ns = kWaitLimitNs) {
-    using namespace ptx;
-    if (mbar_try_wait(bar, parity)) return;
+    auto arrived = [&] { return CLUSTER ? ptx::mbar_try_wait_cluster(bar, parity) : ptx::mbar_try_wait(bar, parity); };
+    if (arrived()) return;
     if (*abort_flag) return;
-    const uint64_t t0 = globaltimer_ns();
+    const uint64_t t0 = ptx::globaltimer_ns();
     uint32_t spins = 0;
-    while (!mbar_try_wait(bar, parity)) {
+    while (!arrived()) {
         if ((++spins & 255u) == 0) {
             if (*abort_flag) return;
-            if (globaltimer_ns() - t0 > limit_ns) {
+            if (ptx::globaltimer_ns() - t0 > limit_ns) {
                 *abort_flag = 1;
                 atomicExch(err_word, kErrTimeout);
                 return;

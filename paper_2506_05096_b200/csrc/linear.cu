@@ -13,9 +13,10 @@
 //   warps 0-15  epilogue: four threads per output row (every fourth group of 32 columns); TMEM -> registers -> (+ bias, GELU, gate,
 //               residual) -> bf16 -> the row of y that idx names (fused scatter);
 //   warp 16     TMA producer: this CTA's half of a W tile per stage (rows past N_out read as zero) and, when the rows
-//               of x are a contiguous matrix (no list, or compact rows), the CTA's 128 rows of x as well;
-//   warp 17     even CTA: tcgen05.mma issuer for the pair, four MMAs per stage; odd CTA: tells the even one which of its
-//               stages have landed;
+//               of x are a contiguous matrix (no list, or compact rows), the CTA's 128 rows of x as well; the bytes of both
+//               CTAs are counted on the even one's barrier;
+//   warp 17     even CTA: tcgen05.mma issuer for the pair, four MMAs per stage; odd CTA (listed rows only): passes on to the
+//               even one that the gathered rows of a stage have landed;
 //   warps 18-19 (listed rows only) gather of the A operand: the listed rows of x, 64 columns (128 bytes) per
 //               pipeline stage, by 16-byte cp.async into the 128-byte-swizzled layout the MMA reads (rows past the end
 //               and entries out of range are zero-filled); the copies arrive on the stage's barrier by themselves, so a
@@ -92,10 +93,11 @@ __device__ __forceinline__ float erf_fast(float x) {
     return copysignf(fmaf(-pl * t, e, 1.0f), x);
 }
 
-// 2-D tiled load global -> shared, completion counted in bytes on an mbarrier
+// 2-D tiled load global -> this CTA's shared memory, completion counted in bytes on an mbarrier of either CTA of the pair
+// (address from map_to_rank)
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *m, uint32_t bar, int c0, int c1) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
         ::"r"(dst), "l"(m), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
 
@@ -147,9 +149,10 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
     if (tid == 0) {
         abort_flag = 0;
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(bar_full + 8 * s, (DENSE ? 0 : kGatherWarps * 32) + 1);     // every gather thread + the TMA producer
+            // every gather thread + in the even CTA its TMA producer, for the bytes of both (odd CTA, contiguous rows: not used)
+            mbar_init(bar_full + 8 * s, (DENSE ? 0 : kGatherWarps * 32) + (DENSE || rank == 0 ? 1 : 0));
             mbar_init(bar_empty + 8 * s, 1);                    // the issuer's commit
-            mbar_init(bar_peer + 8 * s, 1);                     // even CTA: the odd CTA's part of the stage has landed
+            mbar_init(bar_peer + 8 * s, 1);                     // even CTA: the odd CTA's gathered rows of the stage have landed
         }
         for (int a = 0; a < kAccSets; ++a) { mbar_init(bar_acc_full + 8 * a, 1); mbar_init(bar_acc_empty + 8 * a, 2 * kEpiWarps); }
         fence_barrier_init();
@@ -289,6 +292,8 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
         }
     } else if (warp == kTmaWarp) {
         // ------------------------------------------------ TMA producer of the W tiles (and of contiguous rows of x)
+        // (the odd CTA's bytes may arrive before the even one has said how many a stage gets: its phase cannot end before that)
+        const uint32_t full0 = map_to_rank(bar_full, 0);
         int g = 0;
         for (int tile = pair; tile < total_tiles; tile += n_pairs) {
             const int tm = tile / tiles_n, tn = tile - tm * tiles_n;
@@ -296,15 +301,15 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
                 const int st = g % kStages;
                 wait_bar(bar_empty + 8 * st, ((g / kStages) & 1) ^ 1, &abort_flag, p.err_word);
                 if (elect_one()) {
-                    mbar_arrive_expect_tx(bar_full + 8 * st, p.bn * kBK + (DENSE ? kABytes : 0));
-                    tma_load_2d(sB + st * kBBytes, &tmap_w, bar_full + 8 * st, ks * kBK, tn * p.bn + (int)rank * (p.bn / 2));
-                    if (DENSE) tma_load_2d(sA + st * kABytes, &tmap_x, bar_full + 8 * st, ks * kBK, tm * kBM + (int)rank * kRowsCta);
+                    if (rank == 0) mbar_arrive_expect_tx(bar_full + 8 * st, 2 * (p.bn * kBK + (DENSE ? kABytes : 0)));
+                    tma_load_2d(sB + st * kBBytes, &tmap_w, full0 + 8 * st, ks * kBK, tn * p.bn + (int)rank * (p.bn / 2));
+                    if (DENSE) tma_load_2d(sA + st * kABytes, &tmap_x, full0 + 8 * st, ks * kBK, tm * kBM + (int)rank * kRowsCta);
                 }
                 __syncwarp();
             }
         }
-        // every copy issued above must have landed before the CTA's shared memory is released
-        for (int gs = (g > kStages ? g - kStages : 0); gs < g; ++gs)
+        // every copy issued above must have landed before either CTA's shared memory is released
+        for (int gs = (g > kStages ? g - kStages : 0); rank == 0 && gs < g; ++gs)
             wait_bar(bar_full + 8 * (gs % kStages), (gs / kStages) & 1, &abort_flag, p.err_word);
     } else if (warp == kMmaWarp && rank == 0) {
         // ------------------------------------------------ MMA issuer of the pair
@@ -312,11 +317,12 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
         int g = 0, it = 0;
         for (int tile = pair; tile < total_tiles; tile += n_pairs, ++it) {
             const int acc = it % kAccSets;
-            wait_bar(bar_acc_empty + 8 * acc, ((it / kAccSets) & 1) ^ 1, &abort_flag, p.err_word);
+            wait_bar<true>(bar_acc_empty + 8 * acc, ((it / kAccSets) & 1) ^ 1, &abort_flag, p.err_word);
             for (int ks = 0; ks < k_steps; ++ks, ++g) {
                 const int st = g % kStages;
                 wait_bar(bar_full + 8 * st, (g / kStages) & 1, &abort_flag, p.err_word);
-                wait_bar(bar_peer + 8 * st, (g / kStages) & 1, &abort_flag, p.err_word);
+                if (!DENSE) wait_bar<true>(bar_peer + 8 * st, (g / kStages) & 1, &abort_flag, p.err_word);
+                fence_acquire_smem();                     // what landed in the odd CTA is in order before the MMAs too
                 if (!DENSE) fence_proxy_async_smem();     // gathered rows were written through the generic proxy
                 tc_fence_after();
                 if (elect_one()) {
@@ -331,14 +337,16 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
             }
         }
     } else if (warp == kMmaWarp) {
-        // ------------------------------------------------ odd CTA: its part of a stage has landed
+        // ------------------------------------------------ odd CTA: the gathered rows of a stage have landed
+        const uint32_t peer0 = map_to_rank(bar_peer, 0);
         int g = 0;
-        for (int tile = pair; tile < total_tiles; tile += n_pairs)
+        for (int tile = pair; !DENSE && tile < total_tiles; tile += n_pairs)
             for (int ks = 0; ks < k_steps; ++ks, ++g) {
                 const int st = g % kStages;
                 wait_bar(bar_full + 8 * st, (g / kStages) & 1, &abort_flag, p.err_word);
-                if (!DENSE) fence_proxy_async_smem();     // gathered rows were written through the generic proxy
-                if (elect_one()) mbar_arrive_cluster(map_to_rank(bar_peer + 8 * st, 0));
+                fence_proxy_async_smem();                 // gathered rows were written through the generic proxy
+                fence_release_smem();
+                if (elect_one()) mbar_arrive_cluster(peer0 + 8 * st);
                 __syncwarp();
             }
     } else if constexpr (!DENSE) {

@@ -57,11 +57,29 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t saddr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
     return r;
 }
-// Arrive on an mbarrier of any CTA of the cluster (address from map_to_rank).  Nothing that the caller wrote to memory
-// is published this way (operands have landed and accumulators have been read before it), so the default scope does:
-// with .release.cluster here and .acquire.cluster in the wait, a handshake per pipeline stage took 1 us.
+// Handshakes between CTAs: arrive on an mbarrier of any CTA of the cluster (address from map_to_rank), wait for it.  Both
+// are relaxed at cluster scope and order nothing by themselves.  Where tensor memory is handed over, the tcgen05 fences
+// around them do; where bytes in shared memory are, the two fences below do.  (A release of everything, as
+// mbarrier.arrive.release.cluster is, also waits for the thread's stores to global memory: 1 us.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t mapped) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(mapped) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapped) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+// what this thread has written or seen written to its CTA's shared memory, before its next relaxed arrive
+__device__ __forceinline__ void fence_release_smem() {
+    asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+}
+// after a relaxed wait: what was released that way is visible, in the shared memory of the whole cluster
+__device__ __forceinline__ void fence_acquire_smem() {
+    asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");

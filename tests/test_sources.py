@@ -19,3 +19,18 @@ def test_no_load_takes_the_read_only_path():
     assert len(names) >= 9
     for name in names:
         assert not re.search(r"__ldg\s*\(|ld\.global\.nc|\bldg\b", _code(name)), name
+
+
+def test_handshakes_between_ctas_have_cluster_scope():
+    """An arrival on another CTA's barrier and the wait for it name the cluster as their scope (the default is the CTA, which
+    promises the other one nothing), and where bytes in shared memory are passed on, a release and an acquire go with them."""
+    ptx, lin = _code("sm100_ptx.cuh"), _code("linear.cu")
+    for arrive in re.findall(r"mbarrier\.arrive\S*shared::cluster\S*", ptx):
+        assert ".cluster.shared::cluster" in arrive, arrive
+    remote = set(re.findall(r"map_to_rank\((bar_\w+)", lin)) - {"bar_full"}          # bar_full: bytes that TMA counts
+    assert remote == {"bar_peer", "bar_acc_empty"}
+    for bar in remote:
+        waits = re.findall(r"wait_bar(<true>)?\(%s\b" % bar, lin)
+        assert waits and all(waits), bar
+    assert re.search(r"fence_release_smem\(\);\s*if \(elect_one\(\)\) mbar_arrive_cluster\(peer0", lin)
+    assert re.search(r"wait_bar<true>\(bar_peer[^;]*;\s*fence_acquire_smem\(\);", lin)
