@@ -37,4 +37,12 @@ __device__ __forceinline__ void wait_bar(uint32_t bar, uint32_t parity, volatile
     }
 }
 
+// Bounded wait for copies (or MMAs) of this CTA that are under way, before its memory is given up: it does not mind that
+// the CTA has given up, and returns after the limit all the same.
+__device__ __forceinline__ void drain_bar(uint32_t bar, uint32_t parity, uint64_t limit_ns = kWaitLimitNs) {
+    if (ptx::mbar_try_wait(bar, parity)) return;
+    const uint64_t t0 = ptx::globaltimer_ns();
+    while (!ptx::mbar_try_wait(bar, parity) && ptx::globaltimer_ns() - t0 <= limit_ns) {}
+}
+
 }  // namespace astraea
