@@ -761,6 +761,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
         tc_fence_before();
         __syncwarp();
         asm volatile("bar.sync 0;" ::: "memory");
+        // a CTA that gave up may still have copies and MMAs in flight: it takes no further unit (nobody waits between the two
+        // barriers, so every thread reads the same flag)
+        if (*static_cast<volatile int *>(&abort_flag)) return false;
         if (tid == 0) {
             redo_flag = 0;
             for (uint32_t a = bars; a < bar.kf; a += 8)

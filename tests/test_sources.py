@@ -34,3 +34,12 @@ def test_handshakes_between_ctas_have_cluster_scope():
         assert waits and all(waits), bar
     assert re.search(r"fence_release_smem\(\);\s*if \(elect_one\(\)\) mbar_arrive_cluster\(peer0", lin)
     assert re.search(r"wait_bar<true>\(bar_peer[^;]*;\s*fence_acquire_smem\(\);", lin)
+
+
+def test_a_cta_that_gave_up_takes_no_further_unit():
+    """Persistent attention CTAs: between the two CTA-wide barriers of a change of unit, the abort flag is looked at by every
+    thread before any mbarrier is set up afresh."""
+    attn = _code("attn.cu")
+    body = attn[attn.index("auto next_unit"):attn.index("return true;")]
+    flag, inval = body.index("(&abort_flag)) return false;"), body.index("mbar_inval")
+    assert body.index("bar.sync 0") < flag < inval < body.rindex("bar.sync 0")
