@@ -42,7 +42,8 @@
 // The producer and issuer warps run warp-uniform code and elect one lane per instruction, so
 // that descriptors and addresses stay in uniform registers (a lone diverged thread issues
 // tcgen05.mma several times slower).  Every mbarrier wait is bounded; on a timeout the CTA raises
-// the error word, the remaining waits return at once, and the CTA runs out.
+// the error word, the remaining waits return at once, no further copy is sent for, and the CTA runs out; it leaves when
+// the copies and MMAs that were under way have ended.
 #include <mutex>
 
 #include "common.cuh"
@@ -641,6 +642,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ int k_stop, v_stop;                                 // the K and V tiles that were sent for before the CTA gave up
     __shared__ volatile int redo_flag;
     __shared__ float2 xchg[C::kTilesM][2 * kBlockM];
 
@@ -658,8 +660,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     bar.ke = bar.kf + 8 * C::kStagesK;
     bar.vf = bar.ke + 8 * C::kStagesK;
     bar.ve = bar.vf + 8 * C::kStagesV;
-    const uint32_t bar_copy = bar.ve + 8 * C::kStagesV;
-    static_assert(160 + 16 * (C::kStagesK + C::kStagesV) + 8 * C::kCopyStages <= C::kBarBytes, "barrier area too small");
+    const uint32_t bar_copy = bar.ve + 8 * C::kStagesV, bar_end = bar_copy + 8 * C::kCopyStages;
+    static_assert(160 + 16 * (C::kStagesK + C::kStagesV) + 8 * (C::kCopyStages + 2) <= C::kBarBytes, "barrier area too small");
 
     const int tid = threadIdx.x;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);        // warp-uniform
@@ -699,9 +701,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     };
     if (tid == 0) {
         abort_flag = 0;
+        k_stop = v_stop = 0x7fffffff;
         redo_flag = 0;
         init_query_bars();
-        for (int u = 0; u < C::kCopyStages; ++u) mbar_init(bar_copy + 8 * u, 1);
+        for (int u = 0; u < C::kCopyStages + 2; ++u) mbar_init(bar_copy + 8 * u, 1);       // (and bar_end)
         fence_barrier_init();
     }
     constexpr int kProducerWarp = C::kSoftmaxWarps, kIssuerWarp = C::kSoftmaxWarps + 1;
@@ -800,10 +803,15 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
         // ------------------------------------------------ TMA producer (warp-uniform, one elected lane issues)
         // g: running count of K (or V) tiles over all passes: stage g % kStages, phase (g / kStages) & 1
+        auto gave_up = [&] { return *static_cast<volatile int *>(&abort_flag) != 0; };
+        auto going = [&](int &stop, int g) -> bool {     // once the CTA has given up, tile g and those after it are not sent for
+            if (gave_up()) stop = min(stop, g);
+            return stop > g;
+        };
         auto load_k = [&](int g, int j) {
             const int st = g % C::kStagesK;
             wait_bar(bar.ke + 8 * st, ((g / C::kStagesK) & 1) ^ 1, &abort_flag, p.err_word);
-            if (elect_one()) {
+            if (elect_one() && going(k_stop, g)) {
                 mbar_arrive_expect_tx(bar.kf + 8 * st, C::kLoadBytes);
 #pragma unroll
                 for (int ch = 0; ch < C::kChunks; ++ch)
@@ -816,7 +824,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
         auto load_v = [&](int g, int j) {
             const int st = g % C::kStagesV;
             wait_bar(bar.ve + 8 * st, ((g / C::kStagesV) & 1) ^ 1, &abort_flag, p.err_word);
-            if (elect_one()) {
+            if (elect_one() && going(v_stop, g)) {
                 mbar_arrive_expect_tx(bar.vf + 8 * st, C::kLoadBytes);
 #pragma unroll
                 for (int ch = 0; ch < C::kChunks; ++ch)
@@ -846,10 +854,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
             k_loads = 3 * n_tiles; v_loads = 2 * n_tiles;
         }
         // every copy issued above must have landed before the CTA's shared memory is released
+        if (gave_up()) { __syncwarp(); k_loads = min(k_loads, k_stop); v_loads = min(v_loads, v_stop); }
         for (int g = (k_loads > C::kStagesK ? k_loads - C::kStagesK : 0); g < k_loads; ++g)
-            wait_bar(bar.kf + 8 * (g % C::kStagesK), (g / C::kStagesK) & 1, &abort_flag, p.err_word);
+            drain_bar(bar.kf + 8 * (g % C::kStagesK), (g / C::kStagesK) & 1);
         for (int g = (v_loads > C::kStagesV ? v_loads - C::kStagesV : 0); g < v_loads; ++g)
-            wait_bar(bar.vf + 8 * (g % C::kStagesV), (g / C::kStagesV) & 1, &abort_flag, p.err_word);
+            drain_bar(bar.vf + 8 * (g % C::kStagesV), (g / C::kStagesV) & 1);
         if constexpr (C::kPersistent) {          // nor may a commit still be on its way to a barrier that is set up afresh
             for (int g = (k_loads > C::kStagesK ? k_loads - C::kStagesK : 0); g < k_loads; ++g)
                 wait_bar(bar.ke + 8 * (g % C::kStagesK), (g / C::kStagesK) & 1, &abort_flag, p.err_word);
@@ -955,6 +964,13 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
 
     tc_fence_before();
     __syncthreads();
+    if (abort_flag) {                                // MMAs that are under way end before their memory is given up
+        if ((warp == kIssuerWarp || warp == kIssuerWarp + 1) && elect_one()) {
+            tc_commit(bar_end + 8 * (warp - kIssuerWarp));
+            drain_bar(bar_end + 8 * (warp - kIssuerWarp), 0);
+        }
+        __syncthreads();
+    }
     if (warp == kIssuerWarp) tmem_dealloc(tmem, kTmemCols);
 }
 

@@ -43,3 +43,33 @@ def test_a_cta_that_gave_up_takes_no_further_unit():
     body = attn[attn.index("auto next_unit"):attn.index("return true;")]
     flag, inval = body.index("(&abort_flag)) return false;"), body.index("mbar_inval")
     assert body.index("bar.sync 0") < flag < inval < body.rindex("bar.sync 0")
+
+
+def _bodies(code, head):
+    """The text of every block that starts with `head` (up to the brace that closes it)."""
+    out, at = [], code.find(head)
+    while at >= 0:
+        depth, i = 0, code.index("{", at + len(head) - 1)
+        start = i
+        while True:
+            depth += {"{": 1, "}": -1}.get(code[i], 0)
+            if depth == 0:
+                break
+            i += 1
+        out.append(code[start:i + 1])
+        at = code.find(head, i)
+    return out
+
+
+def test_an_attention_cta_that_gave_up_sends_for_nothing_and_leaves_with_nothing_under_way():
+    """Copies after the first tiles are sent for only while the CTA goes on; those that were sent are waited for without a look
+    at the abort flag; the MMAs under way are committed and waited for before tensor memory is freed."""
+    attn, wait = _code("attn.cu"), _code("bounded_wait.cuh")
+    assert "abort" not in wait[wait.index("void drain_bar"):]
+    for kv in "kv":
+        (load,) = _bodies(attn, "auto load_%s = [&](int g, int j) {" % kv)
+        assert load.index("wait_bar") < load.index("elect_one() && going(%s_stop, g)" % kv) < load.index("tma_load_4d")
+        assert re.search(r"%s_loads = min\(%s_loads, %s_stop\)" % (kv, kv, kv), attn)
+        assert "drain_bar(bar.%sf" % kv in attn
+    end = attn[attn.rindex("if (abort_flag) {"):]
+    assert end.index("tc_commit(bar_end") < end.index("drain_bar(bar_end") < end.index("__syncthreads()") < end.index("tmem_dealloc")
