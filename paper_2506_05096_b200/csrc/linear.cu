@@ -22,8 +22,9 @@
 //               and entries out of range are zero-filled); the copies arrive on the stage's barrier by themselves, so a
 //               thread never waits for its own copies, only for a free stage.  (TMA gather4, one per lane and stage, was
 //               measured at 331 us where this takes 119, 9001 x 3072 x 3072.)
-// Every mbarrier wait is bounded; on a timeout the CTA raises the error word, its remaining waits return at once, the
-// other CTA of the pair runs into its own limit, and both run out.
+// Every mbarrier wait is bounded; on a timeout the CTA raises the error word, its remaining waits return at once, it sends
+// for no further copy, the other CTA of the pair runs into its own limit, and both run out; they leave together, when the copies
+// and MMAs that were under way have ended.
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 #include "bounded_wait.cuh"
@@ -47,7 +48,7 @@ constexpr int kMaxBN = 256, kBNStep = 32;                // columns of an output
 constexpr int kStages = 6;
 constexpr int kABytes = kRowsCta * kBK * 2, kBBytes = kMaxBN / 2 * kBK * 2;
 constexpr int kBarBytes = 256;
-static_assert(8 * (3 * kStages + 2 * kAccSets) <= kBarBytes, "barrier area too small");
+static_assert(8 * (3 * kStages + 2 * kAccSets + 1) <= kBarBytes, "barrier area too small");
 constexpr int kSmemBytes = kStages * (kABytes + kBBytes) + kBarBytes + kEpiWarps * kEpiStageBytes + 1024;
 static_assert(kSmemBytes + 1536 <= 227 * 1024, "shared memory of one CTA");
 constexpr uint32_t kAccCols = kMaxBN, kTmemCols = kAccSets * kAccCols;
@@ -129,13 +130,15 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ int stop;                                           // the stages that were sent for before the CTA gave up
     __shared__ int row_list[2][kRowsCta];                          // listed rows only: the rows of x of a tile
 
     // (both CTAs of a pair run the same kernel with the same static shared memory, so every offset below is the same in both)
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sA = smem_base, sB = sA + kStages * kABytes, bars = sB + kStages * kBBytes;
     const uint32_t bar_full = bars, bar_empty = bars + 8 * kStages, bar_peer = bars + 16 * kStages,
-                   bar_acc_full = bars + 24 * kStages, bar_acc_empty = bar_acc_full + 8 * kAccSets;
+                   bar_acc_full = bars + 24 * kStages, bar_acc_empty = bar_acc_full + 8 * kAccSets,
+                   bar_end = bar_acc_empty + 8 * kAccSets;
 
     const int tid = threadIdx.x;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);        // warp-uniform
@@ -148,6 +151,8 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
 
     if (tid == 0) {
         abort_flag = 0;
+        stop = 0x7fffffff;
+        mbar_init(bar_end, 1);
         for (int s = 0; s < kStages; ++s) {
             // every gather thread + in the even CTA its TMA producer, for the bytes of both (odd CTA, contiguous rows: not used)
             mbar_init(bar_full + 8 * s, (DENSE ? 0 : kGatherWarps * 32) + (DENSE || rank == 0 ? 1 : 0));
@@ -294,13 +299,18 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
         // ------------------------------------------------ TMA producer of the W tiles (and of contiguous rows of x)
         // (the odd CTA's bytes may arrive before the even one has said how many a stage gets: its phase cannot end before that)
         const uint32_t full0 = map_to_rank(bar_full, 0);
+        auto gave_up = [&] { return *static_cast<volatile int *>(&abort_flag) != 0; };
+        auto going = [&](int g) -> bool {                          // once the CTA has given up, stage g and those after it are not sent for
+            if (gave_up()) stop = min(stop, g);
+            return stop > g;
+        };
         int g = 0;
         for (int tile = pair; tile < total_tiles; tile += n_pairs) {
             const int tm = tile / tiles_n, tn = tile - tm * tiles_n;
             for (int ks = 0; ks < k_steps; ++ks, ++g) {
                 const int st = g % kStages;
                 wait_bar(bar_empty + 8 * st, ((g / kStages) & 1) ^ 1, &abort_flag, p.err_word);
-                if (elect_one()) {
+                if (elect_one() && going(g)) {
                     if (rank == 0) mbar_arrive_expect_tx(bar_full + 8 * st, 2 * (p.bn * kBK + (DENSE ? kABytes : 0)));
                     tma_load_2d(sB + st * kBBytes, &tmap_w, full0 + 8 * st, ks * kBK, tn * p.bn + (int)rank * (p.bn / 2));
                     if (DENSE) tma_load_2d(sA + st * kABytes, &tmap_x, full0 + 8 * st, ks * kBK, tm * kBM + (int)rank * kRowsCta);
@@ -308,9 +318,11 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
                 __syncwarp();
             }
         }
-        // every copy issued above must have landed before either CTA's shared memory is released
+        // Every copy issued above must have landed before either CTA's shared memory is released.  (The odd CTA may be stages
+        // ahead of one that gave up; the wait for one stage more, which does not come, outlasts them.)
+        if (gave_up()) { __syncwarp(); g = min(g, stop) + 1; }
         for (int gs = (g > kStages ? g - kStages : 0); rank == 0 && gs < g; ++gs)
-            wait_bar(bar_full + 8 * (gs % kStages), (gs / kStages) & 1, &abort_flag, p.err_word);
+            drain_bar(bar_full + 8 * (gs % kStages), (gs / kStages) & 1);
     } else if (warp == kMmaWarp && rank == 0) {
         // ------------------------------------------------ MMA issuer of the pair
         const uint32_t idesc = idesc_bf16(kBM, p.bn, false);
@@ -400,6 +412,10 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
     // neither CTA leaves (or gives up its TMEM) while the other may still arrive on its barriers or read its shared memory
     tc_fence_before();
     __syncthreads();
+    if (abort_flag && rank == 0 && warp == kMmaWarp) {             // MMAs that are under way end before their memory is given up
+        if (elect_one()) { tc_commit_pair(bar_end); drain_bar(bar_end, 0); }
+        __syncwarp();
+    }
     cluster_sync_all();
     if (warp == kMmaWarp) tmem_dealloc_pair(tmem, kTmemCols);
 }

@@ -73,3 +73,12 @@ def test_an_attention_cta_that_gave_up_sends_for_nothing_and_leaves_with_nothing
         assert "drain_bar(bar.%sf" % kv in attn
     end = attn[attn.rindex("if (abort_flag) {"):]
     assert end.index("tc_commit(bar_end") < end.index("drain_bar(bar_end") < end.index("__syncthreads()") < end.index("tmem_dealloc")
+
+
+def test_a_gemm_pair_that_gave_up_sends_for_nothing_and_leaves_with_nothing_under_way():
+    lin = _code("linear.cu")
+    producer = lin[lin.index("const uint32_t full0"):lin.index("warp == kMmaWarp && rank == 0")]
+    assert producer.index("wait_bar(bar_empty") < producer.index("elect_one() && going(g)") < producer.index("tma_load_2d")
+    assert producer.index("min(g, stop)") < producer.index("drain_bar(bar_full") and "wait_bar(bar_full" not in producer
+    end = lin[lin.rindex("if (abort_flag && rank == 0"):]
+    assert end.index("tc_commit_pair(bar_end)") < end.index("drain_bar(bar_end") < end.index("cluster_sync_all()") < end.index("tmem_dealloc_pair")
