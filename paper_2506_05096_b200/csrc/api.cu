@@ -326,18 +326,14 @@ int32_t astraea_layernorm_modulate(const void *x, const int32_t *idx, int M, con
 }
 
 // ------------------------------------------------------------------ a whole compute block
-// workspace: [256 bytes: error word | the key shares of a split self-attention launch (room for gathered keys and values
-//             too)] [select scratch]
+// workspace: [256 bytes: error word | the key shares of a split self-attention launch] [select scratch]
 //            [5 token-sized buffers] [hidden-sized buffer]
-// (the first part is laid out as the workspace of astraea_sparse_attn with kv_idx, so that every call of the block
-// shares the one error word at the very start)
+// (the first part is laid out as the workspace of astraea_sparse_attn, so that every call of the block shares the one error
+// word at the very start)
 static size_t block_buffer_bytes(int B, int N, int width) { return align_up((size_t)B * N * width * 2, 256); }
-// the head of the block's workspace serves the self-attention: the key shares of a split launch
-static size_t block_attn_region_bytes(int B, int H, int N, int d)
-{
-    const size_t kv = attn_kv_workspace_bytes(B, H, N, d), plain = attn_workspace_bytes(B, H, N, N, d);
-    return align_up(kv > plain ? kv : plain, 256);
-}
+// the head of the block's workspace serves the self-attention: the key shares of a split launch (enough for every number of
+// queries, and of keys where SelectQ&K keeps only those of the selected tokens)
+static size_t block_attn_region_bytes(int B, int H, int N, int d) { return align_up(attn_workspace_bytes(B, H, N, N, d), 256); }
 
 size_t astraea_block_workspace_bytes(int B, int H, int N, int d, int hidden)
 {

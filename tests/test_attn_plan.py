@@ -49,6 +49,20 @@ def test_plan_invariants(d):
             assert _plan(B, H, N, M, d, flags=A.ATTN_SMALL_CTAS)["small_ctas"] == (d != 128)
 
 
+@pytest.mark.parametrize("B,H,N,d,hidden", [(1, 48, 17776, 64, 12288), (2, 16, 16384, 72, 4608), (1, 4, 300, 128, 512)])
+def test_block_workspace_holds_what_the_block_uses_and_no_more(B, H, N, d, hidden):
+    """The key shares of a split self-attention, the selection's scratch, five token-sized buffers and the hidden one; the room for
+    the shares is enough for the shorter key sequences of SelectQ&K too."""
+    up = lambda n: (n + 255) // 256 * 256  # noqa: E731
+    attn = up(A.astraea_workspace_bytes(A.OP_SPARSE_ATTN, B, H, N, N, d))
+    want = attn + up(A.astraea_workspace_bytes(A.OP_SELECT, B, H, N, N, d)) + 5 * up(B * N * H * d * 2) + up(B * N * hidden * 2)
+    assert A.astraea_block_workspace_bytes(B, H, N, d, hidden) == want
+    for M in (1, 257, N // 2, N - 1):
+        if M <= N:
+            assert A.astraea_workspace_bytes(A.OP_SPARSE_ATTN, B, H, M, M, d) <= attn
+            assert _plan(B, H, M, M, d, workspace_bytes=attn) == _plan(B, H, M, M, d)
+
+
 def test_plan_rejects_bad_arguments():
     with pytest.raises(A.AstraeaError) as e:
         _plan(1, 2, 100, 101, 64)
