@@ -214,7 +214,7 @@ def test_scatter_with_no_rows_leaves_cache_alone():
 
 # ------------------------------------------------------------------ attention
 def _attn_case(oracle, B, H, N, d, M, seed, layout="bnhd", compact=False, dense=False, scale=0.0, amp=1.0, small_ctas=False,
-               whole_keys=False, expect_split=None):
+               whole_keys=False, expect_split=None, lse_tol=None):
     rng = np.random.default_rng(seed)
     # amp sharpens the logits only (q, k); values and the cache stay N(0,1)
     q, k, v, cache = (synth.f32_to_bf16_bits((a * rng.standard_normal((B, N, H, d))).astype(np.float32)) for a in (amp, amp, 1.0, 1.0))
@@ -266,7 +266,8 @@ def _attn_case(oracle, B, H, N, d, M, seed, layout="bnhd", compact=False, dense=
     assert_attn_close(got_rows, want_o, ATTN_MAX_ABS, ATTN_MEAN_ABS)
     # head_dim 64 takes the row sums from the tensor core, i.e. of the bf16-rounded probabilities: where one key
     # dominates a row the LSE carries that rounding (2^-8 relative at worst); elsewhere it averages out
-    lse_tol = 5e-3 if (d == 64 and amp > 1.0) else LSE_ABS
+    if lse_tol is None:
+        lse_tol = 5e-3 if (d == 64 and amp > 1.0) else LSE_ABS
     assert np.abs(got_lse_rows - want_lse).max() < lse_tol, np.abs(got_lse_rows - want_lse).max()
 
 
@@ -908,17 +909,17 @@ def test_cross_attention_of_selected_rows(oracle, d, N_kv):
 
 
 # ------------------------------------------------------------------ small CTAs that walk over several units
-@pytest.mark.parametrize("H,N,M,amp", [(60, 700, 700, 1.0),      # three units a CTA, eleven key tiles
-                                       (50, 400, 390, 12.0),     # sharp logits: some units are redone, their neighbours not
-                                       # one key tile (the odd warpgroups have none); two, the second with one key.  A row sum
-                                       # of bf16-rounded probabilities is within 2^-9 of the exact one, so a row's LSE within
-                                       # 2.0e-3: with 40 keys the roundings do not average out to the 1e-3 of long rows, and
-                                       # amp > 1 selects the 5e-3 bound that such rows have elsewhere
-                                       (150, 40, 33, 1.01),
-                                       (160, 65, 65, 1.01)])
-def test_small_ctas_walk_over_units(oracle, H, N, M, amp):
+@pytest.mark.parametrize("H,N,M,amp,lse_tol", [(60, 700, 700, 1.0, None),      # three units a CTA, eleven key tiles
+                                               (50, 400, 390, 12.0, None),     # sharp logits: some units are redone, their neighbours not
+                                               # one key tile (the odd warpgroups have none); two, the second with one key.  The
+                                               # row sum of bf16-rounded probabilities is within 2^-9 of the exact one, so the
+                                               # LSE within 2.0e-3; over 40 keys the roundings do not average out to the 1e-3
+                                               # of long rows.  The cubic and fp32 add less than 1e-4 to that.
+                                               (150, 40, 33, 1.0, 2.1e-3),
+                                               (160, 65, 65, 1.0, 2.1e-3)])
+def test_small_ctas_walk_over_units(oracle, H, N, M, amp, lse_tol):
     """More units than the 296 slots of a B200's SMs, so that barriers, stages and TMEM are reused from unit to unit."""
-    _attn_case(oracle, 2, H, N, 64, M, seed=H + N, amp=amp, small_ctas=True)
+    _attn_case(oracle, 2, H, N, 64, M, seed=H + N, amp=amp, small_ctas=True, lse_tol=lse_tol)
 
 
 # ------------------------------------------------------------------ refresh of the reference inputs beside the attention
