@@ -9,11 +9,16 @@ One "step" is one pass of the whole path for one attention block at one keep-rat
 (`value`, `ms_per_step`, `roofline`, `e2e`, `cpu_baseline`) is the keep-ratio-sweep workload (24 heads,
 head_dim 128, 65536 tokens) at keep-ratio 0.5: `value` is the attention's algorithmic FLOPs (4*B*H*M*N*d)
 per second of whole-step time with the inputs resident in HBM; `e2e` is the same through astraea_step_host
-with pinned HOST buffers (host<->device copies inside the timed region).  The same line also carries
-`keep_ratio_sweep` (all twenty keep-ratios 0.05 .. 1.0 over ten seeds) and `workloads`: the CogVideoX-, Open-Sora-
-and HunyuanVideo-shaped configurations (the last one as 50 consecutive steps of a drifting latent after a dense
-step 0) and the tiny one, each with per-kernel times and roofline fractions, and `worst_attn_frac` /
-`worst_hbm_frac` over all of them.  Prints ONE JSON line on rank 0.
+with pinned HOST buffers (host<->device copies inside the timed region), `step_call` the same steps through the one
+call astraea_step, whose attention launch carries the reference refresh along.  Rank 0 prints ONE JSON line, kept
+short (a few lines of a terminal) so that whatever captures the output keeps all of it.
+
+The rest is one JSON object on standard error (or in the file that --details names): the headline's kernels in full,
+`keep_ratio_sweep` (all twenty keep-ratios 0.05 .. 1.0 over ten seeds), `workloads` (the CogVideoX-, Open-Sora- and
+HunyuanVideo-shaped configurations, the last one as 50 consecutive steps of a drifting latent after a dense step 0, and
+the tiny one, each with per-kernel times and roofline fractions), `block`, `model_schedules`, `next`, and what
+`worst_attn_frac` / `worst_hbm_frac` are the
+worst of.
 """
 from __future__ import annotations
 
@@ -151,6 +156,15 @@ def config_of(w, theta, world):
             "l2": "two alternating input sets, %.0f MB touched per step > 126 MB L2" % ((6 * w.B * w.N * w.D * 2) / 1e6)}
 
 
+def short(v):
+    """The line's numbers to six digits, but for the fractions, which have to be the quotients of what they are quotients of."""
+    if isinstance(v, dict):
+        return {k: (x if k in ("frac", "achieved", "peak") else short(x)) for k, x in v.items()}
+    if isinstance(v, list):
+        return [short(x) for x in v]
+    return float("%.6g" % v) if isinstance(v, float) else v
+
+
 def run_reference(args):
     rank = int(os.environ.get("RANK", "0"))
     if rank != 0:
@@ -260,6 +274,21 @@ class Block:
         A.astraea_scatter_reuse(self.x_ref, s["x_cur"], self.idx_sel, B, N, M, D, A.SCATTER_SRC_FULL, workspace=self.ws)
         if ev:
             ev[4].record()
+
+    def timed_step_call(self, k_keep, steps, barrier, warmup=3, t_base=1):
+        """Mean time of a step through astraea_step: the same work, the refresh of x_ref inside the attention launch."""
+        torch, A, w = self.torch, self.A, self.w
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        for t in range(warmup + steps):
+            if t == warmup:
+                barrier()
+                ev[0].record()
+            s = self.sets[(t_base + t) % len(self.sets)]
+            A.astraea_step(s["x_cur"], self.x_ref, self.lse, self.n_skip, s["q"], s["k"], s["v"], self.out, self.score, self.idx_sel,
+                           self.idx_rem, w.B, w.H, w.N, w.N_v, w.d, k_keep, self.w_alpha, 1.0, workspace=self.ws)
+        ev[1].record()
+        barrier()
+        return ev[0].elapsed_time(ev[1]) / steps
 
     def timed(self, k_keep, steps, warmup, barrier, t_base=1):
         """`steps` consecutive steps after `warmup` untimed ones; returns (total ms, median ms of each of the four calls
@@ -569,8 +598,8 @@ def model_leg(torch, A, w, theta, sampler, L=2, T=8, hidden_mult=4, N_text=226, 
     dense = out["schedules"]["dense"]["ms_per_generation"]
     for e in out["schedules"].values():
         e["speedup_vs_dense"] = dense / e["ms_per_generation"]
-    out["note"] = ("one graph launch per generation; SelectQ&K gathers the selected K / V rows in a pass of its own before the "
-                   "attention (twice the K / V bytes of those rows through HBM); Fixed-token scores and selects in block 0 only")
+    out["note"] = ("one graph launch per generation; SelectQ&K projects keys and values of the selected rows only, into compact "
+                   "buffers; Fixed-token scores and selects in block 0 only")
     return out
 
 
@@ -629,6 +658,7 @@ def main():
     ap.add_argument("--no-workloads", action="store_true", help="headline only")
     ap.add_argument("--no-next", action="store_true", help="skip the query projection of the selected rows (astraea_gathered_linear)")
     ap.add_argument("--no-model", action="store_true", help="skip the scheduled generations (astraea_model_schedule_*: 2 blocks x 8 steps, four variants); --no-block skips them too")
+    ap.add_argument("--details", default="", help="file for everything beside the headline (default: one JSON line on standard error)")
     ap.add_argument("--no-block", action="store_true", help="skip the whole-block leg (astraea_block_step on the CogVideoX shape)")
     args = ap.parse_args()
     if args.impl == "reference":
@@ -721,6 +751,7 @@ def main():
     total_ms, job_flops = replicas.aggregate(total_ms, flops * args.steps, device="cuda")
     ms_per_step = total_ms / args.steps
     value = replicas.throughput(job_flops, total_ms) / 1e12
+    call_ms = blk.timed_step_call(k_keep, args.steps, barrier) if extras else None
     pair_ms = blk.timed_pair(k_keep) if extras else None
     # the headline's roofline divides by the kernel's AVERAGE launch duration over the timed steps
     roofline, kernels = kernel_report(w, theta, all_parts.mean(axis=0), peaks, pair_ms=pair_ms, all_parts=all_parts, stat="mean")
@@ -876,19 +907,26 @@ def main():
     if rank == 0:
         worst_a = min(attn_fracs, key=attn_fracs.get)
         worst_h = min(hbm_fracs, key=hbm_fracs.get)
+        keep = ("ms", "GB/s", "TFLOP/s", "frac_hbm", "schedule")
+        brief = {n: {k: x for k, x in e.items() if k in keep} for n, e in kernels.items() if n != "hbm_peaks_gbs"}
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
                 "scaling": "weak", "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
                 "config": config_of(w, theta, world),
-                "gpu_launches": (3 + kernels["sparse_attn"]["schedule"]["launches"]) * args.steps, "clocks": clocks, "roofline": roofline, "kernels": kernels,
-                "worst_attn_frac": {"value": attn_fracs[worst_a], "where": worst_a, "of": "measured burst bf16",
-                                    "of_nominal_2250": attn_fracs[worst_a] * peaks["bf16_tflops"] / NOMINAL_BF16_TFLOPS,
-                                    "all": attn_fracs},
-                "worst_hbm_frac": {"value": hbm_fracs[worst_h], "where": worst_h, "of": "measured copy bandwidth",
-                                   "of_nominal_8000": hbm_fracs[worst_h] * peaks["hbm_gbs"] / NOMINAL_HBM_GBS, "all": hbm_fracs},
-                "keep_ratio_sweep": sweep, "workloads": workloads, "next": nxt, "block": block, "model_schedules": model, "e2e": e2e, "cpu_baseline": cpu,
-                "bench_seconds": time.perf_counter() - t_start}
-        print(json.dumps(line))
+                "gpu_launches": (3 + kernels["sparse_attn"]["schedule"]["launches"]) * args.steps, "clocks": clocks,
+                "roofline": {k: x for k, x in roofline.items() if not k.startswith("dense_equivalent")}, "kernels": brief,
+                "worst_attn_frac": {"value": attn_fracs[worst_a], "where": worst_a, "of": "measured burst bf16"},
+                "worst_hbm_frac": {"value": hbm_fracs[worst_h], "where": worst_h, "of": "measured copy bandwidth"},
+                "step_call": None if call_ms is None else {"ms_per_step": call_ms, "value": flops / (call_ms * 1e-3) / 1e12, "unit": UNIT},
+                "e2e": e2e, "cpu_baseline": cpu, "bench_seconds": time.perf_counter() - t_start}
+        details = {"headline": {"roofline": roofline, "kernels": kernels}, "keep_ratio_sweep": sweep, "workloads": workloads, "next": nxt, "block": block, "model_schedules": model,
+                   "attn_fracs": attn_fracs, "hbm_fracs": hbm_fracs}
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(details, f, indent=1)
+        else:
+            print(json.dumps(details), file=sys.stderr, flush=True)
+        print(json.dumps(short(line)))
     if world > 1:
         dist.destroy_process_group()
 
