@@ -74,6 +74,7 @@ constexpr uint32_t kGaveUpLse = 0xffc0dead;
 // one (head_dim 64 / 72 only) lets two CTAs share an SM, which costs ~5 % of throughput per SM but halves the
 // granularity of the schedule: launches of only a few rounds of CTAs are faster with it.
 template <int DH, int TM> struct Cfg {
+    static_assert(TM == 2 || DH != 128, "head_dim 128 needs the whole SM");
     static constexpr int kDH = DH;
     static constexpr int kTilesM = TM;
     static constexpr int kCtasPerSM = (TM == 1) ? 2 : 1;
@@ -103,8 +104,8 @@ template <int DH, int TM> struct Cfg {
     // launch, under the power cap: head_dim 64, 9001 x 17776 x 48 heads, 4 / 5 / 6 / 7 / 8 of 16: 2143 / 2123 / 2083 / 2140 /
     // 2203; 72, 2 x 6553 x 16384 x 16, 2 / 4 / 5 / 6 / 8: 1190 / 1150 / 1152 / 1165 / 1233).  None at 128, whose row sums are
     // fp32 sums of what the XU returns: a polynomial as exact as that (degree 5, the argument formed as for the XU) is
-    // slower than the XU in every share (0 / 1 / 2 / 3 of eight pairs: 3276 x 65536 x 24 heads 2128 / 2117 / 2149 / 2227,
-    // 35640 x 118800 x 24 40200 / 40300 / 40700 / 42300, 1132 x 3594 x 24 53.8 / 60 / 53.8 / 53.8).
+    // no faster than the XU in any share (0 / 1 / 2 / 3 of eight pairs: 3276 x 65536 x 24 heads 2128 / 2117 / 2149 / 2227,
+    // 35640 x 118800 x 24 40200 / 40300 / 40700 / 42300).
     static constexpr int kPolyPeriod = (DH == 72 && TM == 2) ? 4 : 8;
     static constexpr int kPolyPairs = (DH == 72) ? 1 : (DH == 64) ? 3 : 0;
     static constexpr int kSoftmaxWarps = 4 * kTilesM * kSplit;
@@ -1118,7 +1119,8 @@ int32_t launch_dh(const AttnArgs &a, cudaStream_t stream, SplitPlan plan = Split
     const int units_per_cta = C::kPersistent ? (int)((p.n_full + grid - 1) / grid) : 1;
     // The rows to copy go with the attention when its CTAs live long enough for their shares: 4 KB a microsecond against
     // 0.4 us a key tile and 4 us for a CTA's set-up and a launch less.  (Measured: a batch of 4 KB takes ~1.5 us with two or
-    // three of them in flight.)
+    // three of them in flight; a key tile 0.55 / 0.66 / 0.82 us at head_dim 64 / 72 / 128, twice that in a small CTA.  0.4
+    // stands for all of them and errs on the side of the scatter.)
     const long long copy_rows = (long long)a.B * a.M;
     const double copy_us = a.copy_dst ? (double)((copy_rows + grid - 1) / grid) * a.copy_elems * 2 / 4096 : 0.0;
     const bool copy_here = a.copy_dst && (long long)a.B * a.N_tok * (a.copy_elems / 8) < 0x7fffffffll && copy_us <= 0.4 * ((a.N + C::kBlockN - 1) / C::kBlockN) * units_per_cta / p.split + 4.0;

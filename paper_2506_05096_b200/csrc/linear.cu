@@ -81,7 +81,8 @@ __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
 
 // erf(x) to 1.5e-7 absolute (rational approximation 7.1.26 of Abramowitz and Stegun: 1 - (a1 t + ... + a5 t^5) e^{-x^2},
 // t = 1 / (1 + p |x|)): two XU operations and nine FMA-pipe ones without a branch, about half of erff()'s cost, which
-// counts because the epilogue of a tile is not hidden.  The result goes into a bf16 (2^-9 relative).
+// counts where the main loop of the next tile is too short to hide the epilogue of this one (K = 1152: 5 us).  The result goes
+// into a bf16 (2^-9 relative).
 __device__ __forceinline__ float erf_fast(float x) {
     const float ax = fabsf(x);
     float t, e;
