@@ -175,7 +175,8 @@ int32_t astraea_select(const float *score, int B, int N_sel, int k, int n_always
  *               in the workspace, which a second kernel merges (out = sum_i exp(lse_i - lse) out_i).  Results agree
  *               with the unsplit launch to fp32 rounding.  A workspace serves one call at a time.
  * Arithmetic: bf16 operands, fp32 logits, softmax and accumulation; probabilities are
- * rounded to bf16 before the P.V product; outputs rounded to bf16.
+ * rounded to bf16 before the P.V product; outputs rounded to bf16.  A logit of NaN or +inf makes
+ * its row NaN (out and lse); one of -inf has no weight.
  * M = 0 is valid: nothing is launched and the caches are untouched.
  * Errors: INVALID_ARG, UNSUPPORTED (d not in {64,72,128}), WORKSPACE_TOO_SMALL, CUDA.
  */
