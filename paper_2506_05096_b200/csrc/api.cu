@@ -271,10 +271,9 @@ int32_t astraea_scatter_reuse(void *cache, const void *rows, const int32_t *idx,
     return launch_scatter(cache, rows, idx, B, N, M, row_elems, flags, reinterpret_cast<int *>(err_workspace), (cudaStream_t)stream);
 }
 
-int32_t astraea_gathered_linear_residual(const void *x, const int32_t *idx, int M, const void *w, const void *bias,
-                                         const void *residual, const void *gate,
-                                         void *y, int B, int N, int K, int N_out, uint32_t flags,
-                                         void *workspace, size_t workspace_bytes, void *stream)
+static int32_t linear_entry(const void *x, const int32_t *idx, int M, const LinearLayer *layers, int n_layers,
+                            const void *residual, const void *gate, int B, int N, int K, int N_out, uint32_t flags,
+                            void *workspace, size_t workspace_bytes, void *stream)
 {
     REQUIRE(B > 0 && N > 0 && K > 0 && N_out > 0, "astraea_gathered_linear: B, N, K, N_out must be positive");
     REQUIRE(!idx || (M >= 0 && M <= N), "astraea_gathered_linear: M=%d outside [0, N=%d]", M, N);
@@ -290,11 +289,22 @@ int32_t astraea_gathered_linear_residual(const void *x, const int32_t *idx, int 
                     workspace_bytes, linear_workspace_bytes());
     REQUIRE((reinterpret_cast<uintptr_t>(workspace) & 255u) == 0, "astraea_gathered_linear: workspace must be 256-byte aligned");
     if (idx && M == 0) return ASTRAEA_OK;
-    REQUIRE(x && w && y, "astraea_gathered_linear: null x, w or y");
-    REQUIRE(aligned16(x) && aligned16(w) && aligned16(y) && aligned16(bias) && aligned16(residual) && aligned16(gate),
-            "astraea_gathered_linear: x, w, bias, residual, gate, y must be 16-byte aligned");
-    return launch_gathered_linear(x, idx, M, w, bias, y, B, N, K, N_out, flags, reinterpret_cast<int *>(workspace),
+    for (int i = 0; i < n_layers; ++i) {
+        REQUIRE(x && layers[i].w && layers[i].y, "astraea_gathered_linear: null x, w or y");
+        REQUIRE(aligned16(x) && aligned16(layers[i].w) && aligned16(layers[i].y) && aligned16(layers[i].bias) && aligned16(residual) && aligned16(gate),
+                "astraea_gathered_linear: x, w, bias, residual, gate, y must be 16-byte aligned");
+    }
+    return launch_gathered_linear(x, idx, M, layers, n_layers, B, N, K, N_out, flags, reinterpret_cast<int *>(workspace),
                                   (cudaStream_t)stream, residual, gate);
+}
+
+int32_t astraea_gathered_linear_residual(const void *x, const int32_t *idx, int M, const void *w, const void *bias,
+                                         const void *residual, const void *gate,
+                                         void *y, int B, int N, int K, int N_out, uint32_t flags,
+                                         void *workspace, size_t workspace_bytes, void *stream)
+{
+    const LinearLayer layer = {w, bias, y, (flags & ASTRAEA_LINEAR_COMPACT_OUT) != 0};
+    return linear_entry(x, idx, M, &layer, 1, residual, gate, B, N, K, N_out, flags, workspace, workspace_bytes, stream);
 }
 
 int32_t astraea_gathered_linear(const void *x, const int32_t *idx, int M, const void *w, const void *bias,
@@ -385,12 +395,11 @@ int32_t astraea_block_step(const void *x, const astraea_block_weights *w, const 
     const int64_t tsb = (int64_t)N_text * D;
     // self-attention group: keys / values from all tokens, everything else on the selected rows
     rc = astraea_layernorm_modulate(x, nullptr, 0, w->s1, w->t1, bufA, B, N, D, eps, 0u, err, stream);
-    // (SelectQ&K: keys and values of the selected tokens only, so only their rows are projected, into compact buffers)
-    const int32_t *kv_rows = select_qk ? idx_sel : nullptr;
-    const uint32_t kv_flags = select_qk ? ASTRAEA_LINEAR_COMPACT_OUT : 0u;
-    if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, kv_rows, M, w->wk, w->bk, bufK, B, N, D, D, kv_flags, err, 256, stream);
-    if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, kv_rows, M, w->wv, w->bv, bufV, B, N, D, D, kv_flags, err, 256, stream);
-    if (rc == ASTRAEA_OK) rc = astraea_gathered_linear(bufA, idx_sel, M, w->wq, w->bq, bufQ, B, N, D, D, 0u, err, 256, stream);
+    // Layers of the same rows go in one launch: the key and value projections of all tokens, or (SelectQ&K: keys and values of the
+    // selected tokens only, into compact buffers) those and the query projection.
+    const LinearLayer qkv[3] = {{w->wk, w->bk, bufK, select_qk}, {w->wv, w->bv, bufV, select_qk}, {w->wq, w->bq, bufQ, false}};
+    if (rc == ASTRAEA_OK) rc = linear_entry(bufA, select_qk ? idx_sel : nullptr, M, qkv, select_qk ? 3 : 2, nullptr, nullptr, B, N, D, D, 0u, err, 256, stream);
+    if (rc == ASTRAEA_OK && !select_qk) rc = linear_entry(bufA, idx_sel, M, qkv + 2, 1, nullptr, nullptr, B, N, D, D, 0u, err, 256, stream);
     // the reference inputs of the tokens that were computed become the current inputs, under the attention where they can
     const size_t xb = (size_t)B * N * D * 2, lb = (size_t)B * H * N * 4, txb = (size_t)B * N_text * D * 2;
     const bool refresh = !(flags & ASTRAEA_BLOCK_REUSE_SELECTION);

@@ -103,7 +103,10 @@ int32_t launch_scatter(void *cache, const void *rows, const int32_t *idx, int B,
                        int row_elems, uint32_t flags, int *err_word, cudaStream_t stream, int pitch_elems = 0);   // pitch 0: rows are dense
 
 size_t linear_workspace_bytes();
-int32_t launch_gathered_linear(const void *x, const int32_t *idx, int M, const void *w, const void *bias, void *y,
+// Up to three linear layers [N_out, K] of the same rows of x in one launch, each with an output of its own ([B, N, N_out], or
+// compact [B, M, N_out]); GELU, residual and gate only with one layer (its output is compact as compact_out says).
+struct LinearLayer { const void *w, *bias; void *y; bool compact_out; };
+int32_t launch_gathered_linear(const void *x, const int32_t *idx, int M, const LinearLayer *layers, int n_layers,
                                int B, int N, int K, int N_out, uint32_t flags, int *err_word, cudaStream_t stream,
                                const void *residual = nullptr, const void *gate = nullptr);
 int32_t launch_layernorm_modulate(const void *x, const int32_t *idx, int M, const void *scale, const void *shift, void *y,

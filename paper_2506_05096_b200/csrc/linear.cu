@@ -22,6 +22,11 @@
 //               and entries out of range are zero-filled); the copies arrive on the stage's barrier by themselves, so a
 //               thread never waits for its own copies, only for a free stage.  (TMA gather4, one per lane and stage, was
 //               measured at 331 us where this takes 119, 9001 x 3072 x 3072.)
+// Layers of the same rows (the key and value projections; with SelectQ&K the query projection, too) share one launch: their column
+// tiles follow one another, so that one partial round of tiles is paid instead of two or three, the rows of x are read once for all, and
+// a launch is saved (7 us of set-up, first loads and last epilogue).  A block of 4276 tokens x 1536 channels: 44 us for two launches of
+// 102 tiles on 74 pairs, 38 for one of 204; four such blocks 1070 -> 1047 us; 32768 x 1152 twice, the Open-Sora block: 1863 ->
+// 1840; 17776 x 3072 twice, the CogVideoX block: 4469 -> 4434.
 // Every mbarrier wait is bounded; on a timeout the CTA raises the error word, its remaining waits return at once, it sends
 // for no further copy, the other CTA of the pair runs into its own limit, and both run out; they leave together, when the copies
 // and MMAs that were under way have ended.
@@ -51,17 +56,21 @@ constexpr int kBarBytes = 256;
 static_assert(8 * (3 * kStages + 2 * kAccSets + 1) <= kBarBytes, "barrier area too small");
 constexpr int kSmemBytes = kStages * (kABytes + kBBytes) + kBarBytes + kEpiWarps * kEpiStageBytes + 1024;
 static_assert(kSmemBytes + 1536 <= 227 * 1024, "shared memory of one CTA");
+constexpr int kMaxMats = 3;
 constexpr uint32_t kAccCols = kMaxBN, kTmemCols = kAccSets * kAccCols;
 
 struct LinParams {
     const __nv_bfloat16 *x;
     const int32_t *idx;
     int M;                       // rows listed per batch element (N when idx == nullptr)
-    const __nv_bfloat16 *bias;
-    __nv_bfloat16 *y;
+    // Up to kMaxMats layers of the same rows in one launch: the column tiles run over the matrices one after the other, each
+    // padded to mat_cols columns, a multiple of half a tile, so that each CTA's half of a W tile comes from one matrix.
+    int n_mats, mat_cols;
+    const __nv_bfloat16 *bias[kMaxMats];
+    __nv_bfloat16 *y[kMaxMats];
     int B, N, K, N_out;
     int bn;                      // columns of an output tile
-    int compact;                 // y is [B, M, N_out]
+    uint32_t compact;            // bit i: y[i] is [B, M, N_out]
     int compact_in;              // x is [B, M, K]
     int gelu;                    // y = GELU(x W^T + bias), exact (erf) form
     const __nv_bfloat16 *residual;   // added to the result after the gate; [B, N, N_out] rows at idx, or compact [B, M, N_out]
@@ -103,30 +112,34 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *m, 
         ::"r"(dst), "l"(m), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
 
-// The g-th listed row (all batch elements in one list): *out_row is the row of y it goes to, *res_row the row of the
-// residual, *batch the batch element.  False past the end of the list and for an index outside [0, N) or one that does
-// not exceed its predecessor (*bad).
-__device__ __forceinline__ bool target_row(const LinParams &p, long long g, long long total, long long *out_row,
-                                           long long *res_row, int *batch, bool *bad) {
+// The g-th listed row (all batch elements in one list): its row of a [B, N, *] tensor, or -1 past the end of the list and for an
+// index outside [0, N) or one that does not exceed its predecessor (*bad); *batch: the batch element.
+__device__ __forceinline__ long long target_row(const LinParams &p, long long g, long long total, int *batch, bool *bad) {
     *bad = false;
-    if (g >= total) return false;
+    if (g >= total) return -1;
     const int b = (int)((unsigned)g / (unsigned)p.M), r = (int)((unsigned)g - (unsigned)b * (unsigned)p.M);   // fewer than 2^31 rows fit the device
     const int tok = p.idx ? __ldcg(p.idx + g) : r;
     const int before = (p.idx && r > 0) ? __ldcg(p.idx + g - 1) : -1;
     // not strictly ascending: a row would be written twice
-    if ((unsigned)tok >= (unsigned)p.N || (r > 0 && before >= tok)) { *bad = true; return false; }
-    *out_row = p.compact ? g : (long long)b * p.N + tok;
-    *res_row = p.res_compact ? g : (long long)b * p.N + tok;
+    if ((unsigned)tok >= (unsigned)p.N || (r > 0 && before >= tok)) { *bad = true; return -1; }
     *batch = b;
-    return true;
+    return (long long)b * p.N + tok;
 }
 
-// DENSE: the rows of x are one contiguous matrix
+// the matrix that column c of the launch belongs to (the last one for what is left of a last tile)
+template <bool MULTI> __device__ __forceinline__ int mat_of(const LinParams &p, int c) {
+    return MULTI ? min(c / p.mat_cols, p.n_mats - 1) : 0;
+}
+
+struct WMaps { CUtensorMap m[kMaxMats]; };
+
+// DENSE: the rows of x are one contiguous matrix; MULTI: more than one layer (the registers of the listed form do not hold the
+// choice between one and several)
 template <bool DENSE> constexpr int kThreads = (kEpiWarps + 2 + (DENSE ? 0 : kGatherWarps)) * 32;
 
-template <bool DENSE>
+template <bool DENSE, bool MULTI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads<DENSE>, 1)
-gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x, const LinParams p)
+gathered_linear_kernel(const __grid_constant__ WMaps tmap_w, const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ LinParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t tmem_slot;
@@ -147,7 +160,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
     const uint32_t rank = cluster_ctarank();
     const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const long long total_rows = (long long)p.B * p.M;
-    const int tiles_m = (int)((total_rows + kBM - 1) / kBM), tiles_n = (p.N_out + p.bn - 1) / p.bn;
+    const int tiles_m = (int)((total_rows + kBM - 1) / kBM), tiles_n = ((MULTI ? p.n_mats * p.mat_cols : p.N_out) + p.bn - 1) / p.bn;
     const int total_tiles = tiles_m * tiles_n, k_steps = p.K / kBK;
 
     if (tid == 0) {
@@ -163,7 +176,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
         for (int a = 0; a < kAccSets; ++a) { mbar_init(bar_acc_full + 8 * a, 1); mbar_init(bar_acc_empty + 8 * a, 2 * kEpiWarps); }
         fence_barrier_init();
     }
-    if (warp == kTmaWarp && elect_one()) { prefetch_tensormap(&tmap_w); if (DENSE) prefetch_tensormap(&tmap_x); }
+    if (warp == kTmaWarp && elect_one()) { for (int i = 0; i < (MULTI ? p.n_mats : 1); ++i) prefetch_tensormap(&tmap_w.m[i]); if (DENSE) prefetch_tensormap(&tmap_x); }
     if (warp == kMmaWarp) {
         tmem_alloc_pair(smem_u32(&tmem_slot), kTmemCols);
         tmem_relinquish_pair();
@@ -186,18 +199,16 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
         int it = 0;
         for (int tile = pair; tile < total_tiles; tile += n_pairs, ++it) {
             const int tm = tile / tiles_n, tn = tile - tm * tiles_n;
-            const int acc = it % kAccSets, n0 = tn * p.bn;
-            long long out_row = -1, res_row = -1;
+            const int acc = it % kAccSets;
             int batch = 0;
             bool bad;
-            target_row(p, (long long)tm * kBM + row, total_rows, &out_row, &res_row, &batch, &bad);
+            long long full_row = target_row(p, (long long)tm * kBM + row, total_rows, &batch, &bad);
             if (bad && tn == 0 && part == 0) atomicExch(p.err_word, kErrBadIndex);
-            if (!p.residual) res_row = -1;
             const __nv_bfloat16 *gate = p.gate ? p.gate + (long long)batch * p.N_out : nullptr;
             wait_bar(bar_acc_full + 8 * acc, (it / kAccSets) & 1, &abort_flag, p.err_word);
             if (tile + n_pairs >= total_tiles) grid_launch_dependents();       // the last epilogue of this CTA
             tc_fence_after();
-            if (abort_flag) out_row = -1;
+            if (abort_flag) full_row = -1;
             auto release = [&] {                                   // this warp's part of the accumulator has been read
                 tc_fence_before();
                 __syncwarp();
@@ -212,9 +223,15 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
             const int q = lane & 3;
 #pragma unroll 1
             for (int c = c0; c < p.bn; c += 32 * kEpiSplit) {
-                const int colq = n0 + c + q * 8;                    // the 8 columns this lane moves
+                const int mat = mat_of<MULTI>(p, tn * p.bn + c), n0 = tn * p.bn + c - mat * p.mat_cols;     // 32 columns of one matrix from n0
+                const __nv_bfloat16 *bias = p.bias[mat];
+                __nv_bfloat16 *y = p.y[mat];
+                // the row of a compact tensor is the row of the list
+                const long long out_row = (full_row >= 0 && (p.compact >> mat & 1u)) ? (long long)tm * kBM + row : full_row;
+                const int colq = n0 + q * 8;                        // the 8 columns this lane moves
                 uint32_t rw[16];                                    // this thread's row of the residual: 32 bf16
-                if (p.residual) {
+                if (!MULTI && p.residual) {
+                    const long long res_row = (full_row >= 0 && p.res_compact) ? (long long)tm * kBM + row : full_row;
                     uint4 rr[4];
 #pragma unroll
                     for (int jj = 0; jj < 4; ++jj) {
@@ -242,13 +259,13 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
                 if (c + 32 * kEpiSplit >= p.bn) release();
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
-                    const int col = n0 + c + v * 8;
+                    const int col = n0 + v * 8;
                     float f[8];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(o[v * 8 + i]);
                     if (col < p.N_out) {                 // N_out is a multiple of 8; columns past it are never stored
-                        if (p.bias) {
-                            const uint4 bb = ld_cached(reinterpret_cast<const uint4 *>(p.bias + col));
+                        if (bias) {
+                            const uint4 bb = ld_cached(reinterpret_cast<const uint4 *>(bias + col));
                             const uint32_t bw[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
@@ -256,11 +273,11 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
                                 f[2 * i + 1] += __uint_as_float(bw[i] & 0xffff0000u);
                             }
                         }
-                        if (p.gelu) {
+                        if (!MULTI && p.gelu) {
 #pragma unroll
                             for (int i = 0; i < 8; ++i) f[i] = 0.5f * f[i] * (1.0f + erf_fast(f[i] * 0.70710678118654752f));
                         }
-                        if (gate) {
+                        if (!MULTI && gate) {
                             const uint4 gg = ld_cached(reinterpret_cast<const uint4 *>(gate + col));
                             const uint32_t gw[4] = {gg.x, gg.y, gg.z, gg.w};
 #pragma unroll
@@ -269,7 +286,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
                                 f[2 * i + 1] *= __uint_as_float(gw[i] & 0xffff0000u);
                             }
                         }
-                        if (p.residual) {
+                        if (!MULTI && p.residual) {
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
                                 f[2 * i] += __uint_as_float(rw[4 * v + i] << 16);
@@ -291,7 +308,7 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
                     const int r = (lane >> 2) + 8 * jj;
                     const long long orow = __shfl_sync(0xffffffffu, out_row, r);
                     const uint4 t = *reinterpret_cast<const uint4 *>(stage + r * 64 + ((q ^ ((r >> 1) & 3)) << 4));
-                    if (orow >= 0 && colq < p.N_out) *reinterpret_cast<uint4 *>(p.y + orow * p.N_out + colq) = t;
+                    if (orow >= 0 && colq < p.N_out) *reinterpret_cast<uint4 *>(y + orow * p.N_out + colq) = t;
                 }
                 __syncwarp();
             }
@@ -308,12 +325,13 @@ gathered_linear_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
         int g = 0;
         for (int tile = pair; tile < total_tiles; tile += n_pairs) {
             const int tm = tile / tiles_n, tn = tile - tm * tiles_n;
+            const int col = tn * p.bn + (int)rank * (p.bn / 2), mat = mat_of<MULTI>(p, col);           // this CTA's half of the W tile
             for (int ks = 0; ks < k_steps; ++ks, ++g) {
                 const int st = g % kStages;
                 wait_bar(bar_empty + 8 * st, ((g / kStages) & 1) ^ 1, &abort_flag, p.err_word);
                 if (elect_one() && going(g)) {
                     if (rank == 0) mbar_arrive_expect_tx(bar_full + 8 * st, 2 * (p.bn * kBK + (DENSE ? kABytes : 0)));
-                    tma_load_2d(sB + st * kBBytes, &tmap_w, full0 + 8 * st, ks * kBK, tn * p.bn + (int)rank * (p.bn / 2));
+                    tma_load_2d(sB + st * kBBytes, &tmap_w.m[mat], full0 + 8 * st, ks * kBK, col - mat * p.mat_cols);
                     if (DENSE) tma_load_2d(sA + st * kABytes, &tmap_x, full0 + 8 * st, ks * kBK, tm * kBM + (int)rank * kRowsCta);
                 }
                 __syncwarp();
@@ -441,57 +459,62 @@ int32_t make_matrix_map(CUtensorMap *map, const void *base, long long rows, int 
     return ASTRAEA_OK;
 }
 
-template <bool DENSE>
-int32_t launch_linear(const LinParams &p, const void *x, const void *w, int pairs, cudaStream_t stream)
-{
-    CUtensorMap mw, mx;
-    int32_t rc = make_matrix_map(&mw, w, p.N_out, p.K, p.bn / 2, "W");
-    if (rc != ASTRAEA_OK) return rc;
-    mx = mw;
-    if (DENSE) rc = make_matrix_map(&mx, x, (long long)p.B * p.M, p.K, kRowsCta, "x");
-    if (rc != ASTRAEA_OK) return rc;
-    static PerDeviceOnce attrs;                   // the attribute is per device
-    if (attrs.run([] { return cudaFuncSetAttribute(gathered_linear_kernel<DENSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes); }) != cudaSuccess)
-        return check_launch("astraea_gathered_linear (shared memory attribute)");
-    const long long tiles = (((long long)p.B * p.M + kBM - 1) / kBM) * ((p.N_out + p.bn - 1) / p.bn);
-    const int grid = 2 * (int)(tiles < pairs ? tiles : pairs);
-    launch_overlapped(gathered_linear_kernel<DENSE>, grid, kThreads<DENSE>, kSmemBytes, stream, mw, mx, p);
-    return check_launch("astraea_gathered_linear");
-}
+// Columns that a matrix takes in a launch over n_mats of them, and the column tiles of the launch.
+int mat_columns(int N_out, int n_mats, int bn) { return n_mats == 1 ? 0 : (N_out + bn / 2 - 1) / (bn / 2) * (bn / 2); }
+int column_tiles(int N_out, int n_mats, int bn) { return ((n_mats == 1 ? N_out : n_mats * mat_columns(N_out, n_mats, bn)) + bn - 1) / bn; }
 
 // Columns of an output tile.  The launch takes ceil(tiles / pairs) rounds, and a round of narrower tiles costs less, but
 // not in proportion (the rows of x are streamed for fewer columns): measured 0.60-0.67 of a 256-column round at 128
 // columns on seven shapes.  256 unless another width saves 3 % by that estimate, which happens where a launch has a
-// few rounds only or the last tile of a row is mostly padding.
-int choose_bn(long long rows, int N_out, int pairs)
+// few rounds only or the last tile of a row is mostly padding.  Several matrices: half a tile is whole groups of 32 columns, since
+// the epilogue's groups must not straddle two matrices.
+int choose_bn(long long rows, int N_out, int n_mats, int pairs)
 {
     const long long tiles_m = (rows + kBM - 1) / kBM;
     int best_bn = kMaxBN;
     double best = 0.0;
-    for (int bn = kMaxBN; bn >= kBNStep; bn -= kBNStep) {
-        const long long tiles = tiles_m * ((N_out + bn - 1) / bn);
+    for (int bn = kMaxBN; bn >= kBNStep; bn -= n_mats == 1 ? kBNStep : 64) {
+        const long long tiles = tiles_m * column_tiles(N_out, n_mats, bn);
         const double t = (double)((tiles + pairs - 1) / pairs) * (0.26 + 0.74 * bn / kMaxBN);
         if (best == 0.0 || t < 0.97 * best) { best = t; best_bn = bn; }
     }
     return best_bn;
 }
 
+template <bool DENSE, bool MULTI>
+int32_t launch_linear(const LinParams &p, const void *x, const LinearLayer *layers, int pairs, cudaStream_t stream)
+{
+    WMaps mw;
+    CUtensorMap mx;
+    int32_t rc = ASTRAEA_OK;
+    for (int i = 0; i < p.n_mats && rc == ASTRAEA_OK; ++i) rc = make_matrix_map(&mw.m[i], layers[i].w, p.N_out, p.K, p.bn / 2, "W");
+    if (rc != ASTRAEA_OK) return rc;
+    for (int i = p.n_mats; i < kMaxMats; ++i) mw.m[i] = mw.m[0];
+    mx = mw.m[0];
+    if (DENSE) rc = make_matrix_map(&mx, x, (long long)p.B * p.M, p.K, kRowsCta, "x");
+    if (rc != ASTRAEA_OK) return rc;
+    static PerDeviceOnce attrs;                   // the attribute is per device
+    if (attrs.run([] { return cudaFuncSetAttribute(gathered_linear_kernel<DENSE, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes); }) != cudaSuccess)
+        return check_launch("astraea_gathered_linear (shared memory attribute)");
+    const long long tiles = (((long long)p.B * p.M + kBM - 1) / kBM) * column_tiles(p.N_out, p.n_mats, p.bn);
+    const int grid = 2 * (int)(tiles < pairs ? tiles : pairs);
+    launch_overlapped(gathered_linear_kernel<DENSE, MULTI>, grid, kThreads<DENSE>, kSmemBytes, stream, mw, mx, p);
+    return check_launch("astraea_gathered_linear");
+}
+
 }  // namespace
 
 size_t linear_workspace_bytes() { return 256; }
 
-int32_t launch_gathered_linear(const void *x, const int32_t *idx, int M, const void *w, const void *bias, void *y,
+int32_t launch_gathered_linear(const void *x, const int32_t *idx, int M, const LinearLayer *layers, int n_layers,
                                int B, int N, int K, int N_out, uint32_t flags, int *err_word, cudaStream_t stream,
                                const void *residual, const void *gate)
 {
-    LinParams p;
+    LinParams p = {};
     p.x = reinterpret_cast<const __nv_bfloat16 *>(x);
     p.idx = idx;
     p.M = idx ? M : N;
-    p.bias = reinterpret_cast<const __nv_bfloat16 *>(bias);
-    p.y = reinterpret_cast<__nv_bfloat16 *>(y);
     p.B = B; p.N = N; p.K = K; p.N_out = N_out;
-    p.compact = (flags & ASTRAEA_LINEAR_COMPACT_OUT) ? 1 : 0;
     p.compact_in = (flags & ASTRAEA_LINEAR_COMPACT_IN) ? 1 : 0;
     p.gelu = (flags & ASTRAEA_LINEAR_GELU) ? 1 : 0;
     p.residual = reinterpret_cast<const __nv_bfloat16 *>(residual);
@@ -499,9 +522,16 @@ int32_t launch_gathered_linear(const void *x, const int32_t *idx, int M, const v
     p.gate = reinterpret_cast<const __nv_bfloat16 *>(gate);
     p.err_word = err_word;
     const int pairs = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
-    p.bn = choose_bn((long long)B * p.M, N_out, pairs);
-    if (!idx || p.compact_in) return launch_linear<true>(p, x, w, pairs, stream);
-    return launch_linear<false>(p, x, w, pairs, stream);
+    p.n_mats = n_layers;
+    p.bn = choose_bn((long long)B * p.M, N_out, n_layers, pairs);
+    p.mat_cols = mat_columns(N_out, n_layers, p.bn);
+    for (int i = 0; i < n_layers; ++i) {
+        p.bias[i] = reinterpret_cast<const __nv_bfloat16 *>(layers[i].bias);
+        p.y[i] = reinterpret_cast<__nv_bfloat16 *>(layers[i].y);
+        if (layers[i].compact_out) p.compact |= 1u << i;
+    }
+    if (!idx || p.compact_in) return n_layers > 1 ? launch_linear<true, true>(p, x, layers, pairs, stream) : launch_linear<true, false>(p, x, layers, pairs, stream);
+    return n_layers > 1 ? launch_linear<false, true>(p, x, layers, pairs, stream) : launch_linear<false, false>(p, x, layers, pairs, stream);
 }
 
 }  // namespace astraea
