@@ -452,7 +452,9 @@ void    astraea_schedule_destroy(astraea_schedule *schedule);
  * sparse attention) and copies the merged output back.  The copies run on streams of
  * their own: x_cur goes first, q / k / v follow in up to twelve groups of heads, the attention
  * of a group starts when its heads have arrived, and the group's columns of the output
- * go back while the next group is computed.  The results are those of astraea_step.
+ * go back while the next group is computed.  A step that computes every token and is bound by the bus moves whole rows
+ * instead: k and v, then q in chunks of rows, a chunk's attention and its way back under the next ones, x_cur last.
+ * The results are those of astraea_step.
  * astraea_session_create allocates device memory (cudaMalloc) on the current device;
  * the first step of a session must be run with k_keep = N_sel (all tokens computed) to
  * fill the caches, as the paper's denoising loop does at its first timestep.

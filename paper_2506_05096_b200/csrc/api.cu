@@ -757,6 +757,69 @@ int32_t astraea_session_create(astraea_session **session, int B, int H, int N, i
 
 size_t astraea_session_last_h2d_bytes(const astraea_session *s) { return s ? s->last_h2d_bytes : 0; }
 
+// A step that computes every token and is bound by the bus.  Nothing depends on its scores: all tokens are selected, their
+// counters become 0 and x_cur becomes the reference input, so it goes straight to its place, last.  Whole rows cross the bus (column
+// slices of 144 / 288 bytes a row run at 32 / 42 GB/s, whole rows at 51): k and v of a batch element, then its q in chunks of
+// rows; a chunk's attention runs while the next ones arrive, alternately on two streams (see astraea_session), and its rows of the
+// output go back while the next one is computed.  (B1 H16 d72 N 16384: 4.66 -> 3.02 ms, of which the bus is 3.0; twelve smaller
+// steps of 0.1 to 1.7 ms are 1.05 to 2.2 times as fast.)
+static int32_t step_host_all_rows(astraea_session *s, const void *x_cur, const void *q, const void *k, const void *v, void *out)
+{
+    const int B = s->B, H = s->H, N = s->N, d = s->d, D = H * d;
+    const size_t row = (size_t)D * 2, one = (size_t)N * row;
+    // chunks of at least 1 MB and whole units of 256 queries, up to kHostGroups in all
+    const int most = kHostGroups / B, want = (int)(one >> 20) < 1 ? 1 : (int)(one >> 20);
+    const int chunks = want < most ? want : most, step = ((N + chunks - 1) / chunks + 255) / 256 * 256;
+    auto at = [](const void *p, size_t bytes) { return static_cast<const char *>(p) + bytes; };
+    auto mut = [](void *p, size_t bytes) { return static_cast<char *>(p) + bytes; };
+    cudaError_t e = cudaMemsetAsync(s->n_skip, 0, (size_t)B * s->N_sel * 4, s->copy_in);
+    for (int b = 0, g = 0; b < B; ++b) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(mut(s->k, b * one), at(k, b * one), one, cudaMemcpyHostToDevice, s->copy_in);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(mut(s->v, b * one), at(v, b * one), one, cudaMemcpyHostToDevice, s->copy_in);
+        for (int r = 0; r < N; r += step, ++g) {
+            const int n = N - r < step ? N - r : step;
+            const size_t off = b * one + r * row;
+            cudaStream_t cs = (g & 1) ? s->stream2 : s->stream;
+            if (e == cudaSuccess) e = cudaMemcpyAsync(mut(s->q, off), at(q, off), n * row, cudaMemcpyHostToDevice, s->copy_in);
+            if (e == cudaSuccess) e = cudaEventRecord(s->ev_in[g], s->copy_in);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, s->ev_in[g], 0);
+            if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy in): %s", cudaGetErrorString(e));
+            AttnArgs a;
+            a.q = mut(s->q, off); a.k = mut(s->k, b * one); a.v = mut(s->v, b * one);
+            a.q_sb = a.k_sb = a.v_sb = (int64_t)N * D;
+            a.q_sh = a.k_sh = a.v_sh = d;
+            a.q_sn = a.k_sn = a.v_sn = D;
+            a.q_idx = nullptr; a.M = n; a.out = mut(s->out_cache, off); a.lse_out = s->lse_cache + (size_t)b * H * N + r;
+            a.B = 1; a.H = H; a.N = N; a.d = d; a.N_tok = N;
+            a.scale = 1.0f / sqrtf((float)d);
+            a.flags = 0;
+            a.err_word = reinterpret_cast<int *>(s->workspace);
+            const int32_t rc = launch_sparse_attn(a, cs);
+            if (rc != ASTRAEA_OK) return rc;
+            e = cudaEventRecord(s->ev_attn[g], cs);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s->copy_out, s->ev_attn[g], 0);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(mut(out, off), at(s->out_cache, off), n * row, cudaMemcpyDeviceToHost, s->copy_out);
+        }
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(s->x_ref, x_cur, s->tensor_bytes, cudaMemcpyHostToDevice, s->copy_in);
+    if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy out): %s", cudaGetErrorString(e));
+    s->last_h2d_bytes = s->tensor_bytes * 4;
+    return ASTRAEA_OK;
+}
+
+// the end of a step: everything that it sent for has ended
+static int32_t step_host_end(astraea_session *s)
+{
+    cudaError_t e = cudaStreamSynchronize(s->copy_out);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->copy_in);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->gather);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream2);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);      // the refresh of x_ref runs beside the attention
+    if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy out): %s", cudaGetErrorString(e));
+    s->steps++;
+    return astraea_poll_error(s->workspace, s->stream);
+}
+
 int32_t astraea_step_host(astraea_session *s, const void *x_cur, const void *q, const void *k,
                           const void *v, void *out, int k_keep,
                           float w_alpha, float w_beta, int delta_mode, int lse_mode)
@@ -780,6 +843,12 @@ int32_t astraea_step_host(astraea_session *s, const void *x_cur, const void *q, 
     // Rough rates: 1e15 flop/s for the attention, 5e10 bytes/s for the bus.
     const void *q_mapped = nullptr;
     const double attn_s = 4.0 * B * H * (double)M * N * d / 1e15, bus_s = 4.0 * (double)s->tensor_bytes / 5e10;
+    // Every token: by rows where the attention takes no longer than q and x_cur on the bus, which arrive under it (N up to about
+    // 20000 whatever the other sizes); beyond that the attention must not wait for all of k and v, and the heads arrive in groups.
+    if (M == N && B <= kHostGroups && attn_s <= 0.5 * bus_s) {
+        const int32_t rc = step_host_all_rows(s, x_cur, q, k, v, out);
+        return rc != ASTRAEA_OK ? rc : step_host_end(s);
+    }
     if (M < N && M > 0 && attn_s < bus_s) {
         cudaPointerAttributes attr;
         if (cudaPointerGetAttributes(&attr, q) == cudaSuccess && attr.type == cudaMemoryTypeHost && attr.devicePointer)
@@ -863,14 +932,7 @@ int32_t astraea_step_host(astraea_session *s, const void *x_cur, const void *q, 
                                   width, rows, cudaMemcpyDeviceToHost, s->copy_out);
         if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy out): %s", cudaGetErrorString(e));
     }
-    e = cudaStreamSynchronize(s->copy_out);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->copy_in);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->gather);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream2);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);      // the refresh of x_ref runs beside the attention
-    if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy out): %s", cudaGetErrorString(e));
-    s->steps++;
-    return astraea_poll_error(s->workspace, s->stream);
+    return step_host_end(s);
 }
 
 }  // extern "C"

@@ -24,9 +24,8 @@
 //               measured at 331 us where this takes 119, 9001 x 3072 x 3072.)
 // Layers of the same rows (the key and value projections; with SelectQ&K the query projection, too) share one launch: their column
 // tiles follow one another, so that one partial round of tiles is paid instead of two or three, the rows of x are read once for all, and
-// a launch is saved (7 us of set-up, first loads and last epilogue).  A block of 4276 tokens x 1536 channels: 44 us for two launches of
-// 102 tiles on 74 pairs, 38 for one of 204; four such blocks 1070 -> 1047 us; 32768 x 1152 twice, the Open-Sora block: 1863 ->
-// 1840; 17776 x 3072 twice, the CogVideoX block: 4469 -> 4434.
+// a launch is saved (7 us of set-up, first loads and last epilogue).  Keys and values of 4276 x 1536, four blocks (102 tiles on 74 pairs,
+// eight times): 1070 -> 1047 us; of 32768 x 1152, the Open-Sora block: 1863 -> 1840; of 17776 x 3072, the CogVideoX block: 4469 -> 4434.
 // Every mbarrier wait is bounded; on a timeout the CTA raises the error word, its remaining waits return at once, it sends
 // for no further copy, the other CTA of the pair runs into its own limit, and both run out; they leave together, when the copies
 // and MMAs that were under way have ended.
