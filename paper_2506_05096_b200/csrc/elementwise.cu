@@ -20,20 +20,6 @@ constexpr int kWarpsPerBlock = 4;
 constexpr int kBlocksPerSM = 16;
 constexpr int kMaxVecPerLane = 16;     // rows of up to 32 * 16 * 8 = 4096 channels
 
-// fp32 pairs: two elements of a row in one 64-bit register
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) { f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; }
-__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) { f32x2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { f32x2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
-// eight bf16 as four fp32 pairs
-__device__ __forceinline__ void unpack8(const uint4 &v, f32x2 (&f)[4]) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) f[i] = pack2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
-}
-
 // VPL: 16-byte vectors per lane (vec_per_row <= 32 * VPL)
 template <int VPL>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, VPL <= 6 ? 8 : VPL <= 8 ? 6 : 4)

@@ -87,20 +87,34 @@ __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// erf(x) to 1.5e-7 absolute (rational approximation 7.1.26 of Abramowitz and Stegun: 1 - (a1 t + ... + a5 t^5) e^{-x^2},
-// t = 1 / (1 + p |x|)): two XU operations and nine FMA-pipe ones without a branch, about half of erff()'s cost, which
-// counts where the main loop of the next tile is too short to hide the epilogue of this one (K = 1152: 5 us).  The result goes
-// into a bf16 (2^-9 relative).
-__device__ __forceinline__ float erf_fast(float x) {
-    const float ax = fabsf(x);
-    float t, e;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f, ax, 1.0f)));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(ax * ax * -1.4426950408889634f));
-    float pl = fmaf(1.061405429f, t, -1.453152027f);
-    pl = fmaf(pl, t, 1.421413741f);
-    pl = fmaf(pl, t, -0.284496736f);
-    pl = fmaf(pl, t, 0.254829592f);
-    return copysignf(fmaf(-pl * t, e, 1.0f), x);
+// GELU(x) = x (1 + erf(x / sqrt 2)) / 2 of two elements, with erf to 1.5e-7 absolute (rational approximation 7.1.26 of Abramowitz
+// and Stegun: erf(z) = 1 - (a1 t + ... + a5 t^5) e^{-z^2} for z >= 0, t = 1 / (1 + p z)): with w = 1/2 + copysign(1/2 - (a1 t +
+// ... + a5 t^5) e^{-x^2 / 2} / 2, x) it is x w.  Issue slots bind it (the epilogue of a tile has four warps on each SM sub-partition,
+// and a main loop of K = 1152 is over in 5 us), so all but the XU operations and the signs are packed pairs: 9.5 instructions per
+// element instead of 17.  13106 x 1152 x 4608 took
+// 108.7 us with the erf element by element and the epilogue's loads behind its wait, 101.9 now; 1846 x 1536 x 6144 31.1 -> 30.3.
+__device__ __forceinline__ f32x2 both(float v) { return pack2(v, v); }
+__device__ __forceinline__ f32x2 gelu2(f32x2 x) {
+    const f32x2 ax = x & 0x7fffffff7fffffffull;
+    float d0, d1, a0, a1, t0, t1, e0, e1;
+    unpack2(fma2(ax, both(0.3275911f * 0.70710678118654752f), both(1.0f)), d0, d1);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(d0));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(d1));
+    unpack2(mul2(mul2(x, x), both(-0.5f * 1.4426950408889634f)), a0, a1);
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(a0));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(a1));
+    const f32x2 t = pack2(t0, t1);
+    f32x2 pl = fma2(both(-0.5f * 1.061405429f), t, both(0.5f * 1.453152027f));           // minus half the polynomial
+    pl = fma2(pl, t, both(-0.5f * 1.421413741f));
+    pl = fma2(pl, t, both(0.5f * 0.284496736f));
+    pl = fma2(pl, t, both(-0.5f * 0.254829592f));
+    const f32x2 half_erf = fma2(mul2(pl, t), pack2(e0, e1), both(0.5f));                // of |x|: >= 0
+    return mul2(x, add2(both(0.5f), half_erf | (x & 0x8000000080000000ull)));
+}
+
+__device__ __forceinline__ uint4 shfl_vec(const uint4 &v, int lane) {
+    return make_uint4(__shfl_sync(0xffffffffu, v.x, lane), __shfl_sync(0xffffffffu, v.y, lane), __shfl_sync(0xffffffffu, v.z, lane),
+                      __shfl_sync(0xffffffffu, v.w, lane));
 }
 
 // 2-D tiled load global -> this CTA's shared memory, completion counted in bytes on an mbarrier of either CTA of the pair
@@ -203,7 +217,33 @@ gathered_linear_kernel(const __grid_constant__ WMaps tmap_w, const __grid_consta
             bool bad;
             long long full_row = target_row(p, (long long)tm * kBM + row, total_rows, &batch, &bad);
             if (bad && tn == 0 && part == 0) atomicExch(p.err_word, kErrBadIndex);
-            const __nv_bfloat16 *gate = p.gate ? p.gate + (long long)batch * p.N_out : nullptr;
+            // What the epilogue reads is fetched while the main loop runs: behind the wait, each of the two groups of columns would pay
+            // a round trip to L2 for its bias, and another one for the residual (rows x K x N_out 1846 x 1536 x 1536, a launch in a
+            // chain: 12.24 -> 11.32 us; 2 x 6553 of 32768 x 1152 x 1152 34.3 -> 32.5; of 3.1 us from the last MMA to the last store).
+            // The vectors that all rows share go round by shuffles: lanes 0-7 hold 8 columns of the bias each (0-3 of the first
+            // group, 4-7 of the second), lanes 8-15 of the gate.
+            const int q = lane & 3;
+            const unsigned in_list = __ballot_sync(0xffffffffu, full_row >= 0);
+            const int batch0 = __shfl_sync(0xffffffffu, batch, in_list ? __ffs(in_list) - 1 : 0);
+            const bool one_batch = __all_sync(0xffffffffu, full_row < 0 || batch == batch0);       // (a gate belongs to a batch element)
+            uint4 vec = make_uint4(0, 0, 0, 0);
+            {
+                const int c = c0 + ((lane >> 2) & 1) * (32 * kEpiSplit), mat = mat_of<MULTI>(p, tn * p.bn + c);
+                const int col = tn * p.bn + c - mat * p.mat_cols + q * 8;
+                const __nv_bfloat16 *src = lane < 8 ? p.bias[mat] : lane < 16 && !MULTI && p.gate ? p.gate + (long long)batch0 * p.N_out : nullptr;
+                if (src && c < p.bn && col < p.N_out) vec = ld_cached(reinterpret_cast<const uint4 *>(src + col));
+            }
+            uint4 rr[4];                                            // rows (lane >> 2) + 8 j of the residual, 8 columns each
+            auto fetch_residual = [&](int colq) {
+                const long long res_row = (full_row >= 0 && p.res_compact) ? (long long)tm * kBM + row : full_row;
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) {
+                    const long long rrow = __shfl_sync(0xffffffffu, res_row, (lane >> 2) + 8 * jj);
+                    rr[jj] = (rrow >= 0 && colq < p.N_out) ? __ldcg(reinterpret_cast<const uint4 *>(p.residual + rrow * p.N_out + colq))
+                                                           : make_uint4(0, 0, 0, 0);
+                }
+            };
+            if (!MULTI && p.residual && c0 < p.bn) fetch_residual(tn * p.bn + c0 + q * 8);
             wait_bar(bar_acc_full + 8 * acc, (it / kAccSets) & 1, &abort_flag, p.err_word);
             if (tile + n_pairs >= total_tiles) grid_launch_dependents();       // the last epilogue of this CTA
             tc_fence_after();
@@ -219,38 +259,23 @@ gathered_linear_kernel(const __grid_constant__ WMaps tmap_w, const __grid_consta
             // 36 us tile, 16 us with a residual).  Instead lane l moves the 16-byte piece l & 3 of rows (l >> 2) + 8 j:
             // 64 contiguous bytes per row, 8 rows per instruction, through 2 KB of shared memory per warp (pieces
             // swizzled by the row so that both directions are free of bank conflicts).
-            const int q = lane & 3;
 #pragma unroll 1
             for (int c = c0; c < p.bn; c += 32 * kEpiSplit) {
                 const int mat = mat_of<MULTI>(p, tn * p.bn + c), n0 = tn * p.bn + c - mat * p.mat_cols;     // 32 columns of one matrix from n0
-                const __nv_bfloat16 *bias = p.bias[mat];
+                const bool bias = p.bias[mat] != nullptr;
+                const int first = c == c0 ? 0 : 4;                  // the lanes that hold this group's vectors
                 __nv_bfloat16 *y = p.y[mat];
                 // the row of a compact tensor is the row of the list
                 const long long out_row = (full_row >= 0 && (p.compact >> mat & 1u)) ? (long long)tm * kBM + row : full_row;
                 const int colq = n0 + q * 8;                        // the 8 columns this lane moves
-                uint32_t rw[16];                                    // this thread's row of the residual: 32 bf16
                 if (!MULTI && p.residual) {
-                    const long long res_row = (full_row >= 0 && p.res_compact) ? (long long)tm * kBM + row : full_row;
-                    uint4 rr[4];
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) {
-                        const int r = (lane >> 2) + 8 * jj;
-                        const long long rrow = __shfl_sync(0xffffffffu, res_row, r);
-                        rr[jj] = (rrow >= 0 && colq < p.N_out) ? __ldcg(reinterpret_cast<const uint4 *>(p.residual + rrow * p.N_out + colq))
-                                                                : make_uint4(0, 0, 0, 0);
-                    }
 #pragma unroll
                     for (int jj = 0; jj < 4; ++jj) {
                         const int r = (lane >> 2) + 8 * jj;
                         *reinterpret_cast<uint4 *>(stage + r * 64 + ((q ^ ((r >> 1) & 3)) << 4)) = rr[jj];
                     }
                     __syncwarp();
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        const uint4 t = *reinterpret_cast<const uint4 *>(stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4));
-                        rw[4 * v] = t.x; rw[4 * v + 1] = t.y; rw[4 * v + 2] = t.z; rw[4 * v + 3] = t.w;
-                    }
-                    __syncwarp();
+                    if (c + 32 * kEpiSplit < p.bn) fetch_residual(colq + 32 * kEpiSplit);
                 }
                 uint32_t o[32];
                 tmem_ld32(t_row + acc * kAccCols + c, o);
@@ -259,47 +284,42 @@ gathered_linear_kernel(const __grid_constant__ WMaps tmap_w, const __grid_consta
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     const int col = n0 + v * 8;
-                    float f[8];
+                    uint4 *mine = reinterpret_cast<uint4 *>(stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4));     // residual in, result out
+                    f32x2 f[4], t[4];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(o[v * 8 + i]);
-                    if (col < p.N_out) {                 // N_out is a multiple of 8; columns past it are never stored
-                        if (bias) {
-                            const uint4 bb = ld_cached(reinterpret_cast<const uint4 *>(bias + col));
-                            const uint32_t bw[4] = {bb.x, bb.y, bb.z, bb.w};
+                    for (int i = 0; i < 4; ++i) f[i] = pack2(__uint_as_float(o[v * 8 + 2 * i]), __uint_as_float(o[v * 8 + 2 * i + 1]));
+                    if (bias) {
+                        unpack8(shfl_vec(vec, first + v), t);
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                f[2 * i] += __uint_as_float(bw[i] << 16);
-                                f[2 * i + 1] += __uint_as_float(bw[i] & 0xffff0000u);
-                            }
-                        }
-                        if (!MULTI && p.gelu) {
+                        for (int i = 0; i < 4; ++i) f[i] = add2(f[i], t[i]);
+                    }
+                    if (!MULTI && p.gelu) {
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) f[i] = 0.5f * f[i] * (1.0f + erf_fast(f[i] * 0.70710678118654752f));
-                        }
-                        if (!MULTI && gate) {
-                            const uint4 gg = ld_cached(reinterpret_cast<const uint4 *>(gate + col));
-                            const uint32_t gw[4] = {gg.x, gg.y, gg.z, gg.w};
+                        for (int i = 0; i < 4; ++i) f[i] = gelu2(f[i]);
+                    }
+                    if (!MULTI && p.gate) {
+                        uint4 g = shfl_vec(vec, 8 + first + v);
+                        if (!one_batch && col < p.N_out) g = ld_cached(reinterpret_cast<const uint4 *>(p.gate + (long long)batch * p.N_out + col));
+                        unpack8(g, t);
+                    }
+                    if (!MULTI && p.residual) {
+                        f32x2 r[4];
+                        unpack8(*mine, r);
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                f[2 * i] *= __uint_as_float(gw[i] << 16);
-                                f[2 * i + 1] *= __uint_as_float(gw[i] & 0xffff0000u);
-                            }
-                        }
-                        if (!MULTI && p.residual) {
+                        for (int i = 0; i < 4; ++i) f[i] = p.gate ? fma2(f[i], t[i], r[i]) : add2(f[i], r[i]);
+                    } else if (!MULTI && p.gate) {
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                f[2 * i] += __uint_as_float(rw[4 * v + i] << 16);
-                                f[2 * i + 1] += __uint_as_float(rw[4 * v + i] & 0xffff0000u);
-                            }
-                        }
+                        for (int i = 0; i < 4; ++i) f[i] = mul2(f[i], t[i]);
                     }
                     uint32_t w[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        __nv_bfloat162 v2 = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
+                        float lo, hi;
+                        unpack2(f[i], lo, hi);
+                        __nv_bfloat162 v2 = __floats2bfloat162_rn(lo, hi);
                         w[i] = *reinterpret_cast<uint32_t *>(&v2);
                     }
-                    *reinterpret_cast<uint4 *>(stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                    *mine = make_uint4(w[0], w[1], w[2], w[3]);
                 }
                 __syncwarp();
 #pragma unroll
