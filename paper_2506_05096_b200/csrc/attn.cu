@@ -13,7 +13,8 @@
 //   two warps  tcgen05.mma issuers, one per query tile: S = Q K^T (SS, K-major operands), O += P V (P from
 //              TMEM, V as an MN-major shared-memory operand); the first owns the TMEM allocation;
 //   one warp   donates registers (setmaxnreg moves registers to the softmax warps) and, when the caller has rows to copy at
-//              the same indices (the reference inputs of a step), moves them by bulk copies through shared memory.
+//              the same indices (the reference inputs of a step), moves them by bulk copies through shared memory, unless the
+//              launch has SMs to spare, where CTAs of their own copy them (copy_cta).
 //
 // Two softmax warpgroups per query tile put four softmax warps on every SM sub-partition, which hides the
 // serial chain of a key tile (wait, load, exponentials, sum, pack, publish).  Even key tiles go to one
@@ -161,6 +162,7 @@ struct Params {
     uint4 *copy_dst;
     uint32_t copy_bytes;
     int copy_rows;               // B * M
+    int n_ctas, copy_ctas;       // CTAs of the attention, and CTAs behind them that copy the rows (0: the attention's CTAs do)
     float *part_o, *part_lse;    // [part][kTilesM * 128 rows][head_dim] and [part][kTilesM * 128 rows]
 };
 
@@ -632,6 +634,30 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Bars &bar, i
 
 #include "copy_rows.cuh"
 
+// A CTA that copies rows only (a launch that leaves SMs idle has some): its share of the listed rows, a warp for each, with plain
+// 16-byte loads, several in flight per lane.
+__device__ __forceinline__ void copy_cta(const Params &p, int cta)
+{
+    const int r0 = (int)((long long)p.copy_rows * cta / p.copy_ctas), r1 = (int)((long long)p.copy_rows * (cta + 1) / p.copy_ctas);
+    const int lane = threadIdx.x & 31, vecs = (int)(p.copy_bytes >> 4);
+    grid_dependency_wait();
+    for (int r = r0 + (threadIdx.x >> 5); r < r1; r += blockDim.x >> 5) {
+        const int b = r / p.M, m = r - b * p.M;
+        const int tok = __ldcg(p.q_idx + r), before = m > 0 ? __ldcg(p.q_idx + r - 1) : -1;
+        if ((unsigned)tok >= (unsigned)p.N_tok || before >= tok) continue;                       // reported by the softmax warps
+        const uint4 *src = p.copy_src + ((size_t)b * p.N_tok + tok) * vecs;
+        uint4 *dst = p.copy_dst + ((size_t)b * p.N_tok + tok) * vecs;
+        constexpr int kIn = 6;
+        for (int v = lane; v < vecs; v += 32 * kIn) {
+            uint4 a[kIn];
+#pragma unroll
+            for (int u = 0; u < kIn; ++u) if (v + 32 * u < vecs) a[u] = ld_stream(src + v + 32 * u);
+#pragma unroll
+            for (int u = 0; u < kIn; ++u) if (v + 32 * u < vecs) dst[v + 32 * u] = a[u];
+        }
+    }
+}
+
 template <class C>
 __global__ void __launch_bounds__(C::kThreads, C::kCtasPerSM)
 sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v,
@@ -664,6 +690,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     const uint32_t bar_copy = bar.ve + 8 * C::kStagesV, bar_end = bar_copy + 8 * C::kCopyStages;
     static_assert(160 + 16 * (C::kStagesK + C::kStagesV) + 8 * (C::kCopyStages + 2) <= C::kBarBytes, "barrier area too small");
 
+    if ((int)blockIdx.x >= p.n_ctas) {
+        copy_cta(p, (int)blockIdx.x - p.n_ctas);
+        return;
+    }
     const int tid = threadIdx.x;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);        // warp-uniform
     constexpr int kBlockN = C::kBlockN;
@@ -759,7 +789,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     // softmax warps for the last MMAs), so the mbarriers are set up afresh and every role counts from zero again.
     auto next_unit = [&]() -> bool {
         if constexpr (!C::kPersistent) return false;
-        unit += gridDim.x;
+        unit += p.n_ctas;
         if (unit >= n_units) return false;
         m0 = (unit % p.tiles_x) * (kTilesM * kBlockM); h = p.h0 + (unit / p.tiles_x) % p.heads; b = unit / (p.tiles_x * p.heads);
         tc_fence_before();
@@ -797,7 +827,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
         do {
             if (tile < q_tiles)
                 softmax_role<C>(p, bar, tile, par, smem_gen + tile * C::kQTileBytes, tmem, m0 + tile * kBlockM, h, b, n_tiles, key0, part,
-                                 !C::kPersistent || unit + (int)gridDim.x >= n_units, &abort_flag, &redo_flag, xchg[tile]);
+                                 !C::kPersistent || unit + p.n_ctas >= n_units, &abort_flag, &redo_flag, xchg[tile]);
             else pass_sync<C>();
         } while (next_unit());
     } else if (warp == kProducerWarp) {
@@ -958,9 +988,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
         } while (next_unit());
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
-        if (p.copy_dst) copy_role<C>(p, sCopy, bar_copy, &abort_flag);
+        // The pass does not wait for the rows that it copies (a CTA of a few key tiles is done before them): it is counted ahead.
+        asm volatile("bar.arrive 5, %0;" ::"n"(C::kThreads) : "memory");
+        if (p.copy_dst && p.copy_ctas == 0) copy_role<C>(p, sCopy, bar_copy, &abort_flag);
         __syncwarp();
-        do pass_sync<C>(); while (next_unit());
+        while (next_unit()) pass_sync<C>();
     }
 
     tc_fence_before();
@@ -1123,12 +1155,22 @@ int32_t launch_dh(const AttnArgs &a, cudaStream_t stream, SplitPlan plan = Split
     // stands for all of them and errs on the side of the scatter.)
     const long long copy_rows = (long long)a.B * a.M;
     const double copy_us = a.copy_dst ? (double)((copy_rows + grid - 1) / grid) * a.copy_elems * 2 / 4096 : 0.0;
-    const bool copy_here = a.copy_dst && (long long)a.B * a.N_tok * (a.copy_elems / 8) < 0x7fffffffll && copy_us <= 0.4 * ((a.N + C::kBlockN - 1) / C::kBlockN) * units_per_cta / p.split + 4.0;
+    // A launch that leaves SMs idle gets CTAs that only copy, at about 30 KB a microsecond each, if they are done within the same
+    // limit; its attention CTAs, which live for a few key tiles there, then copy nothing.  (Step of 128 x 256 tokens, 2 heads of 64: with
+    // the copying warp in the pass's barrier the CTA waited 4.7 us for it; graph 15.6 -> 11.8 us, step behind a copy of the LSE
+    // cache 20.3 -> 17.4; 250 x 500 tokens, 3 heads of 128: 21.3 -> 19.7; launches of 120 units and more: no difference.)
+    const double copy_all = (double)copy_rows * a.copy_elems * 2;
+    const int idle = slots - (int)grid;
+    const int wanted = a.copy_dst ? (int)(copy_all / 8192 < 1024 ? copy_all / 8192 + 1 : 1024) : 0, copy_ctas = idle < wanted ? idle : wanted;
+    const bool copy_idle = copy_ctas > 0 && copy_all / copy_ctas <= 30e3 * (0.4 * ((a.N + C::kBlockN - 1) / C::kBlockN) * units_per_cta / p.split + 4.0);
+    const bool copy_here = copy_idle || a.copy_dst && (long long)a.B * a.N_tok * (a.copy_elems / 8) < 0x7fffffffll && copy_us <= 0.4 * ((a.N + C::kBlockN - 1) / C::kBlockN) * units_per_cta / p.split + 4.0;
     p.copy_src = copy_here ? reinterpret_cast<const uint4 *>(a.copy_src) : nullptr;
     p.copy_dst = copy_here ? reinterpret_cast<uint4 *>(a.copy_dst) : nullptr;
     p.copy_bytes = (uint32_t)a.copy_elems * 2;
     p.copy_rows = copy_here ? (int)copy_rows : 0;
-    launch_overlapped(sparse_attn_kernel<C>, grid, C::kThreads, C::kSmemBytes, stream, mk, mv, mkt, mvt, p);
+    p.n_ctas = (int)grid;
+    p.copy_ctas = copy_idle ? copy_ctas : 0;
+    launch_overlapped(sparse_attn_kernel<C>, grid + (unsigned)p.copy_ctas, C::kThreads, C::kSmemBytes, stream, mk, mv, mkt, mvt, p);
     if (split) {
         static_assert((TM * kBlockM * (DH / 8)) % (TM * kBlockM) == 0, "whole blocks per unit");
         launch_overlapped(merge_parts_kernel<DH, TM * kBlockM>, dim3(DH / 8, plan.units), TM * kBlockM, 0, stream, p);
