@@ -176,6 +176,7 @@ constexpr int kMaxCluster = 8;
 constexpr int kBinsWide = 4096;                  // 12-bit digits (the last digit has 8 bits and uses 256 of the bins)
 constexpr int kPasses = 3;
 constexpr size_t kClusterSmem = 2 * kPasses * kBinsWide * sizeof(uint32_t);      // own + cluster histogram per pass: 96 KB
+constexpr size_t kBlockSmem = (2 * kBinsWide + 256) * sizeof(uint32_t);          // one histogram per pass, the last one of 8 bits at most
 
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -198,20 +199,25 @@ __device__ __forceinline__ void remote_store(uint32_t addr, uint32_t v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-template <int ITEMS>
+// CLUSTER false: the row fits one CTA.  Nothing goes through DSMEM and no cluster barrier is paid then, and the digits are
+// taken from the top of the range that the row's keys span rather than of the 32 bits: scores of one step lie within a few
+// powers of two, whose keys share most of the leading 12 bits, so that the first fixed digit hardly parts them and ties in the leading 24
+// bits cost a third pass.
+template <int ITEMS, bool CLUSTER>
 __global__ void __launch_bounds__(kThreads)
 select_cluster_kernel(const float *__restrict__ score, int N_sel, int k, int n_always,
                       int32_t *__restrict__ idx_sel, int32_t *__restrict__ idx_rem, int32_t *__restrict__ n_skip)
 {
     extern __shared__ __align__(16) uint32_t smem_hist[];      // [kPasses][kBinsWide] own counts, then [kPasses][kBinsWide] cluster counts
+    constexpr size_t kSmem = CLUSTER ? kClusterSmem : kBlockSmem;
     uint32_t *hist = smem_hist, *ghist = smem_hist + kPasses * kBinsWide;
     __shared__ uint32_t cta_gt[kMaxCluster], cta_eq[kMaxCluster];   // selected-by-greater / equal totals of every CTA
-    __shared__ uint32_t warp_tot[32], warp_gt[32], warp_eq[32];
+    __shared__ uint32_t warp_tot[32], warp_gt[32], warp_eq[32], warp_min[32], warp_max[32];
     __shared__ uint32_t s_prefix, s_kk, s_cnt;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.y;
-    const uint32_t rank = cluster_rank(), csize = gridDim.x;
+    const uint32_t rank = CLUSTER ? cluster_rank() : 0u, csize = CLUSTER ? gridDim.x : 1u;
     const float *s = score + (size_t)b * N_sel;
     int32_t *sel = idx_sel ? idx_sel + (size_t)b * (k + n_always) : nullptr;
     int32_t *rem = idx_rem ? idx_rem + (size_t)b * (N_sel - k) : nullptr;
@@ -220,9 +226,9 @@ select_cluster_kernel(const float *__restrict__ score, int N_sel, int k, int n_a
     const int base = ((int)rank * kThreads + tid) * ITEMS;      // this thread's consecutive tokens
     {
         uint4 *z = reinterpret_cast<uint4 *>(smem_hist);
-        for (int i = tid; i < (int)(kClusterSmem / 16); i += kThreads) z[i] = make_uint4(0, 0, 0, 0);
+        for (int i = tid; i < (int)(kSmem / 16); i += kThreads) z[i] = make_uint4(0, 0, 0, 0);
     }
-    cluster_sync_all();                          // every CTA's histograms are zero before anyone adds to them (still ahead of the wait)
+    if constexpr (CLUSTER) cluster_sync_all();   // every CTA's histograms are zero before anyone adds to them (still ahead of the wait)
     grid_launch_dependents();                    // the next kernel may set itself up; it waits for this one before it reads anything
     grid_dependency_wait();                      // the scores (and whatever else the kernel before wrote) are complete
     uint32_t key[ITEMS];
@@ -271,15 +277,35 @@ select_cluster_kernel(const float *__restrict__ score, int N_sel, int k, int n_a
         }
     }
 
+    int bits = 32;                               // of the keys, from here on
+    if constexpr (!CLUSTER) {
+        // the keys become their distance from the row's least
+        uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+        for (int u = 0; u < ITEMS; ++u)
+            if (base + u < N_sel) { lo = min(lo, key[u]); hi = max(hi, key[u]); }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (lane == 0) { warp_min[warp] = lo; warp_max[warp] = hi; }
+        __syncthreads();                         // (the cleared histograms, too)
+        lo = __reduce_min_sync(0xffffffffu, warp_min[lane]);
+        hi = __reduce_max_sync(0xffffffffu, warp_max[lane]);
+#pragma unroll
+        for (int u = 0; u < ITEMS; ++u) key[u] -= lo;
+        bits = 32 - __clz(hi - lo);
+    }
+
     // token i is selected iff key > T, or key == T and fewer than need_eq equal keys precede it
     uint32_t T = 0xffffffffu, need_eq = 0;       // no key reaches 0xffffffff
-    if (k > 0) {
+    if (k > 0 && bits == 0) { T = 0; need_eq = (uint32_t)k; }      // all alike
+    else if (k > 0) {
         uint32_t prefix = 0, mask = 0, kk = (uint32_t)k;
 #pragma unroll 1
         for (int pass = 0; pass < kPasses; ++pass) {
-            const int shift = pass == 0 ? 20 : pass == 1 ? 8 : 0;
-            const uint32_t digit_mask = pass == 2 ? 255u : 4095u;
-            uint32_t *h = hist + pass * kBinsWide, *gh = ghist + pass * kBinsWide;
+            // 12, 12 and 8 bits, fewer where the keys have fewer
+            const int shift = CLUSTER ? (pass == 0 ? 20 : pass == 1 ? 8 : 0) : max(bits - 12 * (pass + 1), 0);
+            const uint32_t digit_mask = CLUSTER ? (pass == 2 ? 255u : 4095u) : (1u << (bits - 12 * pass - shift)) - 1u;
+            uint32_t *h = hist + pass * kBinsWide, *gh = CLUSTER ? ghist + pass * kBinsWide : h;
 #pragma unroll
             for (int u = 0; u < ITEMS; ++u) {
                 const bool live = (base + u < N_sel) && ((key[u] & mask) == prefix);
@@ -297,21 +323,23 @@ select_cluster_kernel(const float *__restrict__ score, int N_sel, int k, int n_a
                 }
             }
             __syncthreads();
-            // this CTA's non-zero counts go into every CTA's copy, so that every CTA searches its own copy
             const int bins = (int)digit_mask + 1;
-            for (int i = tid; i < bins; i += kThreads) {
-                const uint32_t c = h[i];
-                if (c != 0)
-                    for (uint32_t r = 0; r < csize; ++r) remote_add(map_to_rank(&gh[i], r), c);
+            if constexpr (CLUSTER) {
+                // this CTA's non-zero counts go into every CTA's copy, so that every CTA searches its own copy
+                for (int i = tid; i < bins; i += kThreads) {
+                    const uint32_t c = h[i];
+                    if (c != 0)
+                        for (uint32_t r = 0; r < csize; ++r) remote_add(map_to_rank(&gh[i], r), c);
+                }
+                cluster_sync_all();
             }
-            cluster_sync_all();
             // search from the top: thread t owns bins top-4t .. top-4t-3 (the 256-bin pass uses the first 64 threads)
             {
                 const int top = bins - 1 - 4 * tid;
                 uint32_t c[4] = {0, 0, 0, 0}, tot = 0;
-                if (top >= 3) {
+                if (CLUSTER ? top >= 3 : top >= 0) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) { c[j] = gh[top - j]; tot += c[j]; }
+                    for (int j = 0; j < 4; ++j) { c[j] = CLUSTER || top >= j ? gh[top - j] : 0u; tot += c[j]; }
                 }
                 uint32_t inc = tot;
 #pragma unroll
@@ -353,7 +381,7 @@ select_cluster_kernel(const float *__restrict__ score, int N_sel, int k, int n_a
                 need_eq = 0xffffffffu;
                 break;
             }
-            if (pass == kPasses - 1) { T = prefix; need_eq = kk; }
+            if (CLUSTER ? pass == kPasses - 1 : shift == 0) { T = prefix; need_eq = kk; break; }
         }
     }
 
@@ -384,20 +412,22 @@ select_cluster_kernel(const float *__restrict__ score, int N_sel, int k, int n_a
     const uint32_t be = warp > 0 ? __shfl_sync(0xffffffffu, we, warp - 1) : 0u;
     // every CTA learns every CTA's totals (the shuffles are outside the branch: all 32 lanes must take part)
     const uint32_t allg = __shfl_sync(0xffffffffu, wg, 31), alle = __shfl_sync(0xffffffffu, we, 31);
-    if (warp == 0 && lane < (int)csize) {
-        remote_store(map_to_rank(&cta_gt[rank], lane), allg);
-        remote_store(map_to_rank(&cta_eq[rank], lane), alle);
-    }
-    cluster_sync_all();
     uint32_t pg = bg + ig - tg, pe = be + ie - te;
-    for (uint32_t r = 0; r < rank; ++r) { pg += cta_gt[r]; pe += cta_eq[r]; }
+    if constexpr (CLUSTER) {
+        if (warp == 0 && lane < (int)csize) {
+            remote_store(map_to_rank(&cta_gt[rank], lane), allg);
+            remote_store(map_to_rank(&cta_eq[rank], lane), alle);
+        }
+        cluster_sync_all();
+        for (uint32_t r = 0; r < rank; ++r) { pg += cta_gt[r]; pe += cta_eq[r]; }
+    }
     // With 8 or 16 tokens per thread a warp's direct stores of the two index lists would touch 32 lines per instruction
     // (a thread's entries are consecutive, the lanes are 32 or 64 bytes apart).  The warp's tokens are consecutive, and
     // so are their places in both lists: the entries are first put in order into the warp's piece of the histogram
     // memory (idle since the last cluster barrier; nobody writes it remotely any more), then copied out by whole lines.
     constexpr bool kStage = ITEMS >= 8;
     int32_t *stage = reinterpret_cast<int32_t *>(smem_hist) + warp * (32 * ITEMS);
-    static_assert(!kStage || (size_t)kThreads * ITEMS * sizeof(int32_t) <= kClusterSmem, "the staged lists fit the histogram memory");
+    static_assert(!kStage || (size_t)kThreads * ITEMS * sizeof(int32_t) <= kSmem, "the staged lists fit the histogram memory");
     const uint32_t before0 = pg + min(pe, need_eq);              // selected tokens ahead of this thread's first token
     const uint32_t takes = tg + min(te, need_eq > pe ? need_eq - pe : 0u);
     const uint32_t w_sel0 = __shfl_sync(0xffffffffu, before0, 0);
@@ -452,12 +482,20 @@ select_cluster_kernel(const float *__restrict__ score, int N_sel, int k, int n_a
 }
 
 template <int ITEMS>
+int32_t launch_block(const float *score, int B, int N_sel, int k, int n_always, int32_t *idx_sel, int32_t *idx_rem, int32_t *n_skip, cudaStream_t stream)
+{
+    static_assert(kBlockSmem <= 48 * 1024 - 1024, "no attribute needed");
+    launch_overlapped(select_cluster_kernel<ITEMS, false>, dim3(1, B), kThreads, kBlockSmem, stream, score, N_sel, k, n_always, idx_sel, idx_rem, n_skip);
+    return check_launch("astraea_select");
+}
+
+template <int ITEMS>
 int32_t launch_cluster(const float *score, int B, int N_sel, int k, int n_always, int32_t *idx_sel,
                        int32_t *idx_rem, int32_t *n_skip, cudaStream_t stream)
 {
     const int csize = (N_sel + ITEMS * kThreads - 1) / (ITEMS * kThreads);
     static PerDeviceOnce attrs;                  // one per instantiation; the attribute is per device
-    if (attrs.run([] { return cudaFuncSetAttribute(select_cluster_kernel<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (attrs.run([] { return cudaFuncSetAttribute(select_cluster_kernel<ITEMS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)kClusterSmem); }) != cudaSuccess)
         return check_launch("astraea_select (shared memory attribute)");
     cudaLaunchConfig_t cfg = {};
@@ -474,7 +512,7 @@ int32_t launch_cluster(const float *score, int B, int N_sel, int k, int n_always
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, select_cluster_kernel<ITEMS>, score, N_sel, k, n_always, idx_sel, idx_rem, n_skip);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, select_cluster_kernel<ITEMS, true>, score, N_sel, k, n_always, idx_sel, idx_rem, n_skip);
     if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_select: %s", cudaGetErrorString(e));
     return check_launch("astraea_select");
 }
@@ -487,6 +525,9 @@ int32_t launch_select(const float *score, int B, int N_sel, int k, int n_always,
                       int32_t *idx_rem, int32_t *n_skip, void *, cudaStream_t stream)
 {
     if (B == 0 || (N_sel == 0 && n_always == 0)) return ASTRAEA_OK;
+    // One CTA with two tokens a thread: 200 / 1000 / 2000 tokens 6.0 / 6.4 / 7.8 us with a cluster, 3.7 / 3.7 / 4.8 without.  With four a
+    // thread it is no faster inside a step (4000 tokens: 27.1 us with a cluster, 27.6 without), and with eight it is slower alone.
+    if (N_sel > 0 && N_sel <= 2 * kThreads) return launch_block<2>(score, B, N_sel, k, n_always, idx_sel, idx_rem, n_skip, stream);
     if (N_sel > 0 && N_sel <= 2 * kThreads * kMaxCluster)
         return launch_cluster<2>(score, B, N_sel, k, n_always, idx_sel, idx_rem, n_skip, stream);
     if (N_sel > 0 && N_sel <= 4 * kThreads * kMaxCluster)
