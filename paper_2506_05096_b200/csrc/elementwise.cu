@@ -8,7 +8,8 @@
 // normalises, modulates and stores in a second pass over the registers.  fp32 arithmetic, one rounding to bf16 at the end.
 // Next to the bytes the issue slots bind it: element by element it is ~105 instructions per 16-byte vector, so the
 // arithmetic is on packed fp32 pairs, and the register array has five and six vectors too, the widths of 1152 and 1536
-// channels (before -> after: 32768 x 1152 36.4 -> 29.1 us, 17776 x 3072 44.7 -> 40.6 = 5.4 TB/s, 4276 x 1536 7.8 -> 5.5).
+// channels (32768 x 1152 36.4 -> 29.1 us, 17776 x 3072 44.7 -> 40.6, 4276 x 1536 7.8 -> 5.5), and whether there are modulation
+// vectors is fixed at compile time (modulated now 26.5, 38.6 = 5.7 TB/s, 4.7).
 // Four warps a block rather than eight even out short launches and are worth 2-5 % of the long ones; two rows a warp,
 // sharing the unpacked modulation vectors, gain nothing.
 #include "common.cuh"
@@ -20,9 +21,19 @@ constexpr int kWarpsPerBlock = 4;
 constexpr int kBlocksPerSM = 16;
 constexpr int kMaxVecPerLane = 16;     // rows of up to 32 * 16 * 8 = 4096 channels
 
+// What the launch knows of the modulation vectors, fixed when the kernel is compiled: with the tests inside the loop over a row's
+// registers a plain norm took 20.7 us where it takes 15.6 now (9001 x 3072), a modulated one 24.1 (20.7 now); 32768 x 1152 27.5 ->
+// 22.7 and 29.5 -> 26.5, 1846 x 1536 4.5 -> 3.5 and 5.2 -> 3.5.
+enum { kPlain = 0,      // there are none
+       kBoth = 1,       // both are there, read from L1 for every row
+       kHeld = 2,       // both are there, each warp keeps its lane's part of them in registers: fewer blocks of an SM
+       kEither = 3 };   // one of them
+template <int VPL, int MOD> constexpr int kBlocks = MOD == kHeld ? (VPL <= 2 ? 8 : VPL <= 5 ? 5 : VPL <= 6 ? 4 : VPL <= 12 ? 3 : 2)
+                                                                 : VPL <= 6 ? 8 : VPL <= 8 ? 6 : 4;
+
 // VPL: 16-byte vectors per lane (vec_per_row <= 32 * VPL)
-template <int VPL>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, VPL <= 6 ? 8 : VPL <= 8 ? 6 : 4)
+template <int VPL, int MOD>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocks<VPL, MOD>)
 layernorm_modulate_kernel(const uint4 *__restrict__ x, const int32_t *__restrict__ idx, int M, const uint4 *__restrict__ scale,
                           const uint4 *__restrict__ shift, uint4 *__restrict__ y, int B, int N, int vec_per_row, float eps,
                           int compact_in, int compact_out, int *__restrict__ err_word)
@@ -32,8 +43,20 @@ layernorm_modulate_kernel(const uint4 *__restrict__ x, const int32_t *__restrict
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long total = (long long)B * M;
     const float inv_D = 1.0f / (float)(vec_per_row * 8);
+    constexpr bool kHold = MOD == kHeld;
+    uint4 sc_v[kHold ? VPL : 1], sh_v[kHold ? VPL : 1];
+    int batch = -1;                                                                          // that they belong to
     for (long long t = (long long)blockIdx.x * kWarpsPerBlock + warp; t < total; t += (long long)gridDim.x * kWarpsPerBlock) {
         const int b = (int)(t / M), r = (int)(t - (long long)b * M);
+        if (kHold && b != batch) {
+            batch = b;
+#pragma unroll
+            for (int u = 0; u < (kHold ? VPL : 0); ++u) {
+                const int c = lane + 32 * u;
+                sc_v[u] = c < vec_per_row ? ld_cached(scale + (long long)b * vec_per_row + c) : make_uint4(0, 0, 0, 0);
+                sh_v[u] = c < vec_per_row ? ld_cached(shift + (long long)b * vec_per_row + c) : make_uint4(0, 0, 0, 0);
+            }
+        }
         const int tok = idx ? __ldcg(idx + t) : r;
         const int before = (idx && r > 0) ? __ldcg(idx + t - 1) : -1;
         if ((unsigned)tok >= (unsigned)N || before >= tok) {                               // see astraea_scatter_reuse
@@ -76,14 +99,15 @@ layernorm_modulate_kernel(const uint4 *__restrict__ x, const int32_t *__restrict
             if (c < vec_per_row) {
                 f32x2 f[4], sc[4], sh[4];
                 unpack8(v[u], f);
-                if (scale) unpack8(ld_cached(scale + (long long)b * vec_per_row + c), sc);
-                if (shift) unpack8(ld_cached(shift + (long long)b * vec_per_row + c), sh);
+                const bool scaled = MOD != kPlain && (MOD != kEither || scale), shifted = MOD != kPlain && (MOD != kEither || shift);
+                if (scaled) unpack8(kHold ? sc_v[kHold ? u : 0] : ld_cached(scale + (long long)b * vec_per_row + c), sc);
+                if (shifted) unpack8(kHold ? sh_v[kHold ? u : 0] : ld_cached(shift + (long long)b * vec_per_row + c), sh);
                 uint32_t w[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     f[i] = mul2(add2(f[i], minus_mean), rstd);
-                    if (scale) f[i] = fma2(f[i], sc[i], f[i]);
-                    if (shift) f[i] = add2(f[i], sh[i]);
+                    if (scaled) f[i] = fma2(f[i], sc[i], f[i]);
+                    if (shifted) f[i] = add2(f[i], sh[i]);
                     unpack2(f[i], lo, hi);
                     __nv_bfloat162 v2 = __floats2bfloat162_rn(lo, hi);
                     w[i] = *reinterpret_cast<uint32_t *>(&v2);
@@ -94,12 +118,12 @@ layernorm_modulate_kernel(const uint4 *__restrict__ x, const int32_t *__restrict
     }
 }
 
-template <int VPL>
+template <int VPL, int MOD>
 void launch_ln(cudaStream_t stream, const uint4 *x, const int32_t *idx, int M, const uint4 *scale, const uint4 *shift, uint4 *y, int B, int N,
                int vec_per_row, float eps, int ci, int co, int *err_word)
 {
-    const long long want = ((long long)B * M + kWarpsPerBlock - 1) / kWarpsPerBlock, cap = (long long)sm_count() * kBlocksPerSM;
-    launch_overlapped(layernorm_modulate_kernel<VPL>, (int)(want < cap ? want : cap), kWarpsPerBlock * 32, 0, stream, x, idx, M, scale, shift, y, B, N,
+    const long long want = ((long long)B * M + kWarpsPerBlock - 1) / kWarpsPerBlock, cap = (long long)sm_count() * (MOD == kHeld ? kBlocks<VPL, MOD> : kBlocksPerSM);
+    launch_overlapped(layernorm_modulate_kernel<VPL, MOD>, (int)(want < cap ? want : cap), kWarpsPerBlock * 32, 0, stream, x, idx, M, scale, shift, y, B, N,
                       vec_per_row, eps, ci, co, err_word);
 }
 
@@ -118,7 +142,12 @@ int32_t launch_layernorm_modulate(const void *x, const int32_t *idx, int M, cons
     uint4 *ys = reinterpret_cast<uint4 *>(y);
     const int ci = (flags & ASTRAEA_LN_COMPACT_IN) ? 1 : 0, co = (flags & ASTRAEA_LN_COMPACT_OUT) ? 1 : 0;
     const int vpl = (vec_per_row + 31) / 32;
-#define LN(V) launch_ln<V>(stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word)
+    // Held vectors pay where a warp has one row or so: their loads run beside the row's, not behind its statistics.  us with the
+    // vectors read per row / held: 1200 x 1536 3.7 / 3.1, 1846 4.5 / 3.5, 2500 4.9 / 4.0, 4276 4.7 / 5.2; 1200 x 3072 5.7 / 4.5,
+    // 2400 6.2 / 7.5, 9001 20.7 / 20.8; 3000 x 1152 4.8 / 4.0, 13106 11.3 / 12.8, 32768 26.5 / 30.1.
+#define LN1(V, MOD) launch_ln<V, MOD>(stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word)
+#define LN(V) do { if (!sc && !sh) LN1(V, kPlain); else if (!sc || !sh) LN1(V, kEither); \
+    else if (10 * total <= 11ll * sm_count() * kBlocks<V, kHeld> * kWarpsPerBlock) LN1(V, kHeld); else LN1(V, kBoth); } while (0)
     if (vpl <= 2) LN(2);
     else if (vpl <= 4) LN(4);
     else if (vpl <= 5) LN(5);
@@ -127,6 +156,7 @@ int32_t launch_layernorm_modulate(const void *x, const int32_t *idx, int M, cons
     else if (vpl <= 12) LN(12);
     else LN(16);
 #undef LN
+#undef LN1
     return check_launch("astraea_layernorm_modulate");
 }
 
