@@ -1021,19 +1021,27 @@ __global__ void __launch_bounds__(ROWS) merge_parts_kernel(const Params p)
     const int r = idx / kChunksRow, c = idx - r * kChunksRow;
     const int m = m0 + r;
     if (m >= p.M) return;
-    const int tok = p.q_idx ? __ldcg(p.q_idx + (size_t)b * p.M + m) : m;
-    if ((unsigned)tok >= (unsigned)p.N_tok || (p.q_idx && m > 0 && __ldcg(p.q_idx + (size_t)b * p.M + m - 1) >= tok)) return;   // reported by the attention kernel
+    // everything that the thread reads is sent for at once: the kernel is one round trip to L2, not the three of list, LSE and rows
+    // (attention and merge of 1846 x 4276 x 24 heads of 64 65.0 -> 62.6 us, 2000 x 4000 x 4 28.5 -> 26.3, of 72 30.4 -> 27.8)
+    const int tok = p.q_idx ? __ldcg(p.q_idx + (size_t)b * p.M + m) : m, before = (p.q_idx && m > 0) ? __ldcg(p.q_idx + (size_t)b * p.M + m - 1) : -1;
     const size_t part0 = (size_t)blockIdx.y * p.split;
     float lse[8], mx = -INFINITY;
-    bool gave_up = false;
+    float4 x[8], y[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         lse[i] = -INFINITY;
         if (i < p.split) {
             lse[i] = __ldcg(p.part_lse + (part0 + i) * ROWS + r);
-            gave_up |= __float_as_uint(lse[i]) == kGaveUpLse;
-            mx = fmaxf(mx, lse[i]);
+            const float4 *src = reinterpret_cast<const float4 *>(p.part_o + ((part0 + i) * ROWS + r) * DH + c * 8);
+            x[i] = __ldcg(src); y[i] = __ldcg(src + 1);
         }
+    }
+    if ((unsigned)tok >= (unsigned)p.N_tok || before >= tok) return;   // reported by the attention kernel
+    bool gave_up = false;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        gave_up |= __float_as_uint(lse[i]) == kGaveUpLse;
+        mx = fmaxf(mx, lse[i]);
     }
     if (gave_up) return;                                            // a share was not finished (a wait ran out): the row stays as it is
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, wsum = 0.f;
@@ -1042,10 +1050,8 @@ __global__ void __launch_bounds__(ROWS) merge_parts_kernel(const Params p)
         if (i < p.split) {
             const float w = __expf(lse[i] - mx);
             wsum += w;
-            const float4 *src = reinterpret_cast<const float4 *>(p.part_o + ((part0 + i) * ROWS + r) * DH + c * 8);
-            const float4 a = __ldcg(src), d = __ldcg(src + 1);
-            acc[0] += w * a.x; acc[1] += w * a.y; acc[2] += w * a.z; acc[3] += w * a.w;
-            acc[4] += w * d.x; acc[5] += w * d.y; acc[6] += w * d.z; acc[7] += w * d.w;
+            acc[0] += w * x[i].x; acc[1] += w * x[i].y; acc[2] += w * x[i].z; acc[3] += w * x[i].w;
+            acc[4] += w * y[i].x; acc[5] += w * y[i].y; acc[6] += w * y[i].z; acc[7] += w * y[i].w;
         }
     }
     const float inv = 1.0f / wsum;
