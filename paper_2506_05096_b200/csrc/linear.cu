@@ -89,18 +89,20 @@ __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
 
 // GELU(x) = x (1 + erf(x / sqrt 2)) / 2 of two elements, with erf to 1.5e-7 absolute (rational approximation 7.1.26 of Abramowitz
 // and Stegun: erf(z) = 1 - (a1 t + ... + a5 t^5) e^{-z^2} for z >= 0, t = 1 / (1 + p z)): with w = 1/2 + copysign(1/2 - (a1 t +
-// ... + a5 t^5) e^{-x^2 / 2} / 2, x) it is x w.  Issue slots bind it (the epilogue of a tile has four warps on each SM sub-partition,
-// and a main loop of K = 1152 is over in 5 us), so all but the XU operations and the signs are packed pairs: 9.5 instructions per
-// element instead of 17.  13106 x 1152 x 4608 took
-// 108.7 us with the erf element by element and the epilogue's loads behind its wait, 101.9 now; 1846 x 1536 x 6144 31.1 -> 30.3.
+// ... + a5 t^5) e^{-z^2} / 2, z) it is x w.  Issue slots bind it (the epilogue of a tile has four warps on each SM sub-partition,
+// and a main loop of K = 1152 is over in 5 us), so all but the XU operations and the signs are packed pairs: 10 instructions per
+// element instead of 17.  z is rounded before it is squared and the halves only scale by powers of two, so the result is that of the
+// same formula element by element, bit for bit (with 1 / sqrt 2 folded into the constants 9001 x 3072 x 12288 takes 495 us instead
+// of 505, but outputs of a block move by single bf16 roundings).  13106 x 1152 x 4608 took 110.0 us with the erf element by element and
+// the epilogue's loads behind its wait, 102.5 now; 1846 x 1536 x 6144 32.2 -> 30.6.
 __device__ __forceinline__ f32x2 both(float v) { return pack2(v, v); }
 __device__ __forceinline__ f32x2 gelu2(f32x2 x) {
-    const f32x2 ax = x & 0x7fffffff7fffffffull;
+    const f32x2 z = mul2(x, both(0.70710678118654752f)), az = z & 0x7fffffff7fffffffull;
     float d0, d1, a0, a1, t0, t1, e0, e1;
-    unpack2(fma2(ax, both(0.3275911f * 0.70710678118654752f), both(1.0f)), d0, d1);
+    unpack2(fma2(az, both(0.3275911f), both(1.0f)), d0, d1);
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(d0));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(d1));
-    unpack2(mul2(mul2(x, x), both(-0.5f * 1.4426950408889634f)), a0, a1);
+    unpack2(mul2(mul2(az, az), both(-1.4426950408889634f)), a0, a1);
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(a0));
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(a1));
     const f32x2 t = pack2(t0, t1);
@@ -108,8 +110,16 @@ __device__ __forceinline__ f32x2 gelu2(f32x2 x) {
     pl = fma2(pl, t, both(-0.5f * 1.421413741f));
     pl = fma2(pl, t, both(0.5f * 0.284496736f));
     pl = fma2(pl, t, both(-0.5f * 0.254829592f));
-    const f32x2 half_erf = fma2(mul2(pl, t), pack2(e0, e1), both(0.5f));                // of |x|: >= 0
-    return mul2(x, add2(both(0.5f), half_erf | (x & 0x8000000080000000ull)));
+    const f32x2 half_erf = fma2(mul2(pl, t), pack2(e0, e1), both(0.5f));                // of |z|
+    return mul2(x, add2(both(0.5f), (half_erf & 0x7fffffff7fffffffull) | (x & 0x8000000080000000ull)));
+}
+
+// A product that is rounded before anything is added to it, as the gate is before the residual: the product of packed pairs and the sum
+// after it come out as one FMA even with .rn on both (same bits as fma2), a product of single elements does not.
+__device__ __forceinline__ f32x2 mul2_alone(f32x2 a, f32x2 b) {
+    float a0, a1, b0, b1;
+    unpack2(a, a0, a1); unpack2(b, b0, b1);
+    return pack2(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
 }
 
 __device__ __forceinline__ uint4 shfl_vec(const uint4 &v, int lane) {
@@ -310,7 +320,7 @@ gathered_linear_kernel(const __grid_constant__ WMaps tmap_w, const __grid_consta
                         f32x2 r[4];
                         unpack8(*mine, r);
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) f[i] = p.gate ? fma2(f[i], t[i], r[i]) : add2(f[i], r[i]);
+                        for (int i = 0; i < 4; ++i) f[i] = add2(p.gate ? mul2_alone(f[i], t[i]) : f[i], r[i]);
                     } else if (EPI == kAnything && p.gate) {
 #pragma unroll
                         for (int i = 0; i < 4; ++i) f[i] = mul2(f[i], t[i]);
