@@ -827,6 +827,9 @@ int32_t astraea_step_host(astraea_session *s, const void *x_cur, const void *q, 
     REQUIRE(s && x_cur && q && k && v && out, "astraea_step_host: null argument");
     REQUIRE(k_keep >= 0 && k_keep <= s->N_sel, "astraea_step_host: k_keep=%d outside [0, N_sel=%d]", k_keep, s->N_sel);
     REQUIRE(s->steps > 0 || k_keep == s->N_sel, "astraea_step_host: the first step of a session must compute every token (k_keep = N_sel)");
+    // looked at here for every path: a step of every token needs no scores
+    if (delta_mode < 0 || delta_mode > 2 || lse_mode < 0 || lse_mode > 1)
+        return fail(ASTRAEA_ERR_UNSUPPORTED, "astraea_step_host: unknown delta_mode %d or lse_mode %d", delta_mode, lse_mode);
     const int B = s->B, H = s->H, N = s->N, N_sel = s->N_sel, d = s->d, D = H * d;
     const int n_always = N - N_sel, M = k_keep + n_always;
     const size_t pitch = (size_t)D * 2, rows = (size_t)B * N;

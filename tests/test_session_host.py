@@ -1,0 +1,40 @@
+"""Host-buffer sessions on a model of the CUDA runtime (tests/session_host.cpp): results under every order that streams and events
+allow, steps that fail half way, arguments, and how much is sent for at a time."""
+import os
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2506_05096_b200", "csrc")
+
+
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
+    where = tmp_path_factory.mktemp("session_host")
+    for header in ("cuda_runtime.h", "cuda_bf16.h"):                  # the model takes their place
+        open(where / header, "w").close()
+    exe = str(where / "session_host")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-Wno-unknown-pragmas", "-I", str(where), "-I", CSRC, "-o", exe, os.path.join(HERE, "session_host.cpp")])
+    return exe
+
+
+def _run(program, *args):
+    r = subprocess.run([program] + [str(a) for a in args], stdout=subprocess.PIPE, timeout=120, text=True)
+    assert r.returncode == 0, (args, r.stdout)
+    return [int(v) for v in r.stdout.split()]
+
+
+# B, H, d, N_sel, n_always: one chunk; chunks of rows with a ragged last one; several batch elements; too many for the path by rows,
+# which go by head groups, one a head and several heads to a group
+SHAPES = [(1, 2, 64, 300, 7), (1, 8, 64, 4000, 96), (2, 3, 64, 700, 0), (12, 1, 64, 300, 0), (13, 2, 64, 300, 3), (13, 14, 72, 40, 1)]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_steps_in_any_order_of_the_streams(program, shape):
+    _run(program, "steps", *shape, 0, 8)
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_unknown_modes_are_refused_before_anything_is_sent_for(program, shape):
+    _run(program, "modes", *shape)
