@@ -807,29 +807,14 @@ static int32_t step_host_all_rows(astraea_session *s, const void *x_cur, const v
     return ASTRAEA_OK;
 }
 
-// the end of a step: everything that it sent for has ended
-static int32_t step_host_end(astraea_session *s)
-{
-    cudaError_t e = cudaStreamSynchronize(s->copy_out);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->copy_in);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->gather);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream2);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);      // the refresh of x_ref runs beside the attention
-    if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy out): %s", cudaGetErrorString(e));
-    s->steps++;
-    return astraea_poll_error(s->workspace, s->stream);
-}
+// Rough times of the attention and of the bus (four tensors in) in a step of M queries: 1e15 flop/s, 5e10 bytes/s.
+static double host_attn_s(const astraea_session *s, int M) { return 4.0 * s->B * s->H * (double)M * s->N * s->d / 1e15; }
+static double host_bus_s(const astraea_session *s) { return 4.0 * (double)s->tensor_bytes / 5e10; }
 
-int32_t astraea_step_host(astraea_session *s, const void *x_cur, const void *q, const void *k,
-                          const void *v, void *out, int k_keep,
-                          float w_alpha, float w_beta, int delta_mode, int lse_mode)
+// A step that moves q, k and v in and the output back in groups of heads.
+static int32_t step_host_groups(astraea_session *s, const void *x_cur, const void *q, const void *k, const void *v, void *out, int k_keep,
+                                float w_alpha, float w_beta, int delta_mode, int lse_mode)
 {
-    REQUIRE(s && x_cur && q && k && v && out, "astraea_step_host: null argument");
-    REQUIRE(k_keep >= 0 && k_keep <= s->N_sel, "astraea_step_host: k_keep=%d outside [0, N_sel=%d]", k_keep, s->N_sel);
-    REQUIRE(s->steps > 0 || k_keep == s->N_sel, "astraea_step_host: the first step of a session must compute every token (k_keep = N_sel)");
-    // looked at here for every path: a step of every token needs no scores
-    if (delta_mode < 0 || delta_mode > 2 || lse_mode < 0 || lse_mode > 1)
-        return fail(ASTRAEA_ERR_UNSUPPORTED, "astraea_step_host: unknown delta_mode %d or lse_mode %d", delta_mode, lse_mode);
     const int B = s->B, H = s->H, N = s->N, N_sel = s->N_sel, d = s->d, D = H * d;
     const int n_always = N - N_sel, M = k_keep + n_always;
     const size_t pitch = (size_t)D * 2, rows = (size_t)B * N;
@@ -843,16 +828,8 @@ int32_t astraea_step_host(astraea_session *s, const void *x_cur, const void *q, 
     // of whole 2*D-byte rows), which takes (N - M) / N of one tensor off the host-to-device traffic that bounds the step.
     // Worth it only while the bus bounds the step: the fetch kernels share the SMs with the attention, and on a step
     // whose attention takes longer than its transfers (the HunyuanVideo shape: 95 -> 101 ms) they only delay it.
-    // Rough rates: 1e15 flop/s for the attention, 5e10 bytes/s for the bus.
     const void *q_mapped = nullptr;
-    const double attn_s = 4.0 * B * H * (double)M * N * d / 1e15, bus_s = 4.0 * (double)s->tensor_bytes / 5e10;
-    // Every token: by rows where the attention takes no longer than q and x_cur on the bus, which arrive under it (N up to about
-    // 20000 whatever the other sizes); beyond that the attention must not wait for all of k and v, and the heads arrive in groups.
-    if (M == N && B <= kHostGroups && attn_s <= 0.5 * bus_s) {
-        const int32_t rc = step_host_all_rows(s, x_cur, q, k, v, out);
-        return rc != ASTRAEA_OK ? rc : step_host_end(s);
-    }
-    if (M < N && M > 0 && attn_s < bus_s) {
+    if (M < N && M > 0 && host_attn_s(s, M) < host_bus_s(s)) {
         cudaPointerAttributes attr;
         if (cudaPointerGetAttributes(&attr, q) == cudaSuccess && attr.type == cudaMemoryTypeHost && attr.devicePointer)
             q_mapped = attr.devicePointer;
@@ -935,7 +912,40 @@ int32_t astraea_step_host(astraea_session *s, const void *x_cur, const void *q, 
                                   width, rows, cudaMemcpyDeviceToHost, s->copy_out);
         if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy out): %s", cudaGetErrorString(e));
     }
-    return step_host_end(s);
+    return ASTRAEA_OK;
+}
+
+// The end of a step, whether it went well or not (rc): nothing that it sent for is under way afterwards, since the caller may free or
+// reuse its buffers.
+static int32_t step_host_end(astraea_session *s, int32_t rc)
+{
+    cudaError_t e = cudaSuccess;
+    for (cudaStream_t st : {s->copy_out, s->copy_in, s->gather, s->stream2, s->stream}) {      // (the refresh of x_ref runs beside the attention)
+        const cudaError_t f = cudaStreamSynchronize(st);
+        if (e == cudaSuccess) e = f;
+    }
+    if (rc != ASTRAEA_OK) return rc;
+    if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy out): %s", cudaGetErrorString(e));
+    s->steps++;
+    return astraea_poll_error(s->workspace, s->stream);
+}
+
+int32_t astraea_step_host(astraea_session *s, const void *x_cur, const void *q, const void *k,
+                          const void *v, void *out, int k_keep,
+                          float w_alpha, float w_beta, int delta_mode, int lse_mode)
+{
+    REQUIRE(s && x_cur && q && k && v && out, "astraea_step_host: null argument");
+    REQUIRE(k_keep >= 0 && k_keep <= s->N_sel, "astraea_step_host: k_keep=%d outside [0, N_sel=%d]", k_keep, s->N_sel);
+    REQUIRE(s->steps > 0 || k_keep == s->N_sel, "astraea_step_host: the first step of a session must compute every token (k_keep = N_sel)");
+    // looked at here for every path: a step of every token needs no scores
+    if (delta_mode < 0 || delta_mode > 2 || lse_mode < 0 || lse_mode > 1)
+        return fail(ASTRAEA_ERR_UNSUPPORTED, "astraea_step_host: unknown delta_mode %d or lse_mode %d", delta_mode, lse_mode);
+    // Every token: by rows where the attention takes no longer than q and x_cur on the bus, which arrive under it (N up to about
+    // 20000 whatever the other sizes); beyond that the attention must not wait for all of k and v, and the heads arrive in groups.
+    const bool by_rows = k_keep == s->N_sel && s->B <= kHostGroups && host_attn_s(s, s->N) <= 0.5 * host_bus_s(s);
+    const int32_t rc = by_rows ? step_host_all_rows(s, x_cur, q, k, v, out)
+                               : step_host_groups(s, x_cur, q, k, v, out, k_keep, w_alpha, w_beta, delta_mode, lse_mode);
+    return step_host_end(s, rc);
 }
 
 }  // extern "C"

@@ -38,3 +38,11 @@ def test_steps_in_any_order_of_the_streams(program, shape):
 @pytest.mark.parametrize("shape", SHAPES)
 def test_unknown_modes_are_refused_before_anything_is_sent_for(program, shape):
     _run(program, "modes", *shape)
+
+
+# the first step of a session, a later dense one and a sparse one behind them
+@pytest.mark.parametrize("k_keep,first", [(100, 1), (100, 0), (40, 0)])
+@pytest.mark.parametrize("shape", [(1, 2, 64, 100, 7), (3, 2, 64, 100, 0), (13, 2, 64, 100, 3)])
+def test_a_step_that_fails_leaves_nothing_under_way(program, shape, k_keep, first):
+    """Whichever call of the step fails: the caller may free its buffers when it gets the error."""
+    _run(program, "fail", *shape, k_keep, first)
