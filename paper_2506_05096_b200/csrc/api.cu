@@ -761,7 +761,7 @@ size_t astraea_session_last_h2d_bytes(const astraea_session *s) { return s ? s->
 // counters become 0 and x_cur becomes the reference input, so it goes straight to its place, last.  Whole rows cross the bus (column
 // slices of 144 / 288 bytes a row run at 32 / 42 GB/s, whole rows at 51): k and v of a batch element, then its q in chunks of
 // rows; a chunk's attention runs while the next ones arrive, alternately on two streams (see astraea_session), and its rows of the
-// output go back while the next one is computed.  (B1 H16 d72 N 16384: 4.66 -> 3.02 ms, of which the bus is 3.0; twelve smaller
+// output go back as soon as they are there.  (B1 H16 d72 N 16384: 4.66 -> 3.02 ms, of which the bus is 3.0; twelve smaller
 // steps of 0.1 to 1.7 ms are 1.05 to 2.2 times as fast.)
 static int32_t step_host_all_rows(astraea_session *s, const void *x_cur, const void *q, const void *k, const void *v, void *out)
 {
@@ -797,11 +797,19 @@ static int32_t step_host_all_rows(astraea_session *s, const void *x_cur, const v
             const int32_t rc = launch_sparse_attn(a, cs);
             if (rc != ASTRAEA_OK) return rc;
             e = cudaEventRecord(s->ev_attn[g], cs);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(s->copy_out, s->ev_attn[g], 0);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(mut(out, off), at(s->out_cache, off), n * row, cudaMemcpyDeviceToHost, s->copy_out);
         }
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(s->x_ref, x_cur, s->tensor_bytes, cudaMemcpyHostToDevice, s->copy_in);
+    // The way back is sent for behind everything else: with pageable buffers the call waits for each of these copies, and between the
+    // chunks that took 1.1 to 1.5 times as long (pageable, us: B1 H2 d64 N 16000 1623 -> 1194, B1 H2 d128 N 8000 1510 -> 1194, B2 H1
+    // d128 N 19900 5121 -> 3142, B1 H16 d72 N 16000 16743 -> 14781; pinned: no difference).
+    for (int b = 0, g = 0; b < B; ++b) {
+        for (int r = 0; r < N; r += step, ++g) {
+            const size_t off = b * one + r * row, bytes = (size_t)(N - r < step ? N - r : step) * row;
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s->copy_out, s->ev_attn[g], 0);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(mut(out, off), at(s->out_cache, off), bytes, cudaMemcpyDeviceToHost, s->copy_out);
+        }
+    }
     if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy out): %s", cudaGetErrorString(e));
     s->last_h2d_bytes = s->tensor_bytes * 4;
     return ASTRAEA_OK;

@@ -46,3 +46,10 @@ def test_unknown_modes_are_refused_before_anything_is_sent_for(program, shape):
 def test_a_step_that_fails_leaves_nothing_under_way(program, shape, k_keep, first):
     """Whichever call of the step fails: the caller may free its buffers when it gets the error."""
     _run(program, "fail", *shape, k_keep, first)
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_no_copy_in_waits_for_a_copy_back(program, shape):
+    """With pageable buffers a copy back holds up the call until it is over, so that whatever is sent for behind it comes late."""
+    copies_in, copies_back, late = _run(program, "steps", *shape, 0, 1)[:3]
+    assert copies_in > 0 and copies_back > 0 and late == 0
