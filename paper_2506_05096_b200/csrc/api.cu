@@ -800,6 +800,11 @@ static int32_t step_host_all_rows(astraea_session *s, const void *x_cur, const v
         }
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(s->x_ref, x_cur, s->tensor_bytes, cudaMemcpyHostToDevice, s->copy_in);
+    const uintptr_t o = reinterpret_cast<uintptr_t>(out), x = reinterpret_cast<uintptr_t>(x_cur);
+    if (o < x + s->tensor_bytes && x < o + s->tensor_bytes) {      // one buffer for both: it is read before it is written, as in the other path
+        if (e == cudaSuccess) e = cudaEventRecord(s->ev_x, s->copy_in);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s->copy_out, s->ev_x, 0);
+    }
     // The way back is sent for behind everything else: with pageable buffers the call waits for each of these copies, and between the
     // chunks that took 1.1 to 1.5 times as long (pageable, us: B1 H2 d64 N 16000 1623 -> 1194, B1 H2 d128 N 8000 1510 -> 1194, B2 H1
     // d128 N 19900 5121 -> 3142, B1 H16 d72 N 16000 16743 -> 14781; pinned: no difference).

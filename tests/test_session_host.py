@@ -31,8 +31,10 @@ SHAPES = [(1, 2, 64, 300, 7), (1, 8, 64, 4000, 96), (2, 3, 64, 700, 0), (12, 1, 
 
 
 @pytest.mark.parametrize("shape", SHAPES)
-def test_steps_in_any_order_of_the_streams(program, shape):
-    _run(program, "steps", *shape, 0, 8)
+@pytest.mark.parametrize("shared", [0, 1])
+def test_steps_in_any_order_of_the_streams(program, shape, shared):
+    """shared: the output goes back into the buffer that x_cur came from."""
+    _run(program, "steps", *shape, shared, 8)
 
 
 @pytest.mark.parametrize("shape", SHAPES)
