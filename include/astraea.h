@@ -453,7 +453,8 @@ void    astraea_schedule_destroy(astraea_schedule *schedule);
  * their own: x_cur goes first, q / k / v follow in up to twelve groups of heads, the attention
  * of a group starts when its heads have arrived, and the group's columns of the output
  * go back while the next group is computed.  A step that computes every token and is bound by the bus moves whole rows
- * instead: k and v, then q in chunks of rows, a chunk's attention and its way back under the next ones, x_cur last.
+ * instead: k and v of a batch element (of several small ones), then q in chunks of rows, a chunk's attention and its way back
+ * under the next ones, x_cur last.
  * The results are those of astraea_step.
  * astraea_session_create allocates device memory (cudaMalloc) on the current device;
  * the first step of a session must be run with k_keep = N_sel (all tokens computed) to

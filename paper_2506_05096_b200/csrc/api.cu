@@ -761,36 +761,49 @@ size_t astraea_session_last_h2d_bytes(const astraea_session *s) { return s ? s->
 // counters become 0 and x_cur becomes the reference input, so it goes straight to its place, last.  Whole rows cross the bus (column
 // slices of 144 / 288 bytes a row run at 32 / 42 GB/s, whole rows at 51): k and v of a batch element, then its q in chunks of
 // rows; a chunk's attention runs while the next ones arrive, alternately on two streams (see astraea_session), and its rows of the
-// output go back as soon as they are there.  (B1 H16 d72 N 16384: 4.66 -> 3.02 ms, of which the bus is 3.0; twelve smaller
-// steps of 0.1 to 1.7 ms are 1.05 to 2.2 times as fast.)
+// output go back as soon as they are there.  (B1 H16 d72 N 16384: 4.66 -> 3.02 ms, of which the bus is 3.0.)
 static int32_t step_host_all_rows(astraea_session *s, const void *x_cur, const void *q, const void *k, const void *v, void *out)
 {
     const int B = s->B, H = s->H, N = s->N, d = s->d, D = H * d;
     const size_t row = (size_t)D * 2, one = (size_t)N * row;
-    // chunks of at least 1 MB and whole units of 256 queries, up to kHostGroups in all
-    const int most = kHostGroups / B, want = (int)(one >> 20) < 1 ? 1 : (int)(one >> 20);
-    const int chunks = want < most ? want : most, step = ((N + chunks - 1) / chunks + 255) / 256 * 256;
+    // Batch elements that go together: half of all, between 1 and 2 MB, since every copy costs the bus 4 us (twelve elements of
+    // 38 KB, one by one: 339 us, by head groups 198, together 177).
+    const size_t half_all = s->tensor_bytes / 2, least = half_all < 1000000 ? 1000000 : half_all < 2000000 ? half_all : 2000000;
+    const size_t fill = (least + one - 1) / one;
+    const int per = fill < (size_t)B ? (int)fill : B, batches = (B + per - 1) / per;
+    // Chunks of rows of one element: at least 1.5 MB, up to kHostGroups in all.  Where a chunk of that size arrives faster than its
+    // attention is done (a unit of 256 queries takes 0.6 us per 64 keys, two chunks run at a time: 234 bytes a key), chunks are longer, up
+    // to units for half of the SMs (2 heads of 128 channels, N 16000: chunks of 2304 rows = 18 units 1138 us, by head groups 956, 796
+    // now).
+    const size_t pace = (size_t)N * 234 / row, half = (size_t)((sm_count() / 2 + H - 1) / H) * 256, short_ = (1500000 + row - 1) / row;
+    const size_t rows = pace < half ? pace : half;
+    const int fit = per > 1 ? 1 : (int)(N / (rows > short_ ? rows : short_)), most = kHostGroups / batches;
+    const int chunks = fit < 1 ? 1 : fit < most ? fit : most, step = ((N + chunks - 1) / chunks + 255) / 256 * 256;
     auto at = [](const void *p, size_t bytes) { return static_cast<const char *>(p) + bytes; };
     auto mut = [](void *p, size_t bytes) { return static_cast<char *>(p) + bytes; };
+    size_t off[kHostGroups], bytes[kHostGroups];             // of a chunk
+    int n_chunks = 0;
     cudaError_t e = cudaMemsetAsync(s->n_skip, 0, (size_t)B * s->N_sel * 4, s->copy_in);
-    for (int b = 0, g = 0; b < B; ++b) {
-        if (e == cudaSuccess) e = cudaMemcpyAsync(mut(s->k, b * one), at(k, b * one), one, cudaMemcpyHostToDevice, s->copy_in);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(mut(s->v, b * one), at(v, b * one), one, cudaMemcpyHostToDevice, s->copy_in);
-        for (int r = 0; r < N; r += step, ++g) {
-            const int n = N - r < step ? N - r : step;
-            const size_t off = b * one + r * row;
+    for (int b = 0; b < B; b += per) {
+        const int nb = B - b < per ? B - b : per;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(mut(s->k, b * one), at(k, b * one), nb * one, cudaMemcpyHostToDevice, s->copy_in);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(mut(s->v, b * one), at(v, b * one), nb * one, cudaMemcpyHostToDevice, s->copy_in);
+        for (int r = 0; r < N; r += step) {
+            const int n = N - r < step ? N - r : step, g = n_chunks++;
+            off[g] = b * one + r * row;
+            bytes[g] = nb > 1 ? nb * one : n * row;
             cudaStream_t cs = (g & 1) ? s->stream2 : s->stream;
-            if (e == cudaSuccess) e = cudaMemcpyAsync(mut(s->q, off), at(q, off), n * row, cudaMemcpyHostToDevice, s->copy_in);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(mut(s->q, off[g]), at(q, off[g]), bytes[g], cudaMemcpyHostToDevice, s->copy_in);
             if (e == cudaSuccess) e = cudaEventRecord(s->ev_in[g], s->copy_in);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, s->ev_in[g], 0);
             if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy in): %s", cudaGetErrorString(e));
             AttnArgs a;
-            a.q = mut(s->q, off); a.k = mut(s->k, b * one); a.v = mut(s->v, b * one);
+            a.q = mut(s->q, off[g]); a.k = mut(s->k, b * one); a.v = mut(s->v, b * one);
             a.q_sb = a.k_sb = a.v_sb = (int64_t)N * D;
             a.q_sh = a.k_sh = a.v_sh = d;
             a.q_sn = a.k_sn = a.v_sn = D;
-            a.q_idx = nullptr; a.M = n; a.out = mut(s->out_cache, off); a.lse_out = s->lse_cache + (size_t)b * H * N + r;
-            a.B = 1; a.H = H; a.N = N; a.d = d; a.N_tok = N;
+            a.q_idx = nullptr; a.M = n; a.out = mut(s->out_cache, off[g]); a.lse_out = s->lse_cache + (size_t)b * H * N + r;
+            a.B = nb; a.H = H; a.N = N; a.d = d; a.N_tok = N;
             a.scale = 1.0f / sqrtf((float)d);
             a.flags = 0;
             a.err_word = reinterpret_cast<int *>(s->workspace);
@@ -808,12 +821,9 @@ static int32_t step_host_all_rows(astraea_session *s, const void *x_cur, const v
     // The way back is sent for behind everything else: with pageable buffers the call waits for each of these copies, and between the
     // chunks that took 1.1 to 1.5 times as long (pageable, us: B1 H2 d64 N 16000 1623 -> 1194, B1 H2 d128 N 8000 1510 -> 1194, B2 H1
     // d128 N 19900 5121 -> 3142, B1 H16 d72 N 16000 16743 -> 14781; pinned: no difference).
-    for (int b = 0, g = 0; b < B; ++b) {
-        for (int r = 0; r < N; r += step, ++g) {
-            const size_t off = b * one + r * row, bytes = (size_t)(N - r < step ? N - r : step) * row;
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(s->copy_out, s->ev_attn[g], 0);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(mut(out, off), at(s->out_cache, off), bytes, cudaMemcpyDeviceToHost, s->copy_out);
-        }
+    for (int g = 0; g < n_chunks; ++g) {
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s->copy_out, s->ev_attn[g], 0);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(mut(out, off[g]), at(s->out_cache, off[g]), bytes[g], cudaMemcpyDeviceToHost, s->copy_out);
     }
     if (e != cudaSuccess) return fail(ASTRAEA_ERR_CUDA, "astraea_step_host (copy out): %s", cudaGetErrorString(e));
     s->last_h2d_bytes = s->tensor_bytes * 4;

@@ -7,8 +7,10 @@ from paper_2506_05096_b200 import binding as A
 pytestmark = pytest.mark.gpu
 
 
-# three chunks of a batch element with a ragged last one; one chunk; two tokens more than the chunks' whole units; a chunk per batch element
-@pytest.mark.parametrize("B,H,d,N_v,N_t", [(2, 6, 64, 4070, 30), (1, 2, 64, 300, 7), (1, 3, 128, 3074, 0), (7, 8, 64, 600, 0)])
+# two chunks of a batch element with a ragged last one; one chunk, of few tokens and of more; four and three batch elements that go
+# together; all of them; eight chunks, the last one of two tokens
+@pytest.mark.parametrize("B,H,d,N_v,N_t", [(2, 6, 64, 4070, 30), (1, 2, 64, 300, 7), (1, 3, 128, 3074, 0), (7, 8, 64, 600, 0), (5, 2, 64, 300, 2),
+                                           (1, 27, 128, 1790, 4)])
 def test_dense_steps_by_rows_equal_the_device_path(B, H, d, N_v, N_t):
     """A dense first step, a sparse one, a dense one again and a sparse one behind it, against the single calls on device buffers (all
     keys in every CTA, as in a session): bit-identical outputs, so the LSE cache, the counters and the reference inputs that the

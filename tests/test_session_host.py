@@ -25,9 +25,9 @@ def _run(program, *args):
     return [int(v) for v in r.stdout.split()]
 
 
-# B, H, d, N_sel, n_always: one chunk; chunks of rows with a ragged last one; several batch elements; too many for the path by rows,
-# which go by head groups, one a head and several heads to a group
-SHAPES = [(1, 2, 64, 300, 7), (1, 8, 64, 4000, 96), (2, 3, 64, 700, 0), (12, 1, 64, 300, 0), (13, 2, 64, 300, 3), (13, 14, 72, 40, 1)]
+# B, H, d, N_sel, n_always: one chunk; two chunks of rows, the second one shorter; batch elements that go together, all of them, and two and
+# one; too many for the path by rows, which go by head groups, one a head and several heads to a group
+SHAPES = [(1, 2, 64, 300, 7), (1, 8, 64, 4000, 60), (2, 3, 64, 700, 0), (12, 1, 64, 300, 0), (3, 8, 64, 1100, 1), (13, 2, 64, 300, 3), (13, 14, 72, 40, 1)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
@@ -55,3 +55,16 @@ def test_no_copy_in_waits_for_a_copy_back(program, shape):
     """With pageable buffers a copy back holds up the call until it is over, so that whatever is sent for behind it comes late."""
     copies_in, copies_back, late = _run(program, "steps", *shape, 0, 1)[:3]
     assert copies_in > 0 and copies_back > 0 and late == 0
+
+
+def test_small_batch_elements_share_their_copies(program):
+    """No more copies than by head groups (x_cur, and q, k and v of each of up to twelve groups)."""
+    for B, H, N in ((2, 1, 300), (5, 2, 300), (12, 1, 300), (12, 4, 100)):
+        copies_in, _, _, *ctas = _run(program, "steps", B, H, 64, N, 0, 0, 3)
+        assert copies_in <= 3 * H + 1 and sum(ctas) == B * H * ((N + 255) // 256)
+
+
+def test_chunks_of_a_long_sequence_of_few_heads_fill_the_chip(program):
+    """126 CTAs of 250 key tiles: cut so that the two launches that run at a time leave no more than a third of the 148 SMs idle."""
+    ctas = _run(program, "steps", 1, 2, 128, 15900, 0, 0, 1)[3:]
+    assert all(2 * c > 98 for c in ctas), ctas
