@@ -27,9 +27,19 @@ constexpr int kMaxVecPerLane = 16;     // rows of up to 32 * 16 * 8 = 4096 chann
 enum { kPlain = 0,      // there are none
        kBoth = 1,       // both are there, read from L1 for every row
        kHeld = 2,       // both are there, each warp keeps its lane's part of them in registers: fewer blocks of an SM
-       kEither = 3 };   // one of them
+       kEither = 3 };   // one of them (or both, see kTestedRows10)
 template <int VPL, int MOD> constexpr int kBlocks = MOD == kHeld ? (VPL <= 2 ? 8 : VPL <= 5 ? 5 : VPL <= 6 ? 4 : VPL <= 12 ? 3 : 2)
                                                                  : VPL <= 6 ? 8 : VPL <= 8 ? 6 : 4;
+
+// Ten times the rows a warp (of the blocks that the held form has room for) up to which a form is taken.  Held vectors pay where a warp
+// has one row or so: their loads run beside the row's, not behind its statistics.  us with the vectors read per row / held, at 1.0, 1.2
+// and 1.4 rows a warp: 512 channels 3.4 / 3.3, from 1.05 on 3.4 / 4.1; 1024 4.6 / 3.1, 4.7 / 4.0, 4.8 / 4.7; 1152 4.9 / 3.5, 5.1 / 4.7,
+// 5.2 / 5.4; 1536 3.7 / 3.3, 4.8 / 4.5, 4.8 / 5.1; 2048 5.3 / 3.3, 5.5 / 4.6, 5.6 / 5.5; 3072 6.3 / 5.4, at 1.05 6.6 / 7.4; 4096 6.9 / 4.4, at
+// 1.1 7.4 / 7.1, at 1.2 7.7 / 7.8.  Long launches: 13106 x 1152 11.3 / 12.8, 9001 x 3072 20.7 / 20.8.
+template <int VPL> constexpr long long kHeldRows10 = VPL <= 2 || VPL == 12 ? 10 : VPL == 16 ? 11 : VPL == 8 ? 14 : 12;
+// With three to five vectors a lane the form that tests for the vectors as it goes is the fastest between the two: 4144 x 1024 4.2 us where
+// kBoth takes 4.8, 4144 x 1152 4.8 and 5.2; from 1.8 rows a warp on it is the slowest (5328 x 1024 6.0 and 4.6).
+template <int VPL> constexpr long long kTestedRows10 = VPL == 4 ? 16 : VPL == 5 ? 14 : 0;
 
 // VPL: 16-byte vectors per lane (vec_per_row <= 32 * VPL)
 template <int VPL, int MOD>
@@ -142,12 +152,11 @@ int32_t launch_layernorm_modulate(const void *x, const int32_t *idx, int M, cons
     uint4 *ys = reinterpret_cast<uint4 *>(y);
     const int ci = (flags & ASTRAEA_LN_COMPACT_IN) ? 1 : 0, co = (flags & ASTRAEA_LN_COMPACT_OUT) ? 1 : 0;
     const int vpl = (vec_per_row + 31) / 32;
-    // Held vectors pay where a warp has one row or so: their loads run beside the row's, not behind its statistics.  us with the
-    // vectors read per row / held: 1200 x 1536 3.7 / 3.1, 1846 4.5 / 3.5, 2500 4.9 / 4.0, 4276 4.7 / 5.2; 1200 x 3072 5.7 / 4.5,
-    // 2400 6.2 / 7.5, 9001 20.7 / 20.8; 3000 x 1152 4.8 / 4.0, 13106 11.3 / 12.8, 32768 26.5 / 30.1.
+#define kHeldWarps(V) (sm_count() * kBlocks<V, kHeld> * kWarpsPerBlock)
 #define LN1(V, MOD) launch_ln<V, MOD>(stream, xs, idx, rows, sc, sh, ys, B, N, vec_per_row, eps, ci, co, err_word)
 #define LN(V) do { if (!sc && !sh) LN1(V, kPlain); else if (!sc || !sh) LN1(V, kEither); \
-    else if (10 * total <= 11ll * sm_count() * kBlocks<V, kHeld> * kWarpsPerBlock) LN1(V, kHeld); else LN1(V, kBoth); } while (0)
+    else if (10 * total <= kHeldRows10<V> * kHeldWarps(V)) LN1(V, kHeld); \
+    else if (10 * total <= kTestedRows10<V> * kHeldWarps(V)) LN1(V, kEither); else LN1(V, kBoth); } while (0)
     if (vpl <= 2) LN(2);
     else if (vpl <= 4) LN(4);
     else if (vpl <= 5) LN(5);
@@ -157,6 +166,7 @@ int32_t launch_layernorm_modulate(const void *x, const int32_t *idx, int M, cons
     else LN(16);
 #undef LN
 #undef LN1
+#undef kHeldWarps
     return check_launch("astraea_layernorm_modulate");
 }
 
