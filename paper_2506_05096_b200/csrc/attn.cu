@@ -1161,15 +1161,17 @@ int32_t launch_dh(const AttnArgs &a, cudaStream_t stream, SplitPlan plan = Split
     // stands for all of them and errs on the side of the scatter.)
     const long long copy_rows = (long long)a.B * a.M;
     const double copy_us = a.copy_dst ? (double)((copy_rows + grid - 1) / grid) * a.copy_elems * 2 / 4096 : 0.0;
-    // A launch that leaves SMs idle gets CTAs that only copy, at about 30 KB a microsecond each, if they are done within the same
-    // limit; its attention CTAs, which live for a few key tiles there, then copy nothing.  (Step of 128 x 256 tokens, 2 heads of 64: with
-    // the copying warp in the pass's barrier the CTA waited 4.7 us for it; graph 15.6 -> 11.8 us, step behind a copy of the LSE
-    // cache 20.3 -> 17.4; 250 x 500 tokens, 3 heads of 128: 21.3 -> 19.7; launches of 120 units and more: no difference.)
-    const double copy_all = (double)copy_rows * a.copy_elems * 2;
+    // A launch of few key tiles that leaves SMs idle gets CTAs that only copy, at about 30 KB a microsecond each, if they are done within the
+    // same limit; its attention CTAs then copy nothing.  (Step of 128 x 256 tokens, 2 heads of 64: with the copying warp in the pass's
+    // barrier the CTA waited 4.7 us for it; graph 15.6 -> 11.8 us, step behind a copy of the LSE cache 20.3 -> 17.4.  24 heads of 128, copying
+    // warp / CTAs: 125 x 250 tokens 19.6 / 16.6 us, 500 x 1000 32.3 / 29.6, 750 x 1500 38.0 / 35.5, 900 x 3000 62.0 / 61.0; from 3500 keys
+    // on no gain: 1200 x 3517 69.1 / 69.9, 12 heads 2500 x 5000 76.6 / 77.4, 2400 x 8000 118.3 / 119.0.)
+    const int tiles = (a.N + C::kBlockN - 1) / C::kBlockN;
+    const double limit_us = 0.4 * tiles * units_per_cta / p.split + 4.0, copy_all = (double)copy_rows * a.copy_elems * 2;
     const int idle = slots - (int)grid;
     const int wanted = a.copy_dst ? (int)(copy_all / 8192 < 1024 ? copy_all / 8192 + 1 : 1024) : 0, copy_ctas = idle < wanted ? idle : wanted;
-    const bool copy_idle = copy_ctas > 0 && copy_all / copy_ctas <= 30e3 * (0.4 * ((a.N + C::kBlockN - 1) / C::kBlockN) * units_per_cta / p.split + 4.0);
-    const bool copy_here = copy_idle || a.copy_dst && (long long)a.B * a.N_tok * (a.copy_elems / 8) < 0x7fffffffll && copy_us <= 0.4 * ((a.N + C::kBlockN - 1) / C::kBlockN) * units_per_cta / p.split + 4.0;
+    const bool copy_idle = copy_ctas > 0 && tiles <= 48 && copy_all / copy_ctas <= 30e3 * limit_us;
+    const bool copy_here = copy_idle || (a.copy_dst && (long long)a.B * a.N_tok * (a.copy_elems / 8) < 0x7fffffffll && copy_us <= limit_us);
     p.copy_src = copy_here ? reinterpret_cast<const uint4 *>(a.copy_src) : nullptr;
     p.copy_dst = copy_here ? reinterpret_cast<uint4 *>(a.copy_dst) : nullptr;
     p.copy_bytes = (uint32_t)a.copy_elems * 2;

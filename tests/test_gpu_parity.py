@@ -924,20 +924,35 @@ def test_small_ctas_walk_over_units(oracle, H, N, M, amp, lse_tol):
 
 # ------------------------------------------------------------------ refresh of the reference inputs beside the attention
 @pytest.mark.parametrize("B,H,d,N_v,n_always,k", [
-    (1, 2, 64, 256, 0, 1),            # one row of 256 bytes: one lane of one batch
-    (2, 3, 72, 700, 5, 333),          # 432-byte rows, nine to a batch, both batch elements in one CTA's share
-    (1, 32, 64, 600, 0, 599),         # 4096-byte rows: a row is a batch
-    (1, 33, 64, 400, 7, 100),         # 4224 bytes: a whole piece and one of 128 bytes
-    (1, 24, 128, 2500, 0, 1200),      # 6144-byte rows, many CTAs
+    # few keys and idle SMs: CTAs of their own copy
+    (1, 2, 64, 256, 0, 1),            # one row of 256 bytes
+    (2, 3, 72, 700, 5, 333),          # 432-byte rows
+    (1, 32, 64, 600, 0, 599),         # 4096-byte rows
+    (1, 33, 64, 400, 7, 100),         # 4224 bytes
+    (1, 24, 128, 2500, 0, 1200),      # 6144-byte rows, many of them
     (1, 8, 128, 300, 0, 300),         # every row
     (2, 16, 72, 40, 3, 0),            # always-kept rows only
     (1, 40, 72, 64, 0, 60),           # one key tile, 5760-byte rows
+    # more than 48 key tiles, or no idle SM: the copying warp of every attention CTA does
+    (1, 2, 64, 3200, 0, 1),           # one row of 256 bytes: one lane of one batch
+    (2, 3, 72, 3200, 5, 333),         # 432-byte rows, nine to a batch, both batch elements in one CTA's share
+    (1, 32, 64, 3200, 0, 1500),       # 4096-byte rows: a row is a batch
+    (1, 33, 64, 3200, 7, 100),        # 4224 bytes: a whole piece and one of 128 bytes
+    (2, 16, 72, 3200, 0, 500),        # 2304-byte rows
+    (1, 24, 128, 3200, 0, 1600),      # 6144-byte rows, more units than SMs
+    (4, 40, 64, 500, 0, 300),         # small CTAs with several units each: counted ahead in the barrier of the first one only
+    (6, 33, 64, 130, 1, 129),         # the same over three key tiles
 ])
 def test_step_refreshes_reference_rows(B, H, d, N_v, n_always, k):
-    """astraea_step leaves x_ref bit-equal to x_cur in the selected rows and untouched elsewhere, whichever kernel copies."""
+    """astraea_step leaves x_ref bit-equal to x_cur in the selected rows and untouched elsewhere, whichever warps copy."""
     g = torch.Generator(device="cuda")
     g.manual_seed(N_v + k)
     N, D, M = N_v + n_always, H * d, k + n_always
+    plan = A.astraea_sparse_attn_plan(B, H, N, M, d)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    units = B * H * -(-M // (128 if plan["small_ctas"] else 256)) + plan["split_units"] * (plan["split"] - 1)
+    copying_warp = N > 48 * 64 or units >= n_sm * (2 if plan["small_ctas"] else 1)
+    assert copying_warp == (N_v == 3200 or B > 2)                     # the shapes are on the side of the rule that their comments say
     mk = lambda: torch.randn(B, N, D, device="cuda", dtype=torch.bfloat16, generator=g)  # noqa: E731
     x, old, q, kk, v, out = (mk() for _ in range(6))
     ref = Guarded((B, N, D), torch.bfloat16, init=old)
