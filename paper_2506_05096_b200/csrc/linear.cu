@@ -30,6 +30,7 @@
 // for no further copy, the other CTA of the pair runs into its own limit, and both run out; they leave together, when the copies
 // and MMAs that were under way have ended.
 #include "common.cuh"
+#include "linear_tiles.cuh"
 #include "sm100_ptx.cuh"
 #include "bounded_wait.cuh"
 
@@ -38,7 +39,7 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kRowsCta = 128, kBM = 2 * kRowsCta, kBK = 64;
+constexpr int kRowsCta = kBM / 2, kBK = 64;
 constexpr int kAccSets = 2;                              // accumulators in TMEM: the epilogue runs under the next main loop
 // Epilogue warps: four cover the CTA's 128 rows (one TMEM lane quarter each); kEpiSplit such groups share the columns.
 // Four groups: a tile of a short contraction (K = 1152: 18 stages) is over in 5 us, and two groups take 6 us for its
@@ -48,7 +49,6 @@ constexpr int kEpiWarps = 4 * kEpiSplit, kGatherWarps = 2;
 constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kTmaWarp + 1, kFirstGatherWarp = kMmaWarp + 1;
 constexpr int kEpiStageBytes = 32 * 64;                  // per epilogue warp: 32 rows x 32 bf16 columns on their way to / from global memory
 
-constexpr int kMaxBN = 256, kBNStep = 32;                // columns of an output tile: what cta_group::2 takes at M = 256
 constexpr int kStages = 6;
 constexpr int kABytes = kRowsCta * kBK * 2, kBBytes = kMaxBN / 2 * kBK * 2;
 constexpr int kBarBytes = 256;
@@ -490,28 +490,6 @@ int32_t make_matrix_map(CUtensorMap *map, const void *base, long long rows, int 
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(ASTRAEA_ERR_INVALID_ARG, "astraea_gathered_linear: tensor map of %s rejected (CUresult %d)", what, (int)r);
     return ASTRAEA_OK;
-}
-
-// Columns that a matrix takes in a launch over n_mats of them, and the column tiles of the launch.
-int mat_columns(int N_out, int n_mats, int bn) { return n_mats == 1 ? 0 : (N_out + bn / 2 - 1) / (bn / 2) * (bn / 2); }
-int column_tiles(int N_out, int n_mats, int bn) { return ((n_mats == 1 ? N_out : n_mats * mat_columns(N_out, n_mats, bn)) + bn - 1) / bn; }
-
-// Columns of an output tile.  The launch takes ceil(tiles / pairs) rounds, and a round of narrower tiles costs less, but
-// not in proportion (the rows of x are streamed for fewer columns): measured 0.60-0.67 of a 256-column round at 128
-// columns on seven shapes.  256 unless another width saves 3 % by that estimate, which happens where a launch has a
-// few rounds only or the last tile of a row is mostly padding.  Several matrices: half a tile is whole groups of 32 columns, since
-// the epilogue's groups must not straddle two matrices.
-int choose_bn(long long rows, int N_out, int n_mats, int pairs)
-{
-    const long long tiles_m = (rows + kBM - 1) / kBM;
-    int best_bn = kMaxBN;
-    double best = 0.0;
-    for (int bn = kMaxBN; bn >= kBNStep; bn -= n_mats == 1 ? kBNStep : 64) {
-        const long long tiles = tiles_m * column_tiles(N_out, n_mats, bn);
-        const double t = (double)((tiles + pairs - 1) / pairs) * (0.26 + 0.74 * bn / kMaxBN);
-        if (best == 0.0 || t < 0.97 * best) { best = t; best_bn = bn; }
-    }
-    return best_bn;
 }
 
 template <bool DENSE, bool MULTI, int EPI>
