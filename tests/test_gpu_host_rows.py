@@ -1,4 +1,4 @@
-"""Host-buffer sessions: steps that compute every token move whole rows, in chunks of rows."""
+"""Host-buffer sessions: steps that compute every token move whole rows, in chunks of rows, or head groups."""
 import pytest
 import torch
 
@@ -10,8 +10,12 @@ pytestmark = pytest.mark.gpu
 # two chunks of a batch element with a ragged last one; one chunk, of few tokens and of more; four and three batch elements that go
 # together; all of them; eight chunks, the last one of two tokens
 @pytest.mark.parametrize("B,H,d,N_v,N_t", [(2, 6, 64, 4070, 30), (1, 2, 64, 300, 7), (1, 3, 128, 3074, 0), (7, 8, 64, 600, 0), (5, 2, 64, 300, 2),
-                                           (1, 27, 128, 1790, 4)])
-def test_dense_steps_by_rows_equal_the_device_path(B, H, d, N_v, N_t):
+                                           (1, 27, 128, 1790, 4),
+                                           # by head groups: too many batch elements, a group a head and two heads in some (head_dim 64: the
+                                           # bits of the others depend on the CTA shape, which a launch of fewer heads may change); N on both
+                                           # sides of the line at 20000
+                                           (13, 2, 64, 300, 3), (13, 14, 64, 200, 5), (1, 1, 64, 20090, 10), (1, 1, 64, 19980, 10)])
+def test_dense_steps_equal_the_device_path(B, H, d, N_v, N_t):
     """A dense first step, a sparse one, a dense one again and a sparse one behind it, against the single calls on device buffers (all
     keys in every CTA, as in a session): bit-identical outputs, so the LSE cache, the counters and the reference inputs that the
     dense steps leave behind are right, too."""
@@ -26,7 +30,8 @@ def test_dense_steps_by_rows_equal_the_device_path(B, H, d, N_v, N_t):
     for step, k in enumerate((N_v, N_v // 3, N_v, N_v // 2)):
         M = k + N_t
         x, q, kk, v = (torch.randn(B, N, D, dtype=torch.bfloat16, device="cuda", generator=g) for _ in range(4))
-        sess.step_host(*(t.cpu().pin_memory() for t in (x, q, kk, v)), host_out, k)
+        host = [t.cpu() for t in (x, q, kk, v)]
+        sess.step_host(*(host if step == 2 else (t.pin_memory() for t in host)), host_out, k)       # the second dense step from pageable memory
         if x_ref is None:
             x_ref = x.clone()
         sel = torch.empty(B, M, dtype=torch.int32, device="cuda")

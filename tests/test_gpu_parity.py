@@ -674,9 +674,9 @@ def test_step_chain_of_fifty_steps_reduced_hunyuan_shape(oracle):
 
 # ------------------------------------------------------------- host-buffer session
 def test_session_step_host_equals_the_device_path_and_the_oracle(oracle):
-    """astraea_step_host (pinned host buffers, copies overlapped with the attention by head group) against
-    astraea_step on device buffers from the same initial state: bit-identical outputs over three steps; the first,
-    dense step also against the oracle."""
+    """astraea_step_host (pinned host buffers, copies overlapped with the attention: the dense step by rows, the others by head
+    group) against astraea_step on device buffers from the same initial state: bit-identical outputs over three steps; the
+    first, dense step also against the oracle."""
     w = synth.Workload("mini-session", B=2, H=6, d=64, N_v=700, N_t=30)
     inp = synth.make_step_inputs(w, 11)
     B, N, H, d, N_sel, n_always = w.B, w.N, w.H, w.d, w.N_v, w.N_t
