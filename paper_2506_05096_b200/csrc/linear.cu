@@ -92,13 +92,14 @@ __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
 // ... + a5 t^5) e^{-z^2} / 2, z) it is x w.  Issue slots bind it (the epilogue of a tile has four warps on each SM sub-partition,
 // and a main loop of K = 1152 is over in 5 us), so all but the XU operations and the signs are packed pairs: 10 instructions per
 // element instead of 17.  z is rounded before it is squared and the halves only scale by powers of two, so the result is that of the
-// same formula element by element, bit for bit (with 1 / sqrt 2 folded into the constants 9001 x 3072 x 12288 takes 495 us instead
-// of 505, but outputs of a block move by single bf16 roundings).  13106 x 1152 x 4608 took 110.0 us with the erf element by element and
-// the epilogue's loads behind its wait, 102.5 now; 1846 x 1536 x 6144 32.2 -> 30.6.
+// same formula element by element, bit for bit (with 1 / sqrt 2 folded into the constants 9001 x 3072 x 12288 takes 488 us instead
+// of 491, but outputs of a block move by single bf16 roundings; with |z| masked out of a packed product 493).  13106 x 1152 x 4608 took
+// 110.0 us with the erf element by element and the epilogue's loads behind its wait, 101.6 now; 1846 x 1536 x 6144 32.2 -> 30.7.
 __device__ __forceinline__ f32x2 both(float v) { return pack2(v, v); }
 __device__ __forceinline__ f32x2 gelu2(f32x2 x) {
-    const f32x2 z = mul2(x, both(0.70710678118654752f)), az = z & 0x7fffffff7fffffffull;
-    float d0, d1, a0, a1, t0, t1, e0, e1;
+    float x0, x1, d0, d1, a0, a1, t0, t1, e0, e1;
+    unpack2(x, x0, x1);
+    const f32x2 az = pack2(__fmul_rn(fabsf(x0), 0.70710678118654752f), __fmul_rn(fabsf(x1), 0.70710678118654752f));     // |z|
     unpack2(fma2(az, both(0.3275911f), both(1.0f)), d0, d1);
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(d0));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(d1));
