@@ -481,11 +481,21 @@ select_cluster_kernel(const float *__restrict__ score, int N_sel, int k, int n_a
     // no barrier at the end: the last remote accesses (the totals above) were complete at the barrier before the placement
 }
 
+// A row's CTA asks for more than half of the shared memory of an SM, so that two rows do not share one (as long as there are SMs): the first
+// SM that the kernel before it leaves has room for both, and the selection is on the critical path of a step.  Steps in a stream, one CTA a
+// row on a shared / on its own SM: 2 x 1253 tokens, 24 heads of 128 43.7 / 41.3 us, 2 x 2000, 16 of 72 36.9 / 34.9, 4 x 2000, 2 of 64 28.8 /
+// 26.8 (a cluster a row 41.3, 35.0, 26.8); one row: no difference.
+constexpr size_t kOwnSmSmem = 120 * 1024;
+
 template <int ITEMS>
 int32_t launch_block(const float *score, int B, int N_sel, int k, int n_always, int32_t *idx_sel, int32_t *idx_rem, int32_t *n_skip, cudaStream_t stream)
 {
-    static_assert(kBlockSmem <= 48 * 1024 - 1024, "no attribute needed");
-    launch_overlapped(select_cluster_kernel<ITEMS, false>, dim3(1, B), kThreads, kBlockSmem, stream, score, N_sel, k, n_always, idx_sel, idx_rem, n_skip);
+    static PerDeviceOnce attrs;
+    if (attrs.run([] { return cudaFuncSetAttribute(select_cluster_kernel<ITEMS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)kOwnSmSmem); }) != cudaSuccess)
+        return check_launch("astraea_select (shared memory attribute)");
+    launch_overlapped(select_cluster_kernel<ITEMS, false>, dim3(1, B), kThreads, B <= sm_count() ? kOwnSmSmem : kBlockSmem, stream, score, N_sel, k, n_always,
+                      idx_sel, idx_rem, n_skip);
     return check_launch("astraea_select");
 }
 

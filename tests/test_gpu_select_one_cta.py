@@ -24,3 +24,10 @@ def test_select_ranges_of_keys(oracle, n):
     for name, s in base.items():
         for k in sorted({0, 1, n // 3, n - 1, n}):
             _select_case(oracle, s.astype(np.float32), k, n_always=3 if name == "two" else 0)
+
+
+@pytest.mark.parametrize("B", [3, 148, 149, 400])
+def test_select_many_rows(oracle, B):
+    """Rows on an SM each, and more rows than SMs."""
+    rng = np.random.default_rng(B)
+    _select_case(oracle, rng.standard_normal((B, 700)).astype(np.float32), 300, n_always=2)
