@@ -1008,8 +1008,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
 }
 
 // Combines the key shares of the split units: row = sum_i w_i row_i with w_i = exp(lse_i - LSE), LSE = log sum_i exp(lse_i)
-// (each share is a complete softmax over its own keys).  One thread per (row, 8 columns); grid (head_dim / 8, units).
-template <int DH, int ROWS>
+// (each share is a complete softmax over its own keys).  One thread per (row, 8 columns); grid (head_dim / 8, units); up to
+// SHARES shares a unit, whose rows a thread holds: two of them leave room for three times as many threads as eight.
+template <int DH, int ROWS, int SHARES>
 __global__ void __launch_bounds__(ROWS) merge_parts_kernel(const Params p)
 {
     constexpr int kChunksRow = DH / 8;
@@ -1025,10 +1026,10 @@ __global__ void __launch_bounds__(ROWS) merge_parts_kernel(const Params p)
     // (attention and merge of 1846 x 4276 x 24 heads of 64 65.0 -> 62.6 us, 2000 x 4000 x 4 28.5 -> 26.3, of 72 30.4 -> 27.8)
     const int tok = p.q_idx ? __ldcg(p.q_idx + (size_t)b * p.M + m) : m, before = (p.q_idx && m > 0) ? __ldcg(p.q_idx + (size_t)b * p.M + m - 1) : -1;
     const size_t part0 = (size_t)blockIdx.y * p.split;
-    float lse[8], mx = -INFINITY;
-    float4 x[8], y[8];
+    float lse[SHARES], mx = -INFINITY;
+    float4 x[SHARES], y[SHARES];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < SHARES; ++i) {
         lse[i] = -INFINITY;
         if (i < p.split) {
             lse[i] = __ldcg(p.part_lse + (part0 + i) * ROWS + r);
@@ -1039,14 +1040,14 @@ __global__ void __launch_bounds__(ROWS) merge_parts_kernel(const Params p)
     if ((unsigned)tok >= (unsigned)p.N_tok || before >= tok) return;   // reported by the attention kernel
     bool gave_up = false;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < SHARES; ++i) {
         gave_up |= __float_as_uint(lse[i]) == kGaveUpLse;
         mx = fmaxf(mx, lse[i]);
     }
     if (gave_up) return;                                            // a share was not finished (a wait ran out): the row stays as it is
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, wsum = 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < SHARES; ++i) {
         if (i < p.split) {
             const float w = __expf(lse[i] - mx);
             wsum += w;
@@ -1181,7 +1182,15 @@ int32_t launch_dh(const AttnArgs &a, cudaStream_t stream, SplitPlan plan = Split
     launch_overlapped(sparse_attn_kernel<C>, grid + (unsigned)p.copy_ctas, C::kThreads, C::kSmemBytes, stream, mk, mv, mkt, mvt, p);
     if (split) {
         static_assert((TM * kBlockM * (DH / 8)) % (TM * kBlockM) == 0, "whole blocks per unit");
-        launch_overlapped(merge_parts_kernel<DH, TM * kBlockM>, dim3(DH / 8, plan.units), TM * kBlockM, 0, stream, p);
+        static_assert(kMaxSplit == 8, "instantiations of the merge");
+        // Two shares always have the form that holds two; three or four theirs only in launches of more than 1.3 rounds of the form that
+        // holds eight (2 CTAs an SM), below which that one is the faster.  Attention and merge with the form for eight / four (head_dim, CTAs
+        // of the merge): 64, 352 61.6 / 62.1 us; 64, 768 44.1 / 43.1; 128, 704 91.7 / 90.9; 128, 1536 68.2 / 65.4; for eight / two: 128, 960
+        // 49.1 / 46.4; 128, 1152 78.1 / 76.0; 64, 64 18.6 / 18.4.
+        const bool few = (DH / 8) * plan.units * 10 <= 27 * sm_count();
+        launch_overlapped(plan.split <= 2 ? merge_parts_kernel<DH, TM * kBlockM, 2> : plan.split <= 4 && !few ? merge_parts_kernel<DH, TM * kBlockM, 4>
+                                                                                                            : merge_parts_kernel<DH, TM * kBlockM, 8>,
+                          dim3(DH / 8, plan.units), TM * kBlockM, 0, stream, p);
     }
     rc = check_launch("astraea_sparse_attn");
     if (rc == ASTRAEA_OK && a.copy_dst && !copy_here)

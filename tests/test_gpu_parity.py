@@ -308,6 +308,7 @@ def test_attn_last_round_split_by_keys(oracle, d):
     _attn_case(oracle, 1, 3, 2100, d, 700, seed=300 + d, expect_split=2)
     _attn_case(oracle, 2, 2, 64 * 53 + 7, d, 300, seed=301 + d, expect_split=3)
     _attn_case(oracle, 1, 2, 64 * 130 + 33, d, 129, seed=302 + d, expect_split=8)
+    _attn_case(oracle, 1, 96, 64 * 49 + 5, d, 130, seed=307 + d, expect_split=3)      # more CTAs of the merge than 1.3 of its rounds
     _attn_case(oracle, 1, 2, 4200, d, 520, seed=303 + d, compact=True, expect_split=4)
     _attn_case(oracle, 1, 2, 2100, d, 260, seed=304 + d, layout="bhnd", expect_split=2)
     _attn_case(oracle, 1, 2, 2100, d, 600, seed=305 + d, amp=12.0, expect_split=2)
