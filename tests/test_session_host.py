@@ -1,4 +1,4 @@
-"""Host-buffer sessions on a model of the CUDA runtime (tests/session_host.cpp): results under every order that streams and events
+"""Host-buffer sessions on a model of the CUDA runtime (tests/session_host.cpp): results under orders that streams and events
 allow, steps that fail half way, arguments, and how much is sent for at a time."""
 import os
 import subprocess
